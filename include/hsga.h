@@ -93,8 +93,8 @@ typedef enum hsga_policy {
 typedef enum hsga_kernel {
   HSGA_KERNEL_AUTO = 0,      /* resident when the grid fits on chip, else streamed */
   HSGA_KERNEL_STREAMED = 1,  /* one launch per generation, population in HBM */
-  HSGA_KERNEL_RESIDENT = 2,  /* persistent launch, genomes in registers; grids of at
-                                most 32 warps run in one block (block barriers), larger
+  HSGA_KERNEL_RESIDENT = 2,  /* persistent launch, genomes in shared memory; grids of a
+                                few islands run in one block (block barriers), larger
                                 ones as a cooperative grid (stamped neighbour records) */
   HSGA_KERNEL_RESIDENT_GRID = 3  /* resident, always the cooperative multi-block form */
 } hsga_kernel;
@@ -186,7 +186,7 @@ typedef struct hsga_stats {
   uint64_t replications;        /* agents x generations advanced by this grid */
   uint64_t kernel_launches;     /* kernels this grid launched */
   uint32_t kernel;              /* hsga_kernel that advances generations */
-  uint32_t islands_per_warp;    /* resident kernel tile shape (0 if streamed) */
+  uint32_t islands_per_warp;    /* resident kernel: a tile's islands over its warps (0 if streamed) */
   uint32_t warps_per_block;
   uint32_t blocks;
   uint32_t fossils;             /* fossil records held */
@@ -348,13 +348,12 @@ int hsga_lookup(uint32_t policy, uint32_t S, uint32_t W, uint64_t T,
 int hsga_sites_device(uint32_t policy, uint32_t S, uint32_t W, uint64_t T0,
                       uint64_t count, uint32_t *out_dev, void *cuda_stream);
 
-/* The bounded waits the resident kernel applies to its neighbours' migrant
+/* The bounded wait the resident kernels apply to their neighbours' migrant
  * records, run on a caller's record: waits until all four 64-bit words of
  * record_dev carry seq in their high 32 bits, giving up after limit_ns
- * (<= 1 s) of the GPU's global timer or 2^22 polls -- first in the form one
- * thread runs (islands polling each neighbour), then in the form a whole
- * warp runs (tiles of islands polling their neighbouring tiles; four lanes,
- * one word each).  Returns HSGA_OK when both saw the record arrive,
+ * (<= 1 s) of the GPU's global timer or 2^22 polls -- first with one lane of
+ * a warp watching the whole record, then with four lanes watching one word
+ * each.  Returns HSGA_OK when both saw the record arrive,
  * HSGA_ERR_WAIT_TIMEOUT when either gave up (the context stays usable);
  * *waited_ns (may be NULL) receives the time spent in both.  record_dev: device, 4 uint64, 8-byte aligned.  Synchronous on
  * cuda_stream.  For checking that an unmet wait ends with a status instead of

@@ -776,10 +776,11 @@ int hsga_get_stats(const hsga_grid *g, hsga_stats *out) {
   out->replications = g->replications;
   out->kernel_launches = g->launches;
   out->kernel = !g->resident ? HSGA_KERNEL_STREAMED
-                : (g->plan.mode == kBlockSync ? HSGA_KERNEL_RESIDENT : HSGA_KERNEL_RESIDENT_GRID);
+                : (g->plan.one_block ? HSGA_KERNEL_RESIDENT : HSGA_KERNEL_RESIDENT_GRID);
   if (g->resident) {
-    out->islands_per_warp = (uint32_t)g->plan.ipw;
-    out->warps_per_block = (uint32_t)g->plan.warps_per_block;
+    const uint32_t warps = (uint32_t)g->plan.threads / 32u;
+    out->islands_per_warp = (g->plan.tile.rows * g->plan.tile.cols + warps - 1u) / warps;
+    out->warps_per_block = warps;
     out->blocks = (uint32_t)g->plan.blocks;
   }
   out->fossils = g->fossil_count;

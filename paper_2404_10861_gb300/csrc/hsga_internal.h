@@ -18,24 +18,22 @@ constexpr int kStagedThreads = 256;     // staged streamed kernel (n = 32) block
 // 78.7 us; 3-5 stages: 76.3-81.2 us).
 constexpr int kStagedBlocksPerSM = 2;
 constexpr uint32_t kStagedStages = 2;   // groups in flight per warp
-constexpr int kResidentThreads = 128;   // resident kernel block: 4 warps
+constexpr int kResidentThreads = 128;   // free-running, float and wide kernels: 4 warps
 constexpr uint32_t kSampleSmemMax = 12288;  // largest k sampled by the shared-memory kernel
 constexpr uint64_t kWaitNs = 1000000000ull; // bounded device wait: 1 s
 
-// How the resident kernel exchanges emigrant records: polled stamped records
-// in global memory; the whole grid in one block (shared memory, block
-// barriers); or tiles of islands per block (shared memory inside a tile,
-// polled records across tiles).
-enum ResidentMode { kPolled = 0, kBlockSync = 1, kTiled = 2 };
-constexpr bool kResidentTiles = true;   // multi-block grids use kTiled when a tile shape fits
+// The resident kernel cuts the torus into tiles of rows x cols islands (the
+// last tile of a row or column may be smaller), tiles_c to a row of tiles.
+struct ResidentTile {
+  uint32_t rows, cols, tiles_c;
+};
 
 struct ResidentPlan {
-  int ap = 0;      // agents per lane (1: n <= 32, 2: n <= 64)
-  int ipw = 0;     // islands per warp
-  int blocks = 0;  // cooperative grid
-  int warps_per_block = kResidentThreads / 32;
-  int mode = kPolled;
-  uint32_t tile = 0;  // kTiled: log2(tile rows) | log2(tile columns) << 8
+  ResidentTile tile{0, 0, 1};
+  int blocks = 0;          // one per tile
+  int threads = 0;
+  uint32_t smem = 0;       // dynamic shared memory per block
+  bool one_block = false;  // a plain launch of one block that holds the whole grid
 };
 
 // err: the grid's device error word (bounded waits report timeouts there).
@@ -50,8 +48,8 @@ cudaError_t launch_step_staged(const RunParams &p, uint32_t G, bool do_mig, cons
                                const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
                                cudaStream_t stream);
 
-// Chooses the resident tile (smallest islands-per-warp whose cooperative
-// grid is co-resident).  Returns false when the grid does not fit on chip.
+// Chooses the resident tiles.  Returns false when the grid does not fit in
+// the SMs' shared memory.
 bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only = false);
 
 cudaError_t launch_step_resident(const RunParams &p, const ResidentPlan &plan, uint32_t G0,
