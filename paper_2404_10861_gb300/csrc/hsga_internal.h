@@ -13,11 +13,13 @@ namespace hsga {
 constexpr int kStreamThreads = 256;     // streamed kernel block: 8 warps
 constexpr int kStreamBlocksPerSM = 3;   // 24 resident warps per SM (<= 80 registers)
 constexpr int kStagedThreads = 256;     // staged streamed kernel (n = 32) block: 8 warps
-// 16 resident warps per SM (<= 128 registers) with two groups in flight per
-// warp: measured fastest at 16.8M agents (75.3 us per generation; 24 warps:
-// 78.7 us; 3-5 stages: 76.3-81.2 us).
-constexpr int kStagedBlocksPerSM = 2;
-constexpr uint32_t kStagedStages = 2;   // groups in flight per warp
+// 24 resident warps per SM (<= 80 registers), each with one group staged:
+// us per generation at 16.8M agents / on 256x256 / 128x128 islands of 32, 24
+// warps and 1 stage 72.1 / 11.9 / 4.9, 24 and 2 72.6 / 12.2 / 5.1, 16 and 2
+// 72.4 / 11.9 / 6.3, 16 and 3 74.2 / 12.1 / 6.3, 32 and 1 72.1 / 11.2 / 5.6
+// (but tournament 5 on 500x500 69.7 against 65.1: 64 registers spill).
+constexpr int kStagedBlocksPerSM = 3;
+constexpr uint32_t kStagedStages = 1;   // groups in flight per warp
 constexpr int kResidentThreads = 128;   // free-running, float and wide kernels: 4 warps
 constexpr uint32_t kSampleSmemMax = 12288;  // largest k sampled by the shared-memory kernel
 constexpr uint64_t kWaitNs = 1000000000ull; // bounded device wait: 1 s

@@ -1,6 +1,6 @@
 // hsga_stage.cuh -- staging of island groups in shared memory by bulk
 // asynchronous copies, shared by the single-run staged generation kernel
-// (hsga_staged.cu) and the batch engine's staged kernel (hsga_batch.cu).
+// (hsga_staged.cu).
 //
 // A warp owns a ring of kStagedStages stages; a stage holds one group of six
 // 32-agent islands: 768 bytes of traits, then 1,536 bytes of surfaces, each
@@ -112,44 +112,59 @@ __device__ __forceinline__ void land_staged(const GroupMigration &gm, uint32_t l
   }
 }
 
-// a3-a6 of child `lane` of one staged island (parents tr[0..31], sr[0..31]).
-// RK: the run's round keys are in the parameter block (single-run kernels);
-// otherwise they are derived from the key.
-template <bool TRACKED, bool T2, bool TWO, bool DEL, bool RK = true>
-__device__ __forceinline__ void replicate_staged(const RunParams &p, const Deposit &dep,
-                                                 uint32_t lane, uint32_t isl, uint32_t G,
-                                                 const Words4 &w, const uint32_t *tr,
-                                                 const uint64_t *sr, uint32_t &ct,
-                                                 uint64_t &cs) {
-  uint32_t best = w.x >> 27;
-  uint32_t fbest = tr[best];
+// a3-a6 of child `lane` of every island of a staged group (parents of island
+// i at tr + 32 i, sr + 32 i), stored to to + 32 i, so + 32 i.  All of the
+// group's reads come before its first store: the stores order memory for the
+// compiler, which would otherwise finish one island before it reads the next.
+template <bool TRACKED, bool T2, bool TWO, bool DEL, class More>
+__device__ __forceinline__ void replicate_group(const RunParams &p, const Deposit &dep,
+                                                const Words4 (&w)[kGroup], const uint32_t *tr,
+                                                const uint64_t *sr, uint32_t *to, uint64_t *so,
+                                                const More &more) {
+  uint32_t best[kGroup], fbest[kGroup];
+  uint64_t cs[kGroup];
+#pragma unroll
+  for (uint32_t i = 0; i < kGroup; ++i) {
+    best[i] = w[i].x >> 27;
+    fbest[i] = tr[32u * i + best[i]];
+  }
   if (T2 || p.tournament >= 2) {
-    const uint32_t c = w.y >> 27;
-    const uint32_t fc = tr[c];
-    const bool take = fc > fbest;
-    best = take ? c : best;
-    fbest = take ? fc : fbest;
+    uint32_t fc[kGroup];
+#pragma unroll
+    for (uint32_t i = 0; i < kGroup; ++i) fc[i] = tr[32u * i + (w[i].y >> 27)];
+#pragma unroll
+    for (uint32_t i = 0; i < kGroup; ++i) {
+      best[i] = fc[i] > fbest[i] ? w[i].y >> 27 : best[i];
+      fbest[i] = max(fc[i], fbest[i]);
+    }
   }
   if constexpr (!T2) {
     for (uint32_t c0 = 2; c0 < p.tournament; c0 += 4) {
-      const Words4 e = philox_p<RK>(p, lane, isl, G, kPurposeReplicate + 1 + (c0 - 2) / 4);
-      const uint32_t ew[4] = {e.x, e.y, e.z, e.w};
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        if (c0 + r < p.tournament) {
-          const uint32_t c = ew[r] >> 27;
-          const uint32_t fc = tr[c];
-          if (fc > fbest) {
-            best = c;
-            fbest = fc;
-          }
+      for (uint32_t i = 0; i < kGroup; ++i) {
+        const Words4 e = more(i, (c0 - 2) / 4);
+        const uint32_t ew[4] = {e.x >> 27, e.y >> 27, e.z >> 27, e.w >> 27};
+        uint32_t fc[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) fc[r] = tr[32u * i + ew[r]];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const bool take = c0 + r < p.tournament && fc[r] > fbest[i];
+          best[i] = take ? ew[r] : best[i];
+          fbest[i] = take ? fc[r] : fbest[i];
         }
       }
     }
   }
-  ct = mutate<DEL>(p, fbest, w.z);
-  if constexpr (TRACKED) cs = deposit_into<TWO>(dep, sr[best], w.w);
-  else cs = 0;
+  if constexpr (TRACKED) {
+#pragma unroll
+    for (uint32_t i = 0; i < kGroup; ++i) cs[i] = sr[32u * i + best[i]];
+  }
+#pragma unroll
+  for (uint32_t i = 0; i < kGroup; ++i) {
+    __stcs(to + 32u * i, mutate<DEL>(p, fbest[i], w[i].z));
+    if constexpr (TRACKED) __stcs(so + 32u * i, deposit_into<TWO>(dep, cs[i], w[i].w));
+  }
 }
 
 constexpr uint32_t kStageBytes = kTraitBytes + kSurfBytes;  // 2304 per group

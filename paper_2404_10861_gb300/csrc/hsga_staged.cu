@@ -7,22 +7,26 @@
 // the surface update).  A persistent grid of warps walks the islands in
 // groups of six (the group of the island-group helpers: six islands' five
 // migration blocks fill 30 lanes of one warp-wide Philox evaluation).  Each
-// warp owns a ring of kStagedStages stages in shared memory; one lane copies
-// a whole group's parents into a stage with cp.async.bulk (768 bytes of
-// traits and 1,536 bytes of surfaces, both contiguous in the island-major
-// planes), completing on that stage's mbarrier, up to kStagedStages groups
-// ahead of the one being replicated.  The bytes in flight therefore cost no registers, and the
-// tournament reads the parents from shared memory: two 4-byte loads for the
-// candidates' fitness and one 8-byte load for the winner's surface per
-// child, where a register-resident island needs its own loads plus four
-// shuffles.  Immigrants are gathered from the neighbours' parent planes as
-// in the register kernel and land with one shared-memory store each (the
-// latest of N, E, S, W wins a shared slot).  Children go straight to the
+// warp stages a group's parents in shared memory; one lane copies them in
+// with cp.async.bulk (768 bytes of traits and 1,536 bytes of surfaces, both
+// contiguous in the island-major planes), completing on the stage's mbarrier,
+// while the group's replication draws are evaluated.  The bytes in flight
+// cost no registers, and the tournament reads the parents from shared memory:
+// two 4-byte loads for the candidates' fitness and one 8-byte load for the
+// winner's surface per child.  Immigrants are gathered from the neighbours'
+// parent planes one group ahead and land with one shared-memory store each
+// (the latest of N, E, S, W wins a shared slot).  Children go straight to the
 // child planes with streaming stores.
 //
-// The replication blocks' counter words other than the island (child slot =
-// lane, generation, purpose) are fixed for a launch, so each lane evaluates
-// round 1's island-independent part once per launch (philox_head).
+// Of the replication blocks' first three rounds only two products depend on
+// the island, one of them the same on every lane (lane_head).
+//
+// What bounds it, per generation at 16.8M agents (copies of the kernel that
+// skip work): without loads and stores 69 us, without migration 64-71, both
+// together 47, everything 72.1; 92 warp instructions per island, 21 of them
+// migration, at 0.56 instructions per cycle and scheduler.  Before: 75.2 us
+// (tournament 5 on 500x500 islands 71.8, now 64.5-65.1), each island's reads
+// behind the stores of the one before it and the gather's latency exposed.
 //
 // Consecutive generations overlap at the launch boundary (programmatic
 // dependent launch): a launch lets the next one be scheduled as soon as it
@@ -47,7 +51,7 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
                        uint64_t *__restrict__ sout, int *__restrict__ err) {
   extern __shared__ __align__(128) unsigned char s_ring[];  // the ring (kRingBytes), padded
   __shared__ __align__(8) uint64_t s_bar[kStagedWarps][kStages];
-  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+  const uint32_t lane = threadIdx.x & 31u, wib = __shfl_sync(kFull, threadIdx.x >> 5, 0);
   const uint32_t warp = blockIdx.x * kStagedWarps + wib;
   const uint32_t nwarps = gridDim.x * kStagedWarps;
   const uint32_t nfull = p.islands / kGroup;
@@ -72,7 +76,9 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
     for (uint32_t st = 0; st < kStages; ++st) mbar_init(&bar[st], 1);
     mbar_init_fence();
   }
-  const PhiloxHead head = philox_head(p.k0, p.k1, lane, G, kPurposeReplicate);
+  const LaneHead head = lane_head(p, lane, G, kPurposeReplicate);
+  [[maybe_unused]] LaneHead head2;  // candidates 2-5
+  if constexpr (!T2) head2 = lane_head(p, lane, G, kPurposeReplicate + 1u);
   // the previous launch (which wrote this launch's parents and read the
   // plane this one writes) has completed and its writes are visible
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -83,14 +89,24 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
   }
   __syncwarp();
 
+  // The immigrants of a group are gathered while the group before it is
+  // replicated: the gather's latency, with nothing to hide it, made up a
+  // third of a generation on L2-resident grids.
+  GroupMigration next_gm{};
+  if constexpr (MIG) {
+    if (warp < nfull) group_migration<TRACKED, true, 32>(p, warp * kGroup, G, tin, sin, next_gm);
+  }
   uint32_t st = 0, phase = 0;  // ring position of the k-th group and its phase parity
   for (uint32_t grp = warp; grp < nfull; grp += nwarps) {
     const uint32_t isl0 = grp * kGroup;
-    GroupMigration gm;
-    if constexpr (MIG) group_migration<TRACKED, true, 32>(p, isl0, G, tin, sin, gm);
+    const GroupMigration gm = next_gm;
+    if constexpr (MIG) {
+      if (grp + nwarps < nfull)
+        group_migration<TRACKED, true, 32>(p, isl0 + nwarps * kGroup, G, tin, sin, next_gm);
+    }
     Words4 w[kGroup];
 #pragma unroll
-    for (uint32_t i = 0; i < kGroup; ++i) w[i] = philox_tail<true>(p, head, isl0 + i);
+    for (uint32_t i = 0; i < kGroup; ++i) w[i] = lane_tail(p, head, isl0 + i);
     if (!__all_sync(kFull, mbar_wait(&bar[st], phase))) {
       // give up: record the timeout, wait (bounded) for this warp's copies
       // still in flight (the groups issued into the ring from this one on),
@@ -117,15 +133,11 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
     }
     uint32_t *to = tout + (size_t)isl0 * 32u + lane;
     uint64_t *so = TRACKED ? sout + (size_t)isl0 * 32u + lane : sout;
-#pragma unroll
-    for (uint32_t i = 0; i < kGroup; ++i) {
-      uint32_t ct;
-      uint64_t cs;
-      replicate_staged<TRACKED, T2, TWO, DEL>(p, dep, lane, isl0 + i, G, w[i], tr + 32u * i,
-                                              sr + (TRACKED ? 32u * i : 0u), ct, cs);
-      __stcs(to + 32u * i, ct);
-      if constexpr (TRACKED) __stcs(so + 32u * i, cs);
-    }
+    replicate_group<TRACKED, T2, TWO, DEL>(
+        p, dep, w, tr, sr, to, so, [&](uint32_t i, uint32_t q) {
+          return q == 0 ? lane_tail(p, head2, isl0 + i)
+                        : philox_rk(p, lane, isl0 + i, G, kPurposeReplicate + 1 + q);
+        });
     __syncwarp();  // every lane is done with this stage before it is refilled
     if (lane == 0 && grp + kStages * nwarps < nfull) issue(grp + kStages * nwarps, st);
     if (++st == kStages) {
