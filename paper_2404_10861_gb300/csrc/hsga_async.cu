@@ -680,47 +680,6 @@ BufferedFn pick_buffered(bool tracked, bool t2, bool two, bool flt, bool n32, bo
                 : pick_buffered_t<false>(tracked, t2, two, flt, n32);
 }
 
-// Synchronous generation with float fitness (after the explicit a1 + a2
-// kernels): one warp per island, IPW islands per warp, every genome's
-// counter equal to G.
-template <bool TRACKED, bool TWO, int IPW>
-__global__ void __launch_bounds__(kResidentThreads)
-    step_float_kernel(RunParams p, uint32_t G, const uint32_t *__restrict__ tin,
-                      const uint64_t *__restrict__ sin, uint32_t *__restrict__ tout,
-                      uint64_t *__restrict__ sout) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const uint32_t first = warp * IPW;
-  if (first >= p.islands) return;
-  const uint32_t n = p.n;
-  uint32_t t[IPW], T[IPW];
-  uint64_t s[IPW];
-#pragma unroll
-  for (int k = 0; k < IPW; ++k) {
-    const uint32_t isl = first + k;
-    t[k] = 0;
-    s[k] = 0;
-    T[k] = G;
-    if (isl < p.islands && lane < n) {
-      t[k] = tin[isl * n + lane];
-      if constexpr (TRACKED) s[k] = sin[isl * n + lane];
-    }
-  }
-  const PhiloxHead h = philox_head(p.k0, p.k1, lane, G, kPurposeReplicate);
-#pragma unroll
-  for (int k = 0; k < IPW; ++k) {
-    const uint32_t isl = first + k;
-    if (isl >= p.islands) break;
-    counter_step<TRACKED, false, TWO, true>(p, h, lane, isl, G, t[k], s[k], T[k]);
-    if (lane < n) {
-      tout[isl * n + lane] = t[k];
-      if constexpr (TRACKED) sout[isl * n + lane] = s[k];
-    }
-  }
-}
-
-constexpr int kFloatIslandsPerWarp = 4;
-
 // Blocks for a free-running launch: one warp per octet, but never more
 // blocks than the device keeps resident at once, so that every island
 // advances in the same pass over the grid (warps then own several octets).
@@ -738,26 +697,6 @@ uint32_t resident_blocks(const void *fn, uint32_t islands, uint32_t ipw, int max
 }
 
 }  // namespace
-
-cudaError_t launch_step_float(const RunParams &p, uint32_t G, const uint32_t *tin,
-                              const uint64_t *sin, uint32_t *tout, uint64_t *sout,
-                              cudaStream_t stream) {
-  constexpr int I = kFloatIslandsPerWarp;
-  const bool tracked = p.policy != HSGA_NONE, two = p.policy == HSGA_HYBRID;
-  const uint32_t wpb = kResidentThreads / 32;
-  const uint32_t warps = (p.islands + I - 1) / I;
-  const uint32_t blocks = (warps + wpb - 1) / wpb;
-  if (!tracked)
-    step_float_kernel<false, false, I><<<blocks, kResidentThreads, 0, stream>>>(p, G, tin, sin,
-                                                                                tout, sout);
-  else if (two)
-    step_float_kernel<true, true, I><<<blocks, kResidentThreads, 0, stream>>>(p, G, tin, sin,
-                                                                              tout, sout);
-  else
-    step_float_kernel<true, false, I><<<blocks, kResidentThreads, 0, stream>>>(p, G, tin, sin,
-                                                                               tout, sout);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_step_buffered(const RunParams &p, uint32_t G0, uint32_t ngen, uint32_t slice,
                                  uint32_t *t, uint64_t *s, uint32_t *T, uint64_t *mail,

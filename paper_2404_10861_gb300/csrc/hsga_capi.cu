@@ -71,6 +71,7 @@ struct hsga_grid {
   bool premigrated = false;
   bool resident = false;
   ResidentPlan plan;
+  StreamPlan splan;  // streamed generations
   bool broken = false;
   uint64_t replications = 0;
   uint64_t launches = 0;
@@ -188,6 +189,7 @@ RunParams make_params(const hsga_config *c) {
   p.flt = c->fitness == HSGA_FITNESS_FLOAT ? 1u : 0u;
   p.gscale = p.flt ? (float)(c->mutation_sigma / sqrt(24.0 + 1.0 / 12.0) / 16777216.0) : 0.0f;
   p.cols_div = make_fastdiv(p.cols);
+  p.n_div = make_fastdiv(p.n);
   set_round_keys(p);
   return p;
 }
@@ -374,6 +376,10 @@ int hsga_init_grid(const hsga_config *cfg, void *cuda_stream, hsga_grid **out) {
       return HSGA_ERR_UNSUPPORTED;
     }
   }
+  if (!g->resident && !g->async && !stream_plan(g->p, &g->splan)) {
+    free_grid(g);
+    return HSGA_ERR_CUDA;
+  }
   *out = g;
   return HSGA_OK;
 }
@@ -514,41 +520,11 @@ int advance(hsga_grid *g, uint64_t n) {
       g->launches++;
       done += m;
     }
-  } else if (g->wide) {
-    // surfaces of several words: explicit a1 + a2, then one warp per island
-    for (uint64_t k = 0; k < n && e == cudaSuccess; ++k) {
-      const uint64_t G = g->G + k;
-      if (migrates(g->p, G) && !(g->premigrated && k == 0)) {
-        e = launch_migrate_wide(g->p, (uint32_t)G, g->trait[g->cur], g->surf[g->cur], g->wrec,
-                                g->stream);
-        g->launches += 2;
-      }
-      if (e == cudaSuccess)
-        e = launch_step_wide(g->p, (uint32_t)G, g->trait[g->cur], g->surf[g->cur],
-                             g->trait[1 - g->cur], g->surf[1 - g->cur], g->stream);
-      g->cur = 1 - g->cur;
-      g->launches++;
-    }
-  } else if (g->p.flt) {
-    // float fitness, synchronous: explicit a1 + a2, then one warp per island
-    for (uint64_t k = 0; k < n && e == cudaSuccess; ++k) {
-      const uint64_t G = g->G + k;
-      if (migrates(g->p, G) && !(g->premigrated && k == 0)) {
-        e = launch_migrate(g->p, (uint32_t)G, g->trait[g->cur], g->surf[g->cur], g->rec,
-                           g->stream);
-        g->launches += 2;
-      }
-      if (e == cudaSuccess)
-        e = launch_step_float(g->p, (uint32_t)G, g->trait[g->cur], g->surf[g->cur],
-                              g->trait[1 - g->cur], g->surf[1 - g->cur], g->stream);
-      g->cur = 1 - g->cur;
-      g->launches++;
-    }
   } else {
     for (uint64_t k = 0; k < n && e == cudaSuccess; ++k) {
       const uint64_t G = g->G + k;
       const bool do_mig = migrates(g->p, G) && !(g->premigrated && k == 0);
-      e = launch_step_streamed(g->p, (uint32_t)G, do_mig, g->trait[g->cur], g->surf[g->cur],
+      e = launch_step_streamed(g->p, g->splan, (uint32_t)G, do_mig, g->trait[g->cur], g->surf[g->cur],
                                g->trait[1 - g->cur], g->surf[1 - g->cur], g->err, g->stream);
       g->cur = 1 - g->cur;
       g->launches++;

@@ -174,6 +174,7 @@ struct RunParams {
   uint32_t flt;            // binary32 fitness with Gaussian mutation amounts
   float gscale;            // float(sigma / sqrt(24 + 1/12) / 2^24)
   FastDiv cols_div;        // island -> (row, column)
+  FastDiv n_div;           // agent of several islands -> (island, slot)
   uint32_t rk0[10], rk1[10];  // Philox round keys k + r * (W0, W1)
 };
 
@@ -324,7 +325,9 @@ struct LaneHead {
   uint32_t l1, l2, l3;  // round 3: words 0, 2 and 3 before the island's parts
 };
 
-__device__ __forceinline__ LaneHead lane_head(const RunParams &p, uint32_t c0, uint32_t c2,
+// p: round keys (RunParams, or a copy of its rk0 and rk1).
+template <class Keys>
+__device__ __forceinline__ LaneHead lane_head(const Keys &p, uint32_t c0, uint32_t c2,
                                               uint32_t c3) {
   const uint64_t p0 = (uint64_t)c0 * kPhiloxM0, p1 = (uint64_t)c2 * kPhiloxM1;
   const uint32_t a2 = (uint32_t)(p0 >> 32) ^ c3 ^ p.rk1[0];
@@ -463,18 +466,30 @@ __device__ __forceinline__ bool fitter(uint32_t a, uint32_t b) {
 // G, kPurposeGauss): the de Moivre-Laplace approximation to a normal of
 // variance 24 + 1/12, smoothed by a 24-bit uniform.  The round-to-nearest
 // intrinsics keep every float step a single correctly rounded operation.
+__device__ __forceinline__ bool mutates_float(const RunParams &p, uint32_t w2) {
+  return (w2 < p.bd32) || p.bd_all;  // thr_ben <= thr_ben + thr_del
+}
+
+__device__ __forceinline__ float gauss_amount(const RunParams &p, const Words4 &q) {
+  const int B = __popc(q.x) + __popc(q.y) + __popc(q.z);
+  const int g = (B - 48) * (1 << 24) + (int)(q.w >> 8) - (1 << 23);
+  return fabsf(__fmul_rn(__int2float_rn(g), p.gscale));
+}
+
+// The mutated fitness, given its amount (not read unless w2 mutates).
+__device__ __forceinline__ uint32_t apply_float(const RunParams &p, uint32_t trait, uint32_t w2,
+                                                float amount) {
+  if (!mutates_float(p, w2)) return trait;
+  const bool ben = (w2 < p.ben32) || p.ben_all;
+  const float f = __uint_as_float(trait);
+  return __float_as_uint(ben ? __fadd_rn(f, amount) : __fsub_rn(f, amount));
+}
+
 __device__ __forceinline__ uint32_t mutate_float(const RunParams &p, uint32_t trait,
                                                  uint32_t w2, uint32_t j, uint32_t isl,
                                                  uint32_t G) {
-  const bool ben = (w2 < p.ben32) || p.ben_all;
-  const bool del = !ben && ((w2 < p.bd32) || p.bd_all);
-  if (!ben && !del) return trait;
-  const Words4 q = philox_rk(p, j, isl, G, kPurposeGauss);
-  const int B = __popc(q.x) + __popc(q.y) + __popc(q.z);
-  const int g = (B - 48) * (1 << 24) + (int)(q.w >> 8) - (1 << 23);
-  const float amount = fabsf(__fmul_rn(__int2float_rn(g), p.gscale));
-  const float f = __uint_as_float(trait);
-  return __float_as_uint(ben ? __fadd_rn(f, amount) : __fsub_rn(f, amount));
+  if (!mutates_float(p, w2)) return trait;
+  return apply_float(p, trait, w2, gauss_amount(p, philox_rk(p, j, isl, G, kPurposeGauss)));
 }
 
 // Device error word values (first error wins).

@@ -1,0 +1,171 @@
+// hsga_flat.cu -- streamed generation kernel for every island size, fitness
+// model and surface width that the staged kernel (32-agent integer islands
+// with one surface word) does not serve: one launch advances one synchronous
+// generation of the whole grid, steps a1-a6, a warp taking groups of eight
+// islands (hsga_flat.cuh).  Consecutive launches overlap by programmatic
+// dependent launch, as in the staged kernel.
+#include <cuda_runtime.h>
+
+#include "hsga_flat.cuh"
+
+namespace hsga {
+namespace {
+
+constexpr int kFlatBlocksPerSM = 5;         // 20 warps
+constexpr int kFlatMaxSmem = 160 * 1024;  // limit set on the kernels; one block uses far less
+
+template <int K, bool T2, int NN, bool FLT>
+__global__ void __launch_bounds__(kFlatThreads, kFlatBlocksPerSM)
+    step_flat_kernel(RunParams p, FlatDeposit<K> dep, uint32_t G, uint32_t group, int migrate,
+                     int bulk,
+                     const uint32_t *__restrict__ tin, const uint64_t *__restrict__ sin,
+                     uint32_t *__restrict__ tout, uint64_t *__restrict__ sout,
+                     int *__restrict__ err) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) uint64_t s_bar[kFlatWarps];
+  const uint32_t lane = threadIdx.x & 31u, wib = __shfl_sync(kFull, threadIdx.x >> 5, 0);
+  // the next launch may be scheduled now; it waits below for this one
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (lane == 0) {
+    mbar_init(&s_bar[wib], 1);
+    mbar_init_fence();
+  }
+  __syncwarp();
+  const uint32_t n = NN ? (uint32_t)NN : p.n;
+  FlatStage st = flat_stage(smem + wib * flat_stage_bytes(n, K), &s_bar[wib], n, K);
+  flat_heads(p, n, G, st);
+  __syncwarp();
+  const uint32_t groups = (p.islands + group - 1) / group;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (uint32_t grp = blockIdx.x * kFlatWarps + wib; grp < groups; grp += gridDim.x * kFlatWarps) {
+    if (!flat_group<K, T2, NN, FLT>(p, p, dep, migrate != 0, bulk != 0, grp * group, group, G, tin,
+                                    sin, tout, sout, st)) {
+      // give up: record the timeout, wait (bounded) for the copy, leave
+      if (lane == 0) {
+        atomicCAS(err, 0, kDevErrWaitTimeout);
+        mbar_wait(st.bar, st.phase);
+      }
+      __syncwarp();
+      return;
+    }
+  }
+}
+
+// Resident blocks and the shared memory to ask for per block: padded so that
+// no further block fits on an SM, since the next launch, scheduled early,
+// would park one there beside the running ones.
+template <int K, bool T2, int NN, bool FLT>
+bool flat_plan(const RunParams &p, StreamPlan *out) {
+  const auto fn = step_flat_kernel<K, T2, NN, FLT>;
+  const size_t need = kFlatWarps * flat_stage_bytes(p.n, K);
+  int dev = 0, sms = 0, per_sm = 0, sm_smem = 0, reserved = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlatMaxSmem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kFlatThreads, need) !=
+          cudaSuccess ||
+      per_sm < 1)
+    return false;
+  const size_t pad = ((size_t)sm_smem / (per_sm + 1) + 255u) & ~(size_t)127;
+  const size_t used = need + (size_t)reserved;  // as the SM counts it
+  // Islands per group: the size (whose groups all start on a 16-byte boundary)
+  // that takes the warps the least work, ceil(groups / warps) rounds of a
+  // group each, counting 1.2 islands' worth for a group's migration draws and
+  // staging.  4,096 groups of 8 on 3,040 warps take two rounds of 8; groups of
+  // 6 two rounds of 6.
+  const uint32_t warps = (uint32_t)(sms * per_sm) * kFlatWarps;
+  const uint32_t step = (p.n & 3u) == 0u ? 1u : (p.n & 1u) == 0u ? 2u : 4u;
+  double best = 1e30;
+  for (uint32_t g = 4; g <= kFlatGroup; g += step) {
+    const uint32_t groups = (p.islands + g - 1) / g;
+    const double cost = (double)((groups + warps - 1) / warps) * (g + 1.2);
+    if (cost <= best) {
+      best = cost;
+      out->group = (int)g;
+    }
+  }
+  out->blocks = sms * per_sm;
+  out->smem = pad > used && pad * per_sm <= (size_t)sm_smem && pad <= kFlatMaxSmem
+                  ? pad - (size_t)reserved
+                  : need;
+  return true;
+}
+
+template <int K, bool T2, int NN, bool FLT>
+cudaError_t launch_flat_t(const RunParams &p, const StreamPlan &plan, const FlatDeposit<K> &dep,
+                          uint32_t G, bool do_mig, const uint32_t *tin, const uint64_t *sin,
+                          uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream) {
+  const uint32_t groups = (p.islands + plan.group - 1) / plan.group;
+  const uint32_t need = (groups + kFlatWarps - 1) / kFlatWarps;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(need < (uint32_t)plan.blocks ? need : (uint32_t)plan.blocks);
+  cfg.blockDim = dim3(kFlatThreads);
+  cfg.dynamicSmemBytes = plan.smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const int bulk = (((uintptr_t)tin | (uintptr_t)sin | (uintptr_t)sout) & 15u) == 0 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, step_flat_kernel<K, T2, NN, FLT>, p, dep, G,
+                            (uint32_t)plan.group, do_mig ? 1 : 0, bulk, tin, sin, tout, sout, err);
+}
+
+// Calls F::run<K, T2, NN, FLT>(args...) for a configuration.
+template <class F, int K, class... A>
+auto flat_pick(const RunParams &p, A &&...args) {
+  const bool t2 = p.tournament == 2, n32 = p.n == 32;
+  if (p.flt)  // general tournament path only
+    return n32 ? F::template run<K, false, 32, true>(p, args...)
+               : F::template run<K, false, 0, true>(p, args...);
+  if constexpr (K > 1) {  // 32-agent islands with at most one word: the staged kernel
+    if (n32)
+      return t2 ? F::template run<K, true, 32, false>(p, args...)
+                : F::template run<K, false, 32, false>(p, args...);
+  }
+  return t2 ? F::template run<K, true, 0, false>(p, args...)
+            : F::template run<K, false, 0, false>(p, args...);
+}
+
+template <class F, class... A>
+auto flat_pick_words(const RunParams &p, A &&...args) {
+  if (p.policy == HSGA_NONE) return flat_pick<F, 0>(p, args...);
+  if (p.words == 4) return flat_pick<F, 4>(p, args...);
+  if (p.words == 2) return flat_pick<F, 2>(p, args...);
+  return flat_pick<F, 1>(p, args...);
+}
+
+struct Plan {
+  template <int K, bool T2, int NN, bool FLT>
+  static bool run(const RunParams &p, StreamPlan *out) {
+    return flat_plan<K, T2, NN, FLT>(p, out);
+  }
+};
+
+struct Launch {
+  template <int K, bool T2, int NN, bool FLT>
+  static cudaError_t run(const RunParams &p, const StreamPlan &plan, uint32_t G, bool do_mig,
+                         const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
+                         int *err, cudaStream_t stream) {
+    return launch_flat_t<K, T2, NN, FLT>(p, plan, flat_deposit<K>(p, G), G, do_mig, tin, sin,
+                                         tout, sout, err, stream);
+  }
+};
+
+}  // namespace
+
+bool flat_stream_plan(const RunParams &p, StreamPlan *out) {
+  return flat_pick_words<Plan>(p, out);
+}
+
+cudaError_t launch_step_flat(const RunParams &p, const StreamPlan &plan, uint32_t G, bool do_mig,
+                             const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
+                             uint64_t *sout, int *err, cudaStream_t stream) {
+  return flat_pick_words<Launch>(p, plan, G, do_mig, tin, sin, tout, sout, err, stream);
+}
+
+}  // namespace hsga

@@ -10,8 +10,6 @@
 
 namespace hsga {
 
-constexpr int kStreamThreads = 256;     // streamed kernel block: 8 warps
-constexpr int kStreamBlocksPerSM = 3;   // 24 resident warps per SM (<= 80 registers)
 constexpr int kStagedThreads = 256;     // staged streamed kernel (n = 32) block: 8 warps
 // 24 resident warps per SM (<= 80 registers), each with one group staged:
 // us per generation at 16.8M agents / on 256x256 / 128x128 islands of 32, 24
@@ -39,9 +37,16 @@ struct ResidentPlan {
 };
 
 // err: the grid's device error word (bounded waits report timeouts there).
-cudaError_t launch_step_streamed(const RunParams &p, uint32_t G, bool do_mig,
-                                 const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
-                                 uint64_t *sout, int *err, cudaStream_t stream);
+// plan: from stream_plan for the same parameters.
+struct StreamPlan {
+  int blocks = 0;   // resident blocks of the whole device
+  size_t smem = 0;  // dynamic shared memory per block
+  int group = 0;    // islands per warp visit
+};
+bool stream_plan(const RunParams &p, StreamPlan *out);
+cudaError_t launch_step_streamed(const RunParams &p, const StreamPlan &plan, uint32_t G,
+                                 bool do_mig, const uint32_t *tin, const uint64_t *sin,
+                                 uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream);
 
 // The same generation for 32-agent islands with the parents staged in shared
 // memory by bulk asynchronous copies (hsga_staged.cu); waits report
@@ -49,6 +54,13 @@ cudaError_t launch_step_streamed(const RunParams &p, uint32_t G, bool do_mig,
 cudaError_t launch_step_staged(const RunParams &p, uint32_t G, bool do_mig, const uint32_t *tin,
                                const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
                                cudaStream_t stream);
+
+// The same generation for any island size, fitness model and surface width
+// (hsga_flat.cu).
+bool flat_stream_plan(const RunParams &p, StreamPlan *out);
+cudaError_t launch_step_flat(const RunParams &p, const StreamPlan &plan, uint32_t G, bool do_mig,
+                             const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
+                             uint64_t *sout, int *err, cudaStream_t stream);
 
 // Chooses the resident tiles.  Returns false when the grid does not fit in
 // the SMs' shared memory.
@@ -80,15 +92,9 @@ struct WideDeposit {
 WideDeposit wide_deposit_for(const RunParams &p, uint64_t G);
 cudaError_t launch_migrate_wide(const RunParams &p, uint32_t G, uint32_t *t, uint64_t *s,
                                 uint64_t *rec, cudaStream_t stream);
-cudaError_t launch_step_wide(const RunParams &p, uint32_t G, const uint32_t *tin,
-                             const uint64_t *sin, uint32_t *tout, uint64_t *sout,
-                             cudaStream_t stream);
 cudaError_t launch_gather_wide(const RunParams &p, uint32_t G, uint32_t k, const uint32_t *t,
                                const uint64_t *s, const uint32_t *where, uint32_t *out,
                                cudaStream_t stream);
-cudaError_t launch_step_float(const RunParams &p, uint32_t G, const uint32_t *tin,
-                              const uint64_t *sin, uint32_t *tout, uint64_t *sout,
-                              cudaStream_t stream);
 // Free-running generations (hsga_async.cu).  slice: generations each warp
 // advances an island octet by per visit (1: the whole grid one generation at
 // a time).

@@ -16,106 +16,20 @@
 namespace hsga {
 
 // ------------------------------------------------------ streamed step ---
-// The group helpers (migration draws, landing plans, island loads/stores)
-// live in hsga_island.cuh.
-// Islands whose Philox chains the streamed kernel interleaves: the whole
-// group (measured at 16.8M agents: 85.9 us per generation against 86.3 with
-// two at a time; 80 registers, 8 bytes spilled).  The batch kernel, which
-// derives the round keys in registers, keeps two.
-constexpr int kStreamInterleave = kGroup;
+// 32-agent integer islands with one surface word (the paper's shape) have a
+// kernel of their own, which plans its launches itself.
+static bool staged_shape(const RunParams &p) { return p.n == 32 && p.words == 1 && !p.flt; }
 
-// MIG: whether this generation migrates (a compile-time flag, so that the
-// full groups carry no run-time branch around the migration draws).
-template <int AP, bool TRACKED, bool T2, int NN, bool MIG>
-__global__ void __launch_bounds__(kStreamThreads, AP == 1 ? kStreamBlocksPerSM : 1)
-    step_streamed_kernel(RunParams p, Deposit dep, uint32_t G,
-                         const uint32_t *__restrict__ tin, const uint64_t *__restrict__ sin,
-                         uint32_t *__restrict__ tout, uint64_t *__restrict__ sout) {
-  constexpr int M = MIG ? 1 : 0;
-  constexpr int IL = kStreamInterleave;
-  const uint32_t wpb = blockDim.x >> 5;
-  const uint32_t nwarps = gridDim.x * wpb;
-  const uint32_t ngroups = (p.islands + kGroup - 1) / kGroup;
-  PhiloxHead head[AP];
-  replication_heads<AP>(p, G, head);
-  for (uint32_t grp = blockIdx.x * wpb + (threadIdx.x >> 5); grp < ngroups; grp += nwarps) {
-    const uint32_t isl0 = grp * kGroup;
-    if (isl0 + kGroup <= p.islands) {
-      if (dep.two)
-        full_group<AP, TRACKED, T2, NN, IL, true, true, true, M>(
-            p, dep, G, MIG, isl0, tin, sin, tout, sout, head);
-      else if (p.has_del)
-        full_group<AP, TRACKED, T2, NN, IL, true, false, true, M>(
-            p, dep, G, MIG, isl0, tin, sin, tout, sout, head);
-      else
-        full_group<AP, TRACKED, T2, NN, IL, true, false, false, M>(
-            p, dep, G, MIG, isl0, tin, sin, tout, sout, head);
-    }
-    else
-      partial_group<AP, TRACKED, T2>(p, dep, G, MIG, isl0, tin, sin, tout, sout);
-  }
+bool stream_plan(const RunParams &p, StreamPlan *out) {
+  return staged_shape(p) || flat_stream_plan(p, out);
 }
 
-template <int AP, bool TRACKED, bool T2, int NN, bool MIG>
-static int streamed_blocks() {
-  static int blocks = 0;
-  if (blocks == 0) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, step_streamed_kernel<AP, TRACKED, T2, NN, MIG>, kStreamThreads, 0);
-    blocks = sms * (per_sm > 0 ? per_sm : 1);
-  }
-  return blocks;
-}
-
-template <int AP, bool TRACKED, bool T2, int NN>
-static void launch_streamed_t(const RunParams &p, const Deposit &dep, uint32_t G, bool do_mig,
-                              const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
-                              uint64_t *sout, cudaStream_t stream) {
-  const uint32_t groups = (p.islands + kGroup - 1) / kGroup;
-  const uint32_t need = (groups + kStreamThreads / 32 - 1) / (kStreamThreads / 32);
-  int b = do_mig ? streamed_blocks<AP, TRACKED, T2, NN, true>()
-                 : streamed_blocks<AP, TRACKED, T2, NN, false>();
-  if ((uint32_t)b > need) b = (int)need;
-  if (do_mig)
-    step_streamed_kernel<AP, TRACKED, T2, NN, true>
-        <<<b, kStreamThreads, 0, stream>>>(p, dep, G, tin, sin, tout, sout);
-  else
-    step_streamed_kernel<AP, TRACKED, T2, NN, false>
-        <<<b, kStreamThreads, 0, stream>>>(p, dep, G, tin, sin, tout, sout);
-}
-
-cudaError_t launch_step_streamed(const RunParams &p, uint32_t G, bool do_mig,
-                                 const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
-                                 uint64_t *sout, int *err, cudaStream_t stream) {
-  // 32-agent islands (the paper's shape): parents staged in shared memory
-  if (p.n == 32) return launch_step_staged(p, G, do_mig, tin, sin, tout, sout, err, stream);
-  const Deposit dep = deposit_for(p, G);
-  const bool tracked = p.policy != HSGA_NONE;
-  const bool t2 = p.tournament == 2;
-  (void)err;  // the register kernel has no waits
-#define HSGA_LAUNCH(AP_, TR_, T2_, NN_) \
-  launch_streamed_t<AP_, TR_, T2_, NN_>(p, dep, G, do_mig, tin, sin, tout, sout, stream)
-#define HSGA_LAUNCH_T(AP_, NN_)                         \
-  if (tracked) {                                        \
-    if (t2) HSGA_LAUNCH(AP_, true, true, NN_);          \
-    else HSGA_LAUNCH(AP_, true, false, NN_);            \
-  } else {                                              \
-    if (t2) HSGA_LAUNCH(AP_, false, true, NN_);         \
-    else HSGA_LAUNCH(AP_, false, false, NN_);           \
-  }
-  if (p.n == 32) {
-    HSGA_LAUNCH_T(1, 32)
-  } else if (p.n < 32) {
-    HSGA_LAUNCH_T(1, 0)
-  } else {
-    HSGA_LAUNCH_T(2, 0)
-  }
-#undef HSGA_LAUNCH_T
-#undef HSGA_LAUNCH
-  return cudaGetLastError();
+cudaError_t launch_step_streamed(const RunParams &p, const StreamPlan &plan, uint32_t G,
+                                 bool do_mig, const uint32_t *tin, const uint64_t *sin,
+                                 uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream) {
+  if (staged_shape(p))
+    return launch_step_staged(p, G, do_mig, tin, sin, tout, sout, err, stream);
+  return launch_step_flat(p, plan, G, do_mig, tin, sin, tout, sout, err, stream);
 }
 
 // --------------------------------------------------- explicit a1 + a2 ---

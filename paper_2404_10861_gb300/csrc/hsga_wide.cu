@@ -1,13 +1,12 @@
-// hsga_wide.cu -- synchronous generations with surfaces of 2 or 4 64-bit
-// words (128- or 256-bit fields; the paper draws a 256-bit field, section
-// "Surface-based Hereditary Stratigraphy Algorithms", and names more and
-// wider differentiae as the remedy for reconstruction precision, "Results ›
-// Clade Reconstruction Trial").
+// hsga_wide.cu -- explicit migration and sampling with surfaces of 2 or 4
+// 64-bit words (128- or 256-bit fields; the paper draws a 256-bit field,
+// section "Surface-based Hereditary Stratigraphy Algorithms", and names more
+// and wider differentiae as the remedy for reconstruction precision, "Results ›
+// Clade Reconstruction Trial").  Generations run in hsga_flat.cu.
 //
 // Surfaces are agent-major: word w of agent a at surf[a K + w]; site s
-// occupies bits [s b mod 64, s b mod 64 + b) of word floor(s b / 64).  One
-// warp serves one island (lane = agent, n <= 32).  The migration step is the
-// explicit a1 + a2 pair with (K + 1)-word records: trait | direction << 32,
+// occupies bits [s b mod 64, s b mod 64 + b) of word floor(s b / 64).  The
+// explicit a1 + a2 pair uses (K + 1)-word records: trait | direction << 32,
 // then the surface words.
 #include <cuda_runtime.h>
 
@@ -50,81 +49,6 @@ __global__ void immigrate_wide_kernel(RunParams p, uint32_t G, uint32_t *__restr
   }
 }
 
-// Writes the b-bit value into the field at (word, shift) of a K-word
-// surface held in registers (word < 0: nothing to write).
-template <int K>
-__device__ __forceinline__ void put_field(uint64_t (&s)[K], int word, uint32_t shift,
-                                          uint64_t vmask, uint32_t value) {
-#pragma unroll
-  for (int w = 0; w < K; ++w)
-    if (w == word) s[w] = (s[w] & ~(vmask << shift)) | (((uint64_t)value & vmask) << shift);
-}
-
-// a3-a6 of one island per warp; every child of generation G deposits at the
-// same field(s) (T = G, or G / k under temporal coarsening).
-template <int K, bool FLT, bool TWO>
-__global__ void __launch_bounds__(kResidentThreads)
-    step_wide_kernel(RunParams p, WideDeposit dep, uint32_t G, const uint32_t *__restrict__ tin,
-                     const uint64_t *__restrict__ sin, uint32_t *__restrict__ tout,
-                     uint64_t *__restrict__ sout) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t isl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (isl >= p.islands) return;
-  const uint32_t n = p.n;
-  uint32_t t = 0;
-  uint64_t s[K];
-#pragma unroll
-  for (int w = 0; w < K; ++w) s[w] = 0;
-  if (lane < n) {
-    const size_t a = (size_t)isl * n + lane;
-    t = tin[a];
-#pragma unroll
-    for (int w = 0; w < K; ++w) s[w] = sin[a * K + w];
-  }
-  const Words4 w4 = philox_rk(p, lane, isl, G, kPurposeReplicate);
-  uint32_t best = uindex(w4.x, n);
-  uint32_t fbest = __shfl_sync(kFull, t, best);
-  if (p.tournament >= 2) {
-    const uint32_t c = uindex(w4.y, n);
-    const uint32_t fc = __shfl_sync(kFull, t, c);
-    if (fitter<FLT>(fc, fbest)) {
-      best = c;
-      fbest = fc;
-    }
-  }
-  for (uint32_t c0 = 2; c0 < p.tournament; c0 += 4) {
-    const Words4 e = philox_rk(p, lane, isl, G, kPurposeReplicate + 1 + (c0 - 2) / 4);
-    const uint32_t ew[4] = {e.x, e.y, e.z, e.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (c0 + q < p.tournament) {
-        const uint32_t c = uindex(ew[q], n);
-        const uint32_t fc = __shfl_sync(kFull, t, c);
-        if (fitter<FLT>(fc, fbest)) {
-          best = c;
-          fbest = fc;
-        }
-      }
-    }
-  }
-  uint32_t child_t;
-  if constexpr (FLT)
-    child_t = mutate_float(p, fbest, w4.z, lane, isl, G);
-  else
-    child_t = mutate(p, fbest, w4.z);
-  uint64_t cs[K];
-#pragma unroll
-  for (int w = 0; w < K; ++w) cs[w] = shfl64(s[w], best);
-  put_field<K>(cs, dep.word1, dep.shift1, p.vmask, w4.w);
-  if constexpr (TWO) put_field<K>(cs, dep.word2, dep.shift2, p.vmask, w4.w >> 16);
-  if (lane < n) {
-    const size_t a = (size_t)isl * n + lane;
-    tout[a] = child_t;
-#pragma unroll
-    for (int w = 0; w < K; ++w) sout[a * K + w] = cs[w];
-  }
-}
-
 // Sample records of 2 + 2K words (trait, surface words as (low, high)
 // pairs, T = G) from (island, slot) pairs.
 __global__ void gather_wide_kernel(uint32_t k, uint32_t n, uint32_t K, uint32_t G,
@@ -150,20 +74,6 @@ void launch_migrate_wide_t(const RunParams &p, uint32_t G, uint32_t *t, uint64_t
   const uint32_t blocks = (p.islands + 255) / 256;
   emigrate_wide_kernel<K><<<blocks, 256, 0, stream>>>(p, G, t, s, rec);
   immigrate_wide_kernel<K><<<blocks, 256, 0, stream>>>(p, G, t, s, rec);
-}
-
-template <int K, bool FLT>
-void launch_step_wide_t(const RunParams &p, const WideDeposit &dep, uint32_t G,
-                        const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
-                        uint64_t *sout, cudaStream_t stream) {
-  const uint32_t wpb = kResidentThreads / 32;
-  const uint32_t blocks = (p.islands + wpb - 1) / wpb;
-  if (p.policy == HSGA_HYBRID)
-    step_wide_kernel<K, FLT, true>
-        <<<blocks, kResidentThreads, 0, stream>>>(p, dep, G, tin, sin, tout, sout);
-  else
-    step_wide_kernel<K, FLT, false>
-        <<<blocks, kResidentThreads, 0, stream>>>(p, dep, G, tin, sin, tout, sout);
 }
 
 }  // namespace
@@ -195,19 +105,6 @@ cudaError_t launch_migrate_wide(const RunParams &p, uint32_t G, uint32_t *t, uin
     launch_migrate_wide_t<2>(p, G, t, s, rec, stream);
   else
     launch_migrate_wide_t<4>(p, G, t, s, rec, stream);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_step_wide(const RunParams &p, uint32_t G, const uint32_t *tin,
-                             const uint64_t *sin, uint32_t *tout, uint64_t *sout,
-                             cudaStream_t stream) {
-  const WideDeposit dep = wide_deposit_for(p, G);
-  if (p.words == 2)
-    p.flt ? launch_step_wide_t<2, true>(p, dep, G, tin, sin, tout, sout, stream)
-          : launch_step_wide_t<2, false>(p, dep, G, tin, sin, tout, sout, stream);
-  else
-    p.flt ? launch_step_wide_t<4, true>(p, dep, G, tin, sin, tout, sout, stream)
-          : launch_step_wide_t<4, false>(p, dep, G, tin, sin, tout, sout, stream);
   return cudaGetLastError();
 }
 
