@@ -407,9 +407,9 @@ int hsga_reconstruct(const uint64_t *surf, uint32_t k, uint32_t surface_words, u
 /* ------------------------------------------------------------ batches ---
  * Many independent runs (uneven grids, agents per island, policies,
  * mutation rates, seeds and generation budgets) advanced together: each
- * "tick" advances every active run by one generation in one launch per
- * agents-per-lane class (n <= 32, n > 32), ticks are replayed from CUDA
- * graphs, and the launch shape is picked by timing real ticks.  Every run
+ * "tick" advances every active run by one generation in one launch, ticks
+ * are replayed from CUDA graphs, and the launch shape is picked by timing real
+ * ticks.  Every run
  * is bit-identical to the same configuration run alone on a grid.  Runs can
  * be added and removed between calls (continuous batching); a run added at
  * tick t starts from founders at generation 0 and is active for its budget
@@ -470,7 +470,8 @@ int hsga_batch_get_stats(const hsga_batch *b, hsga_batch_stats *out);
  * memory footprint).  Host function. */
 int hsga_run_footprint(const hsga_config *cfg, uint64_t *bytes);
 
-/* Waits for the batch's stream (all ticks issued so far). */
+/* Waits for the batch's stream (all ticks issued so far) and returns the first
+ * error a kernel reported. */
 int hsga_batch_synchronize(hsga_batch *b);
 
 void hsga_batch_destroy(hsga_batch *b);

@@ -3,15 +3,14 @@
 // A batch holds runs of uneven size and configuration (grid shape, agents
 // per island, policy, mutation rates, seed, generation budget).  One "tick"
 // advances every active run by one synchronous generation: a single launch
-// per agents-per-lane class covers all of them, so small runs that could not
-// fill the GPU alone share it.  The work list is a flat array of (run, first
-// island) items of up to kGroup islands each; each run's parameters, planes
-// and start tick live in a device descriptor, and the current tick lives in
-// device memory so that a CUDA graph of many ticks can be captured once per
-// active set and replayed.  Runs are admitted and retired between calls,
-// which is what the serving loop builds on.  The launch shape (threads per
-// block, resident blocks) is chosen by timing real ticks (launch shape never
-// changes results).
+// covers all of them, so small runs that could not fill the GPU alone share
+// it.  The work list is a flat array of (run, first island) items of up to
+// kFlatGroup islands each, which warps advance as hsga_flat.cuh describes;
+// each run's parameters, planes and start tick live in a device descriptor,
+// and the current tick lives in device memory so that a CUDA graph of many
+// ticks can be captured once per active set and replayed.  Runs are admitted
+// and retired between calls, which is what the serving loop builds on.
+// Consecutive ticks overlap by programmatic dependent launch.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -23,7 +22,7 @@
 
 #include "hsga.h"
 #include "hsga_internal.h"
-#include "hsga_island.cuh"
+#include "hsga_flat.cuh"
 
 namespace hsga {
 namespace {
@@ -40,47 +39,78 @@ struct WorkItem {
   uint32_t run, isl0;
 };
 
-template <int AP>
-__global__ void __launch_bounds__(512)
+constexpr int kBatchBlocksPerSM = 5;  // 20 warps (<= 96 registers)
+
+__global__ void __launch_bounds__(kFlatThreads, kBatchBlocksPerSM)
     batch_step_kernel(const BatchRun *__restrict__ runs, const WorkItem *__restrict__ items,
                       uint32_t n_items, const uint32_t *__restrict__ tick_base,
-                      uint32_t tick_off) {
-  const uint32_t tick = *tick_base + tick_off;
-  const uint32_t wpb = blockDim.x >> 5;
-  const uint32_t nwarps = gridDim.x * wpb;
-  for (uint32_t i = blockIdx.x * wpb + (threadIdx.x >> 5); i < n_items; i += nwarps) {
-    const WorkItem w = items[i];
-    const BatchRun &R = runs[w.run];
+                      uint32_t tick_off, uint32_t stage_bytes, int *__restrict__ err) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) uint64_t s_bar[kFlatWarps];
+  const uint32_t lane = threadIdx.x & 31u, wib = __shfl_sync(kFull, threadIdx.x >> 5, 0);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (lane == 0) {
+    mbar_init(&s_bar[wib], 1);
+    mbar_init_fence();
+  }
+  __syncwarp();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const uint32_t tick = *tick_base + tick_off, par = tick & 1u;
+  // Items are strided over the warps, which so sweep the list together and find
+  // migrants in L2 (a contiguous share of the list per warp: 123 against 108 ms
+  // for a 16-run mix); a run's descriptor is read, and its generator heads and
+  // deposit evaluated, only where a warp's next item belongs to another run.
+  const uint32_t nwarps = gridDim.x * kFlatWarps;
+  uint32_t i = blockIdx.x * kFlatWarps + wib;
+  uint32_t phase = 0;
+  WorkItem w = i < n_items ? items[i] : WorkItem{0u, 0u};
+  while (i < n_items) {
+    const uint32_t run = w.run;
+    const BatchRun &R = runs[run];
     const RunParams &p = R.p;  // read in place (a copy would live in local memory)
     const uint32_t G = tick - R.start_tick;
-    const uint32_t par = tick & 1u;
     const uint32_t *tin = R.trait[par];
     const uint64_t *sin = R.surf[par];
     uint32_t *tout = R.trait[par ^ 1u];
     uint64_t *sout = R.surf[par ^ 1u];
-    const Deposit dep = deposit_for(p, G);
-    // 32-bit test, every-generation case first (a 64-bit modulo per work item otherwise)
+    const bool bulk = (((uintptr_t)tin | (uintptr_t)sin) & 15u) == 0u;
+    const FlatDeposit<1> dep = flat_deposit<1>(p, G);
+    // 32-bit test, every-generation case first (a 64-bit modulo otherwise)
     const bool do_mig = p.interval == 1u || (p.interval != 0u && G % p.interval == 0u);
-    if (w.isl0 + kGroup <= p.islands) {
-      PhiloxHead head[AP];
-      replication_heads<AP>(p, G, head);
-      if (dep.two)
-        full_group<AP, true, false, 0, kInterleave, false, true>(p, dep, G, do_mig, w.isl0, tin,
-                                                                 sin, tout, sout, head);
-      else if (p.tournament == 2)
-        full_group<AP, true, true, 0, kInterleave, false>(p, dep, G, do_mig, w.isl0, tin, sin,
-                                                          tout, sout, head);
-      else
-        full_group<AP, true, false, 0, kInterleave, false>(p, dep, G, do_mig, w.isl0, tin, sin,
-                                                           tout, sout, head);
-    } else {
-      partial_group<AP, true, false, false>(p, dep, G, do_mig, w.isl0, tin, sin, tout, sout);
+    const bool t2 = p.tournament == 2u;
+    RoundKeys keys;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+      keys.rk0[r] = p.rk0[r];
+      keys.rk1[r] = p.rk1[r];
     }
+    FlatStage st = flat_stage(smem + wib * stage_bytes, &s_bar[wib], p.n, 1);
+    st.phase = phase;
+    flat_heads(keys, p.n, G, st);
+    __syncwarp();
+    do {
+      const uint32_t isl0 = w.isl0;
+      i += nwarps;
+      if (i < n_items) w = items[i];
+      const bool ok = t2 ? flat_group<1, true, 0, false>(p, keys, dep, do_mig, bulk, isl0,
+                                                         kFlatGroup, G, tin, sin, tout, sout, st)
+                         : flat_group<1, false, 0, false>(p, keys, dep, do_mig, bulk, isl0,
+                                                          kFlatGroup, G, tin, sin, tout, sout, st);
+      if (!ok) {
+        // give up: record the timeout, wait (bounded) for the copy, leave
+        if (lane == 0) {
+          atomicCAS(err, 0, kDevErrWaitTimeout);
+          mbar_wait(st.bar, st.phase);
+        }
+        __syncwarp();
+        return;
+      }
+    } while (i < n_items && w.run == run);
+    phase = st.phase;
   }
 }
 
 __global__ void advance_tick_kernel(uint32_t *tick, uint32_t by) { *tick += by; }
-__global__ void set_tick_kernel(uint32_t *tick, uint32_t v) { *tick = v; }
 
 struct HostRun {
   hsga_config cfg;
@@ -91,11 +121,6 @@ struct HostRun {
   uint64_t *surf[2] = {nullptr, nullptr};
   uint64_t agents = 0;
   bool live = false;
-};
-
-struct LaunchShape {
-  int threads = 256;
-  int blocks[2] = {0, 0};  // per agents-per-lane class
 };
 
 constexpr uint64_t kMaxTick = 0xFFFFFFFFull - 64;
@@ -114,21 +139,23 @@ struct hsga_batch {
   BatchRun *d_runs = nullptr;
   size_t d_runs_cap = 0;
   bool runs_dirty = true;
-  WorkItem *d_items[2] = {nullptr, nullptr};
-  size_t items_cap[2] = {0, 0};
-  uint32_t n_items[2] = {0, 0};
-  std::vector<WorkItem> h_items[2];
+  WorkItem *d_items = nullptr;
+  size_t items_cap = 0;
+  uint32_t n_items = 0;
+  std::vector<WorkItem> h_items;
   bool items_dirty = true;
-  // runs in the work lists are ordered by finishing tick, latest first, so
-  // the runs still active at any later tick are a prefix of each list:
+  // runs in the work list are ordered by finishing tick, latest first, so
+  // the runs still active at any later tick are a prefix of the list:
   // (finishing tick, items up to and including that run)
-  std::vector<std::pair<uint64_t, uint32_t>> prefix[2];
-  uint32_t *d_tick = nullptr;
+  std::vector<std::pair<uint64_t, uint32_t>> prefix;
+  uint32_t stage_bytes = 0;  // shared memory per warp for the largest island in the list
+  int most_per_sm = 1;       // blocks that an SM keeps resident with it
+  int per_sm = 0;            // blocks per SM that ticks are launched with
+  std::map<int, int> tuned;  // per_sm by log4 of the item count
+  uint32_t *d_tick = nullptr;  // the tick, then the kernels' error word
   uint64_t tick = 0;
   cudaGraphExec_t graph = nullptr;
   bool graph_valid = false;
-  LaunchShape shape;
-  std::map<int, LaunchShape> tuned;  // by log4 of the item count
   int sms = 0;
   uint64_t launches = 0, replications = 0, phases = 0;
 };
@@ -178,8 +205,8 @@ cudaError_t upload_runs(hsga_batch *b) {
   return e;
 }
 
-// Work lists of the runs active at the current tick, one per agents-per-lane
-// class (n <= 32, n > 32), each ordered by finishing tick, latest first.
+// Work list of the runs active at the current tick, ordered by finishing tick,
+// latest first.
 cudaError_t rebuild_items(hsga_batch *b) {
   std::vector<uint32_t> order;
   for (size_t r = 0; r < b->runs.size(); ++r)
@@ -187,138 +214,133 @@ cudaError_t rebuild_items(hsga_batch *b) {
   std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
     return b->runs[x].start_tick + b->runs[x].budget > b->runs[y].start_tick + b->runs[y].budget;
   });
-  for (int c = 0; c < 2; ++c) {
-    b->h_items[c].clear();
-    b->prefix[c].clear();
-  }
+  b->h_items.clear();
+  b->prefix.clear();
+  uint32_t n_max = 1;
   for (uint32_t r : order) {
     const HostRun &R = b->runs[r];
-    const int c = R.p.n <= 32 ? 0 : 1;
-    for (uint32_t i0 = 0; i0 < R.p.islands; i0 += kGroup)
-      b->h_items[c].push_back(WorkItem{r, i0});
-    b->prefix[c].push_back({R.start_tick + R.budget, (uint32_t)b->h_items[c].size()});
+    n_max = std::max(n_max, R.p.n);
+    for (uint32_t i0 = 0; i0 < R.p.islands; i0 += kFlatGroup)
+      b->h_items.push_back(WorkItem{r, i0});
+    b->prefix.push_back({R.start_tick + R.budget, (uint32_t)b->h_items.size()});
   }
-  cudaError_t e = cudaSuccess;
-  for (int c = 0; c < 2 && e == cudaSuccess; ++c) {
-    const size_t n = b->h_items[c].size();
-    if (n > b->items_cap[c]) {
-      device_free(b->alloc, b->d_items[c], b->stream);
-      const size_t cap = std::max(n, 2 * b->items_cap[c]);
-      b->d_items[c] = (WorkItem *)device_alloc(b->alloc, sizeof(WorkItem) * cap, b->stream);
-      if (!b->d_items[c]) {
-        b->items_cap[c] = 0;
-        return cudaErrorMemoryAllocation;
-      }
-      b->items_cap[c] = cap;
+  b->stage_bytes = flat_stage_bytes(n_max, 1);
+  int per_sm = 0;
+  cudaError_t e = cudaFuncSetAttribute(batch_step_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_step_kernel, kFlatThreads,
+                                                      kFlatWarps * b->stage_bytes);
+  if (e != cudaSuccess) return e;
+  b->most_per_sm = std::max(per_sm, 1);
+  const size_t n = b->h_items.size();
+  if (n > b->items_cap) {
+    device_free(b->alloc, b->d_items, b->stream);
+    const size_t cap = std::max(n, 2 * b->items_cap);
+    b->d_items = (WorkItem *)device_alloc(b->alloc, sizeof(WorkItem) * cap, b->stream);
+    if (!b->d_items) {
+      b->items_cap = 0;
+      return cudaErrorMemoryAllocation;
     }
-    if (n)
-      e = cudaMemcpyAsync(b->d_items[c], b->h_items[c].data(), sizeof(WorkItem) * n,
-                          cudaMemcpyHostToDevice, b->stream);
+    b->items_cap = cap;
   }
+  if (n)
+    e = cudaMemcpyAsync(b->d_items, b->h_items.data(), sizeof(WorkItem) * n,
+                        cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   b->items_dirty = false;
-  b->n_items[0] = b->n_items[1] = 0xFFFFFFFFu;  // force a prefix update
+  b->n_items = 0xFFFFFFFFu;  // force a prefix update
   return e;
 }
 
-// Items of the runs still active at the current tick (a prefix of each list).
+// Items of the runs still active at the current tick (a prefix of the list).
 void select_active_prefix(hsga_batch *b) {
-  for (int c = 0; c < 2; ++c) {
-    uint32_t n = 0;
-    for (const auto &pe : b->prefix[c]) {
-      if (pe.first > b->tick) n = pe.second;
-      else break;
-    }
-    if (n != b->n_items[c]) {
-      b->n_items[c] = n;
-      drop_graph(b);
-    }
+  uint32_t n = 0;
+  for (const auto &pe : b->prefix) {
+    if (pe.first > b->tick) n = pe.second;
+    else break;
+  }
+  if (n != b->n_items) {
+    b->n_items = n;
+    drop_graph(b);
   }
 }
 
-void launch_tick(hsga_batch *b, const LaunchShape &s, uint32_t off) {
-  if (b->n_items[0])
-    batch_step_kernel<1><<<s.blocks[0], s.threads, 0, b->stream>>>(b->d_runs, b->d_items[0],
-                                                                   b->n_items[0], b->d_tick, off);
-  if (b->n_items[1])
-    batch_step_kernel<2><<<s.blocks[1], s.threads, 0, b->stream>>>(b->d_runs, b->d_items[1],
-                                                                   b->n_items[1], b->d_tick, off);
+int tick_blocks(const hsga_batch *b) {
+  const uint64_t need = ((uint64_t)b->n_items + kFlatWarps - 1) / kFlatWarps;
+  const uint64_t most = (uint64_t)b->sms * (uint64_t)std::max(b->per_sm, 1);
+  return (int)std::max<uint64_t>(1, std::min<uint64_t>(need, most));
 }
 
-int launches_per_tick(const hsga_batch *b) {
-  return (b->n_items[0] ? 1 : 0) + (b->n_items[1] ? 1 : 0);
+cudaError_t launch_tick(hsga_batch *b, uint32_t off) {
+  if (!b->n_items) return cudaSuccess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)tick_blocks(b));
+  cfg.blockDim = dim3(kFlatThreads);
+  cfg.dynamicSmemBytes = kFlatWarps * b->stage_bytes;
+  cfg.stream = b->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, batch_step_kernel, (const BatchRun *)b->d_runs,
+                            (const WorkItem *)b->d_items, b->n_items,
+                            (const uint32_t *)b->d_tick, off, b->stage_bytes,
+                            (int *)(b->d_tick + 1));
 }
 
-LaunchShape shape_for(hsga_batch *b, int threads, bool persistent) {
-  LaunchShape s;
-  s.threads = threads;
-  const int wpb = threads / 32;
-  for (int c = 0; c < 2; ++c) {
-    const uint32_t n = b->n_items[c];
-    const uint64_t need = (n + wpb - 1) / wpb;
-    int per_sm = 1;
-    if (persistent) {
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm, c == 0 ? (const void *)batch_step_kernel<1> : (const void *)batch_step_kernel<2>,
-          threads, 0);
-      per_sm = std::max(per_sm, 1);
-      s.blocks[c] = (int)std::max<uint64_t>(1, std::min<uint64_t>(need, (uint64_t)per_sm * b->sms));
-    } else {
-      s.blocks[c] = (int)std::max<uint64_t>(1, need);
-    }
-  }
-  return s;
-}
-
-// Launch-shape autotuner: each candidate advances the batch by a few real
-// ticks (results do not depend on the shape) and the fastest is kept per
-// work-list size class.
+// Launch-shape autotuner: each candidate number of resident blocks per SM
+// advances the batch by a few real ticks (results do not depend on the shape)
+// and the fastest is kept per work-list size class.
 cudaError_t autotune(hsga_batch *b, uint64_t *ticks_left) {
-  const uint32_t total = b->n_items[0] + b->n_items[1];
   int bucket = 0;
-  for (uint32_t x = total; x > 3; x >>= 2) ++bucket;
-  auto it = b->tuned.find(bucket);
+  for (uint32_t x = b->n_items; x > 3; x >>= 2) ++bucket;
+  const int before = b->per_sm;
+  const auto it = b->tuned.find(bucket);
   if (it != b->tuned.end()) {
-    b->shape = shape_for(b, it->second.threads, true);
+    b->per_sm = std::min(it->second, b->most_per_sm);
+    if (b->per_sm != before) drop_graph(b);
     return cudaSuccess;
   }
-  const int cand_threads[3] = {128, 256, 512};
   const uint32_t per_cand = 4;
+  const int candidates = std::min(3, b->most_per_sm);
   float best = 1e30f;
-  LaunchShape best_shape = shape_for(b, 256, true);
+  int best_per_sm = b->most_per_sm, tried = 0;
   cudaEvent_t e0, e1;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  int tried = 0;
-  for (int t : cand_threads) {
-    if (*ticks_left < per_cand) break;
-    const LaunchShape s = shape_for(b, t, true);
-    cudaEventRecord(e0, b->stream);
-    for (uint32_t k = 0; k < per_cand; ++k) launch_tick(b, s, k);
+  cudaError_t e = cudaEventCreate(&e0);
+  if (e != cudaSuccess) return e;
+  e = cudaEventCreate(&e1);
+  if (e != cudaSuccess) {
+    cudaEventDestroy(e0);
+    return e;
+  }
+  for (int c = 0; c < candidates && *ticks_left >= per_cand && e == cudaSuccess; ++c) {
+    b->per_sm = b->most_per_sm - c;
+    e = cudaEventRecord(e0, b->stream);
+    for (uint32_t k = 0; k < per_cand && e == cudaSuccess; ++k) e = launch_tick(b, k);
+    if (e != cudaSuccess) break;
     advance_tick_kernel<<<1, 1, 0, b->stream>>>(b->d_tick, per_cand);
     cudaEventRecord(e1, b->stream);
-    cudaError_t e = cudaEventSynchronize(e1);
-    if (e != cudaSuccess) {
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
-      return e;
-    }
+    e = cudaEventSynchronize(e1);
+    if (e != cudaSuccess) break;
     float ms = 0;
     cudaEventElapsedTime(&ms, e0, e1);
     b->tick += per_cand;
     *ticks_left -= per_cand;
-    b->launches += per_cand * launches_per_tick(b) + 1;
+    b->launches += per_cand + 1;
     ++tried;
     if (ms < best) {
       best = ms;
-      best_shape = s;
+      best_per_sm = b->per_sm;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  b->shape = best_shape;
-  if (tried == 3) b->tuned[bucket] = best_shape;  // keep only complete comparisons
-  return cudaGetLastError();
+  b->per_sm = best_per_sm;
+  if (b->per_sm != before) drop_graph(b);
+  if (e == cudaSuccess && tried == candidates) b->tuned[bucket] = best_per_sm;
+  return e;
 }
 
 cudaError_t run_ticks(hsga_batch *b, uint64_t L) {
@@ -328,12 +350,12 @@ cudaError_t run_ticks(hsga_batch *b, uint64_t L) {
       cudaGraph_t g = nullptr;
       e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
       if (e != cudaSuccess) return e;
-      for (uint32_t k = 0; k < kGraphTicks; ++k) launch_tick(b, b->shape, k);
+      for (uint32_t k = 0; k < kGraphTicks && e == cudaSuccess; ++k) e = launch_tick(b, k);
       advance_tick_kernel<<<1, 1, 0, b->stream>>>(b->d_tick, kGraphTicks);
-      e = cudaStreamEndCapture(b->stream, &g);
-      if (e != cudaSuccess) return e;
-      e = cudaGraphInstantiate(&b->graph, g, 0);
-      cudaGraphDestroy(g);
+      const cudaError_t end = cudaStreamEndCapture(b->stream, &g);
+      if (e == cudaSuccess) e = end;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
+      if (g) cudaGraphDestroy(g);
       if (e != cudaSuccess) return e;
       b->graph_valid = true;
     }
@@ -341,15 +363,15 @@ cudaError_t run_ticks(hsga_batch *b, uint64_t L) {
       e = cudaGraphLaunch(b->graph, b->stream);
       L -= kGraphTicks;
       b->tick += kGraphTicks;
-      b->launches += (uint64_t)kGraphTicks * launches_per_tick(b) + 1;
+      b->launches += (uint64_t)kGraphTicks + 1;
     }
   }
   if (e == cudaSuccess && L > 0) {
-    for (uint32_t k = 0; k < L; ++k) launch_tick(b, b->shape, k);
+    for (uint32_t k = 0; k < L && e == cudaSuccess; ++k) e = launch_tick(b, k);
     advance_tick_kernel<<<1, 1, 0, b->stream>>>(b->d_tick, (uint32_t)L);
     b->tick += L;
-    b->launches += L * launches_per_tick(b) + 1;
-    e = cudaGetLastError();
+    b->launches += L + 1;
+    if (e == cudaSuccess) e = cudaGetLastError();
   }
   return e;
 }
@@ -394,14 +416,13 @@ int hsga_batch_create(void *cuda_stream, hsga_batch **out) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
-  b->d_tick = (uint32_t *)device_alloc(b->alloc, sizeof(uint32_t), b->stream);
+  b->d_tick = (uint32_t *)device_alloc(b->alloc, 2 * sizeof(uint32_t), b->stream);
   if (!b->d_tick) {
     if (b->own_stream) cudaStreamDestroy(b->stream);
     delete b;
     return HSGA_ERR_OOM;
   }
-  set_tick_kernel<<<1, 1, 0, b->stream>>>(b->d_tick, 0);
-  if (cudaGetLastError() != cudaSuccess) {
+  if (cudaMemsetAsync(b->d_tick, 0, 2 * sizeof(uint32_t), b->stream) != cudaSuccess) {
     device_free(b->alloc, b->d_tick, b->stream);
     delete b;
     return HSGA_ERR_CUDA;
@@ -558,8 +579,10 @@ int hsga_batch_get_stats(const hsga_batch *b, hsga_batch_stats *out) {
   out->replications = b->replications;
   out->kernel_launches = b->launches;
   out->phases = b->phases;
-  out->threads_per_block = (uint32_t)b->shape.threads;
-  out->blocks = (uint32_t)(b->shape.blocks[0] + b->shape.blocks[1]);
+  out->threads_per_block = (uint32_t)kFlatThreads;
+  out->blocks = b->d_items && !b->items_dirty && b->n_items != 0xFFFFFFFFu
+                    ? (uint32_t)tick_blocks(b)
+                    : 0u;
   for (const HostRun &R : b->runs) {
     if (R.live) {
       out->live_runs++;
@@ -575,14 +598,21 @@ int hsga_run_footprint(const hsga_config *cfg, uint64_t *bytes) {
   const int v = validate_config(cfg);
   if (v != HSGA_OK) return v;
   const uint64_t agents = (uint64_t)cfg->rows * cfg->cols * cfg->agents_per_island;
-  *bytes = agents * 24 + sizeof(BatchRun) + sizeof(WorkItem) * ((uint64_t)cfg->rows * cfg->cols / kGroup + 1);
+  *bytes = agents * 24 + sizeof(BatchRun) +
+           sizeof(WorkItem) * ((uint64_t)cfg->rows * cfg->cols / kFlatGroup + 1);
   return HSGA_OK;
 }
 
 int hsga_batch_synchronize(hsga_batch *b) {
   if (!b) return HSGA_ERR_INVALID_ARG;
   if (stream_capturing(b->stream)) return HSGA_ERR_NOT_CAPTURABLE;
-  return cudaStreamSynchronize(b->stream) == cudaSuccess ? HSGA_OK : HSGA_ERR_CUDA;
+  // the ticks' bounded waits report a copy that did not arrive
+  int err = 0;
+  cudaError_t e = cudaMemcpyAsync(&err, b->d_tick + 1, sizeof(int), cudaMemcpyDeviceToHost,
+                                  b->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  if (e != cudaSuccess) return HSGA_ERR_CUDA;
+  return err == 0 ? HSGA_OK : err == kDevErrWaitTimeout ? HSGA_ERR_WAIT_TIMEOUT : HSGA_ERR_DEVICE;
 }
 
 void hsga_batch_destroy(hsga_batch *b) {
@@ -592,7 +622,7 @@ void hsga_batch_destroy(hsga_batch *b) {
   for (HostRun &R : b->runs)
     if (R.live) free_run(b, R);
   device_free(b->alloc, b->d_runs, b->stream);
-  for (int c = 0; c < 2; ++c) device_free(b->alloc, b->d_items[c], b->stream);
+  device_free(b->alloc, b->d_items, b->stream);
   device_free(b->alloc, b->d_tick, b->stream);
   cudaStreamSynchronize(b->stream);
   if (b->own_stream) cudaStreamDestroy(b->stream);

@@ -189,7 +189,7 @@ RunParams make_params(const hsga_config *c) {
   p.flt = c->fitness == HSGA_FITNESS_FLOAT ? 1u : 0u;
   p.gscale = p.flt ? (float)(c->mutation_sigma / sqrt(24.0 + 1.0 / 12.0) / 16777216.0) : 0.0f;
   p.cols_div = make_fastdiv(p.cols);
-  p.n_div = make_fastdiv(p.n);
+  p.n_recip = 65536u / p.n + 1u;
   set_round_keys(p);
   return p;
 }

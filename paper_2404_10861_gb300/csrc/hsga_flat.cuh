@@ -16,12 +16,14 @@
 //
 // us per generation, here and on the kernels before it (a lane per agent in
 // registers; for binary32 fitness and wide surfaces a warp per island after
-// two migration launches): 128x256 islands of 48 9.5 (18.5), of 17 5.9
-// (10.3), of 64 with tournament 5 21.9 (43.0); 500x500 of 32, tournament 5,
-// binary32 95 (110); 256x512 of 32 with four surface words 54.6 (66.2), of
+// two migration launches): 128x256 islands of 48 8.7 (18.5), of 17 5.5
+// (10.3), of 64 with tournament 5 21.3 (43.0); 500x500 of 32, tournament 5,
+// binary32 94 (110); 256x512 of 32 with four surface words 54.6 (66.2), of
 // which 44.5 are its 72 bytes per agent at the measured copy bandwidth; 20x20
 // of 32, binary32 3.5 (14.4).  Three children per lane in flight and 20 warps
-// per SM: 128x256x48 takes 11.7 with four, 10.6 with two (32 warps).
+// per SM: 128x256x48 takes a fifth longer with four, a tenth with two (32
+// warps).  Bound by issue: 113 warp instructions per 32 children at n = 48, 51
+// of them on the ALU pipe (two cycles each).
 #pragma once
 
 #include "hsga_stage.cuh"
@@ -181,7 +183,7 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
   const size_t base = (size_t)isl0 * n;
   const auto island_of = [&](uint32_t c) {  // child number -> island of the group
     if constexpr (NN == 32) return c >> 5;
-    else return fastdiv(p.n_div, c);
+    else return (c * p.n_recip) >> 16;  // exact for c < kFlatGroup n, n <= 64
   };
   // stage the parents (the previous group's reads are behind a warp barrier)
   const bool copy = bulk && ((total | (uint32_t)base) & 3u) == 0u;  // whole 16-byte pieces
@@ -285,6 +287,8 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
     __syncwarp();
   }
   // a3-a6 of children c0 + 32 u + lane, u < U
+  uint32_t *const tlane = tout + base + lane;
+  uint64_t *const slane = K > 0 ? sout + (base + lane) * K : sout;
   const bool del = p.has_del != 0u;
   const auto children = [&](auto count, uint32_t c0, const uint32_t (&isl)[decltype(count)::value],
                             const uint32_t (&slot)[decltype(count)::value],
@@ -365,14 +369,15 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
         ct[u] = del ? mutate(p, fbest[u], w[u].z) : mutate<false>(p, fbest[u], w[u].z);
       if constexpr (K > 0) flat_put<K>(dep, cs[u], w[u].w);
     }
+    uint32_t *const to = tlane + c0;
+    [[maybe_unused]] uint64_t *const so = slane + (size_t)c0 * K;
 #pragma unroll
     for (uint32_t u = 0; u < U; ++u) {
-      const uint32_t c = c0 + 32u * u + lane;
-      if (c < total) {
-        __stcs(tout + base + c, ct[u]);
-        if constexpr (K == 1) __stcs(sout + base + c, cs[u][0]);
+      if (c0 + 32u * u + lane < total) {
+        __stcs(to + 32u * u, ct[u]);
+        if constexpr (K == 1) __stcs(so + 32u * u, cs[u][0]);
         if constexpr (K == 2 || K == 4) {
-          uint64_t *const o = sout + (base + c) * K;
+          uint64_t *const o = so + 32u * u * K;
           if (bulk) {  // 16-byte aligned planes
 #pragma unroll
             for (int q = 0; q < KS; q += 2)

@@ -38,16 +38,6 @@ __device__ __forceinline__ uint64_t fetch64(const uint64_t (&v)[AP], uint32_t id
   }
 }
 
-// Heads of the replication blocks Philox(seed; j, *, G, 1) of this lane's
-// children j = lane + 32a, for a whole launch at generation G.
-template <int AP>
-__device__ __forceinline__ void replication_heads(const RunParams &p, uint32_t G,
-                                                  PhiloxHead (&h)[AP]) {
-  const uint32_t lane = threadIdx.x & 31u;
-#pragma unroll
-  for (int a = 0; a < AP; ++a) h[a] = philox_head(p.k0, p.k1, lane + 32u * a, G, kPurposeReplicate);
-}
-
 // Replication words of child j (lane-owned): Philox(seed; j, island, G, 1).
 template <int AP, bool RK = true>
 __device__ __forceinline__ void replication_words(const RunParams &p, uint32_t isl, uint32_t G,
@@ -245,56 +235,6 @@ __device__ __forceinline__ void store_island(const RunParams &p, uint32_t isl,
       __stcs(tout + base + j, t[a]);
       if constexpr (TRACKED) __stcs(sout + base + j, s[a]);
     }
-  }
-}
-
-// One full group: all six islands' genomes are requested up front (deep
-// memory-level parallelism), then the islands are processed ILV at a time so
-// that each lane runs ILV independent Philox chains (instruction-level
-// parallelism hides the multiply-xor dependency chain of the rounds).
-constexpr int kInterleave = 2;
-
-// MIG: 1 or 0 when the launch is known to migrate or not (the migration draws
-// then share a basic block with the first islands' replication draws, and the
-// scheduler interleaves the chains); -1 reads do_mig at run time.
-template <int AP, bool TRACKED, bool T2, int NN, int ILV = kInterleave, bool RK = true,
-          bool TWO = false, bool DEL = true, int MIG = -1>
-__device__ __forceinline__ void full_group(const RunParams &p, const Deposit &dep, uint32_t G,
-                                           bool do_mig, uint32_t isl0,
-                                           const uint32_t *__restrict__ tin,
-                                           const uint64_t *__restrict__ sin,
-                                           uint32_t *__restrict__ tout,
-                                           uint64_t *__restrict__ sout,
-                                           const PhiloxHead (&head)[AP]) {
-  static_assert(kGroup % ILV == 0, "interleave width must divide the group");
-  if constexpr (MIG >= 0) do_mig = MIG == 1;
-  uint32_t pt[kGroup][AP];
-  uint64_t ps[kGroup][AP];
-#pragma unroll
-  for (uint32_t k = 0; k < kGroup; ++k)
-    load_island<AP, TRACKED, NN>(p, isl0 + k, tin, sin, pt[k], ps[k]);
-  GroupMigration gm;
-  if (do_mig) group_migration<TRACKED, RK, NN>(p, isl0, G, tin, sin, gm);
-#pragma unroll
-  for (uint32_t k = 0; k < kGroup; k += ILV) {
-    Words4 w[ILV][AP];
-#pragma unroll
-    for (int i = 0; i < ILV; ++i)
-#pragma unroll
-      for (int a = 0; a < AP; ++a) w[i][a] = philox_tail<RK>(p, head[a], isl0 + k + i);
-    if (do_mig) {
-#pragma unroll
-      for (int i = 0; i < ILV; ++i) group_land<AP, TRACKED>(gm, k + i, pt[k + i], ps[k + i]);
-    }
-    uint32_t ct[ILV][AP];
-    uint64_t cs[ILV][AP];
-#pragma unroll
-    for (int i = 0; i < ILV; ++i)
-      replicate<AP, TRACKED, T2, RK, TWO, DEL, NN>(p, dep, isl0 + k + i, G, w[i], pt[k + i],
-                                                   ps[k + i], ct[i], cs[i]);
-#pragma unroll
-    for (int i = 0; i < ILV; ++i)
-      store_island<AP, TRACKED, NN>(p, isl0 + k + i, tout, sout, ct[i], cs[i]);
   }
 }
 
