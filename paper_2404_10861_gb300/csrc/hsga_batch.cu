@@ -542,7 +542,7 @@ int hsga_batch_sample(hsga_batch *b, uint32_t run, uint32_t k, uint32_t *out_wor
   if (stream_capturing(b->stream)) return HSGA_ERR_NOT_CAPTURABLE;
   const uint64_t G = run_generation(b, R);
   const int par = (int)((R.start_tick + G) & 1);
-  const size_t scratch_bytes = sample_scratch_bytes(R.p, k);
+  const size_t scratch_bytes = sample_scratch_bytes(k);
   uint32_t *scratch = scratch_bytes
                           ? (uint32_t *)device_alloc(b->alloc, scratch_bytes, b->stream)
                           : nullptr;

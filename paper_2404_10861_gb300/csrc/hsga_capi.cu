@@ -431,7 +431,7 @@ int hsga_get_population(hsga_grid *g, uint32_t *trait, uint64_t *surf) {
 namespace {
 
 int ensure_sample_scratch(hsga_grid *g, uint32_t k) {
-  const size_t scratch = sample_scratch_bytes(g->p, k);
+  const size_t scratch = sample_scratch_bytes(k);
   if (scratch > g->sample_scratch_bytes) {
     dev_free(g->alloc, g->sample_scratch, g->stream);
     g->sample_scratch = (uint32_t *)dev_alloc(g->alloc, scratch, g->stream);
@@ -554,6 +554,13 @@ int hsga_set_fossil_sampling(hsga_grid *g, uint64_t every, uint32_t k, uint32_t 
   g->fossil_where = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * 2 * (size_t)capacity,
                                           g->stream);
   if (!g->fossil_words || !g->fossil_where) {
+    dev_free(g->alloc, g->fossil_words, g->stream);
+    dev_free(g->alloc, g->fossil_where, g->stream);
+    g->fossil_words = g->fossil_where = nullptr;
+    return HSGA_ERR_OOM;
+  }
+  // held from now on, so that a run under stream capture allocates nothing
+  if (ensure_sample_scratch(g, k) != HSGA_OK) {
     dev_free(g->alloc, g->fossil_words, g->stream);
     dev_free(g->alloc, g->fossil_where, g->stream);
     g->fossil_words = g->fossil_where = nullptr;

@@ -19,7 +19,6 @@ constexpr int kStagedThreads = 256;     // staged streamed kernel (n = 32) block
 constexpr int kStagedBlocksPerSM = 3;
 constexpr uint32_t kStagedStages = 1;   // groups in flight per warp
 constexpr int kResidentThreads = 128;   // free-running, float and wide kernels: 4 warps
-constexpr uint32_t kSampleSmemMax = 12288;  // largest k sampled by the shared-memory kernel
 constexpr uint64_t kWaitNs = 1000000000ull; // bounded device wait: 1 s
 
 // The resident kernel cuts the torus into tiles of rows x cols islands (the
@@ -73,7 +72,8 @@ cudaError_t launch_step_resident(const RunParams &p, const ResidentPlan &plan, u
 cudaError_t launch_migrate(const RunParams &p, uint32_t G, uint32_t *t, uint64_t *s,
                            uint4 *rec, cudaStream_t stream);
 
-size_t sample_scratch_bytes(const RunParams &p, uint32_t k);
+// Scratch that launch_sample needs for k genomes (8-byte aligned; may be 0).
+size_t sample_scratch_bytes(uint32_t k);
 
 // T: per-genome deposition counters (free-running grids) written as word 3,
 // or NULL to write G.
