@@ -16,8 +16,10 @@
 //             the most significant bits (of a key as wide as the surface), so
 //             that numeric order is path order;
 //   2. sort:  least-significant-digit radix sort of (key, sample) over the
-//             key's significant bits (8-bit digits; stable block scatter
-//             ranked with warp match);
+//             key's significant bits (8-bit digits, stable).  Up to
+//             kSmallSort one-word keys are sorted by one block in shared
+//             memory; above, each pass counts digits per tile, scans the
+//             counts of each digit over the tiles, and scatters;
 //   3. lcp:   L[j] = number of leading differentiae shared by sorted keys j
 //             and j + 1;
 //   4. tree:  the collapsed trie's internal nodes are exactly the maximal
@@ -26,10 +28,20 @@
 //             with its lcp array into a suffix tree.  An interval's parent is
 //             the interval holding the larger of the two lcps just outside
 //             it; a leaf hangs from the interval holding the larger of its
-//             two neighbouring lcps; value 0 (or nothing) is the root.  The
-//             nearest smaller values this needs come from a 32-ary tree of
-//             minima, and each interval is named by its leftmost position
-//             (pointer jumping along equal values).
+//             two neighbouring lcps; value 0 (or nothing) is the root.  An
+//             interval is named by its leftmost position, the first lcp at
+//             most l after the nearest smaller one.  The searches this needs
+//             run inside blocks of 1,024 positions, against 32 values at a
+//             time on bit planes; what lies outside a block is known per
+//             value (an lcp is at most 256) from a scan over the blocks.
+//             Nodes are numbered in the order of the naming positions, from
+//             per-warp masks and counts.
+//
+// Latency bounds a sample of 10,000 genomes: 7 launches of 2.5-31 us, one
+// allocation and one wait for the node count (33, 17 and 2 before); from host
+// arrays to host arrays 127 us, 306 before.  1M genomes, all on the device:
+// 202 us (1,662 before), of which the three-pass sort 90, lcps 12, intervals
+// 34, nodes 17; 16.8M genomes 2.05 ms (41 before).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -42,17 +54,14 @@
 namespace hsga {
 namespace {
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;
-
+constexpr unsigned kAll = 0xFFFFFFFFu;
 constexpr int kMaxWords = 4;
+constexpr int kMaxFields = 64 * kMaxWords;
 
 struct KeyPlan {
-  uint32_t fields;     // retained differentiae m
-  uint32_t bits;       // differentia width b
-  uint32_t words;      // surface (and key) width K in 64-bit words
-  uint32_t src[64 * kMaxWords];  // bit offset of field j (time order) in the surface
+  uint32_t fields;           // retained differentiae m
+  uint32_t bits;             // differentia width b
+  uint32_t src[kMaxFields];  // bit offset of field j (time order) in the surface
 };
 
 // A key of K words: field j (time order) at key bits [j b, (j + 1) b)
@@ -61,262 +70,634 @@ struct KeyWords {
   uint64_t *w[kMaxWords];
 };
 
-__global__ void make_keys_kernel(KeyPlan kp, const uint64_t *__restrict__ surf, uint32_t k,
-                                 KeyWords key, uint32_t *__restrict__ val) {
+template <int K>
+__device__ __forceinline__ void make_key(const KeyPlan &kp, const uint64_t *__restrict__ surf,
+                                         uint64_t (&out)[K]) {
+  const uint64_t mask = (1ull << kp.bits) - 1;  // bits <= 16
+  const uint32_t per_word = 64u / kp.bits;
+  uint64_t s0 = K == 1 ? surf[0] : 0ull;
+  uint32_t j = 0;
+#pragma unroll
+  for (int w = 0; w < K; ++w) {
+    const uint32_t end = min(kp.fields, j + per_word);
+    uint64_t acc = 0;
+    const uint32_t first = j;
+    for (; j < end; ++j) {
+      const uint32_t src = kp.src[j];
+      if constexpr (K > 1) s0 = surf[src >> 6];
+      acc = (acc << kp.bits) | ((s0 >> (src & 63u)) & mask);
+    }
+    const uint32_t used = (j - first) * kp.bits;
+    out[w] = used == 0u ? 0ull : acc << (64u - used);
+  }
+}
+
+template <int K>
+__global__ void make_keys_kernel(const __grid_constant__ KeyPlan kp,
+                                 const uint64_t *__restrict__ surf, uint32_t k, KeyWords key,
+                                 uint32_t *__restrict__ val) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= k) return;
-  const uint64_t mask = (kp.bits == 64) ? ~0ull : ((1ull << kp.bits) - 1);
-  uint64_t out[kMaxWords] = {0, 0, 0, 0};
-  for (uint32_t j = 0; j < kp.fields; ++j) {
-    const uint32_t src = kp.src[j];
-    const uint64_t v = (surf[(size_t)i * kp.words + src / 64] >> (src % 64)) & mask;
-    const uint32_t g = j * kp.bits;  // global key bit from the top
-    out[g / 64] |= v << (64u - g % 64 - kp.bits);
-  }
-  for (uint32_t w = 0; w < kp.words; ++w) key.w[w][i] = out[w];
+  uint64_t out[K];
+  make_key<K>(kp, surf + (size_t)i * K, out);
+#pragma unroll
+  for (int w = 0; w < K; ++w) key.w[w][i] = out[w];
   val[i] = i;
 }
 
 // ------------------------------------------------------------ radix sort ---
-__global__ void digit_histogram_kernel(const uint64_t *__restrict__ key, uint32_t k,
-                                       uint32_t shift, uint32_t nblocks,
-                                       uint32_t *__restrict__ hist) {
-  // key: the key word that holds this pass's digit
+// Lanes of the warp with the same digit, from eight votes: a match
+// instruction takes one step per distinct value (47 against 42 us for keys and
+// sort of 10,000 samples by one block).
+__device__ __forceinline__ uint32_t same_digit(uint32_t digit) {
+  uint32_t peers = kAll;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const bool bit = digit >> b & 1u;
+    const uint32_t set = __ballot_sync(kAll, bit);
+    peers &= bit ? set : ~set;
+  }
+  return peers;
+}
+
+// A warp ranks its elements of one digit pass stably: 32 at a time, an
+// element's rank among equal digits is (its warp's count so far) + (earlier
+// lanes with the same digit).  cnt: the warp's 256 counts.
+__device__ __forceinline__ uint32_t warp_rank(uint32_t *cnt, uint32_t digit, bool live,
+                                              uint32_t lane) {
+  const uint32_t peers = same_digit(digit) & __ballot_sync(kAll, live);
+  const uint32_t old = cnt[digit];
+  __syncwarp();
+  const uint32_t before = __popc(peers & ((1u << lane) - 1u));
+  if (live && before == 0u) cnt[digit] = old + __popc(peers);
+  __syncwarp();
+  return old + before;
+}
+
+// Exclusive sum of v over the block's threads in thread order (blockDim.x a
+// multiple of 32, at most 1,024); sums: 32 words of shared memory.
+__device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *sums) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (uint32_t o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kAll, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31u) sums[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t t = lane < warps ? sums[lane] : 0u;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kAll, t, o);
+      if (lane >= o) t += y;
+    }
+    if (lane < warps) sums[lane] = t;
+  }
+  __syncthreads();
+  const uint32_t r = x - v + (warp ? sums[warp - 1u] : 0u);
+  __syncthreads();
+  return r;
+}
+
+constexpr uint32_t kSmallSort = 12288;  // one-word keys that one block sorts
+constexpr uint32_t kSmallItems = kSmallSort / 1024;
+
+constexpr size_t small_sort_smem(uint32_t k) {
+  const size_t n = (k + 1023u) / 1024u * 1024u;
+  return n * 8 + 2 * n * 2 + 32 * 256 * 4 + 32 * 4;
+}
+
+// Keys stay in place in shared memory and their 16-bit positions are sorted;
+// the sorted keys and samples go out at the end.
+__global__ void __launch_bounds__(1024)
+    small_sort_kernel(const uint64_t *__restrict__ key_in, uint32_t k, uint32_t passes,
+                      uint64_t *__restrict__ key_out, uint32_t *__restrict__ val_out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const uint32_t rounds = (k + 1023u) / 1024u, n = rounds * 1024u;
+  uint64_t *const key = (uint64_t *)smem;
+  uint16_t *idx = (uint16_t *)(key + n), *idx2 = idx + n;
+  uint32_t *const cnt = (uint32_t *)(idx2 + n);  // [warp][digit]
+  uint32_t *const sums = cnt + 32 * 256;
+  const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+  for (uint32_t i = t; i < k; i += 1024u) {
+    key[i] = key_in[i];
+    idx[i] = (uint16_t)i;
+  }
+  __syncthreads();
+  const uint32_t first = warp * rounds * 32u + lane;  // this warp's run of positions
+  for (uint32_t ps = 0; ps < passes; ++ps) {
+    const uint32_t byte = 7u - (passes - 1u - ps);  // little endian: byte 7 is the top digit
+    for (uint32_t c = t; c < 32u * 256u; c += 1024u) cnt[c] = 0;
+    __syncthreads();
+    uint32_t held[kSmallItems], rank[kSmallItems];  // position of the key, digit << 16
+#pragma unroll
+    for (uint32_t r = 0; r < kSmallItems; ++r) {
+      if (r < rounds) {
+        const uint32_t e = first + 32u * r;
+        const bool live = e < k;
+        const uint32_t i = live ? idx[e] : 0u;
+        const uint32_t d = live ? ((const unsigned char *)(key + i))[byte] : 0u;
+        held[r] = i | (d << 16);
+        rank[r] = warp_rank(cnt + 256u * warp, d, live, lane);
+      }
+    }
+    __syncthreads();
+    // thread 4d + q: digit d, warps 8q .. 8q + 7 -- thread order is (digit, warp) order
+    const uint32_t d = t >> 2, w0 = 8u * (t & 3u);
+    uint32_t s = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < 8; ++w) s += cnt[256u * (w0 + w) + d];
+    uint32_t run = block_exclusive(s, sums);
+#pragma unroll
+    for (uint32_t w = 0; w < 8; ++w) {
+      const uint32_t c = cnt[256u * (w0 + w) + d];
+      cnt[256u * (w0 + w) + d] = run;
+      run += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t r = 0; r < kSmallItems; ++r)
+      if (r < rounds && first + 32u * r < k)
+        idx2[cnt[256u * warp + (held[r] >> 16)] + rank[r]] = (uint16_t)held[r];
+    __syncthreads();
+    uint16_t *const x = idx;
+    idx = idx2;
+    idx2 = x;
+  }
+  for (uint32_t e = t; e < k; e += 1024u) {
+    key_out[e] = key[idx[e]];
+    val_out[e] = idx[e];
+  }
+}
+
+constexpr int kSortThreads = 256;
+constexpr int kSortItems = 8;
+constexpr int kSortTile = kSortThreads * kSortItems;
+
+// Digit counts of every tile, digit-major; key: the key word that holds this
+// pass's digit.
+__global__ void __launch_bounds__(kSortThreads)
+    digit_histogram_kernel(const uint64_t *__restrict__ key, uint32_t k, uint32_t shift,
+                           uint32_t ntiles, uint32_t *__restrict__ hist) {
   __shared__ uint32_t cnt[256];
   cnt[threadIdx.x] = 0;
   __syncthreads();
-  const uint32_t base = blockIdx.x * kSortTile;
+  // equal digits of a warp (the rule, not the exception, in an evolved
+  // population) are counted by one of its lanes
+  const uint32_t base = blockIdx.x * kSortTile, lane = threadIdx.x & 31u;
+  uint32_t d[kSortItems];
+#pragma unroll
   for (int r = 0; r < kSortItems; ++r) {
     const uint32_t e = base + r * kSortThreads + threadIdx.x;
-    if (e < k) atomicAdd(&cnt[(uint32_t)(key[e] >> shift) & 0xFFu], 1u);
+    d[r] = e < k ? (uint32_t)(key[e] >> shift) & 0xFFu : 0u;
+  }
+#pragma unroll
+  for (int r = 0; r < kSortItems; ++r) {
+    const bool live = base + r * kSortThreads + threadIdx.x < k;
+    const uint32_t peers = same_digit(d[r]) & __ballot_sync(kAll, live);
+    if (live && (peers & ((1u << lane) - 1u)) == 0u)
+      atomicAdd(&cnt[d[r]], (uint32_t)__popc(peers));
   }
   __syncthreads();
-  hist[threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
+  hist[threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// Exclusive prefix sum of n uint32 in place, one block of 1024 threads
-// (each thread scans a contiguous chunk).
-__global__ void exclusive_scan_kernel(uint32_t *__restrict__ a, uint32_t n,
-                                      uint32_t *__restrict__ total) {
-  __shared__ uint32_t part[1024];
-  const uint32_t t = threadIdx.x;
-  const uint32_t chunk = (n + 1023) / 1024;
-  const uint32_t lo = min(n, t * chunk), hi = min(n, lo + chunk);
-  uint32_t s = 0;
-  for (uint32_t i = lo; i < hi; ++i) s += a[i];
-  part[t] = s;
+// Block d: exclusive scan of digit d's counts over the tiles, in place, and
+// their total.
+__global__ void __launch_bounds__(256)
+    digit_scan_kernel(uint32_t *__restrict__ hist, uint32_t ntiles, uint32_t *__restrict__ total) {
+  __shared__ uint32_t sums[32];
+  __shared__ uint32_t carry;
+  uint32_t *const row = hist + (size_t)blockIdx.x * ntiles;
+  if (threadIdx.x == 0) carry = 0;
   __syncthreads();
-  for (uint32_t off = 1; off < 1024; off <<= 1) {
-    const uint32_t v = t >= off ? part[t - off] : 0u;
+  for (uint32_t i0 = 0; i0 < ntiles; i0 += 256u) {
+    const uint32_t i = i0 + threadIdx.x;
+    const uint32_t v = i < ntiles ? row[i] : 0u;
+    const uint32_t x = block_exclusive(v, sums) + carry;
+    if (i < ntiles) row[i] = x;
     __syncthreads();
-    part[t] += v;
+    if (threadIdx.x == 255u) carry = x + v;
     __syncthreads();
   }
-  uint32_t run = part[t] - s;
+  if (threadIdx.x == 0) total[blockIdx.x] = carry;
+}
+
+// Stable scatter of one digit pass.
+template <int K>
+__global__ void __launch_bounds__(kSortThreads)
+    digit_scatter_kernel(KeyWords key_in, const uint32_t *__restrict__ val_in, uint32_t k,
+                         uint32_t dword, uint32_t shift, uint32_t ntiles,
+                         const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ total,
+                         KeyWords key_out, uint32_t *__restrict__ val_out) {
+  constexpr int kWarps = kSortThreads / 32;
+  __shared__ uint32_t cnt[kWarps][256];
+  __shared__ uint32_t sums[32];
+  const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) cnt[w][t] = 0;
+  __syncthreads();
+  const uint64_t *const dkey = key_in.w[dword];
+  const uint32_t first = blockIdx.x * kSortTile + warp * (32u * kSortItems) + lane;
+  uint32_t rank[kSortItems];  // rank in the warp | digit << 16
+#pragma unroll
+  for (int r = 0; r < kSortItems; ++r) {
+    const uint32_t e = first + 32u * r;
+    rank[r] = e < k ? (uint32_t)(dkey[e] >> shift) & 0xFFu : 0u;
+  }
+#pragma unroll
+  for (int r = 0; r < kSortItems; ++r)
+    rank[r] = warp_rank(cnt[warp], rank[r], first + 32u * r < k, lane) | (rank[r] << 16);
+  const uint32_t base = block_exclusive(total[t], sums);  // ends with a block barrier
+  {  // thread t owns digit t: the tile's elements of it, warp by warp
+    uint32_t run = base + offsets[(size_t)t * ntiles + blockIdx.x];
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const uint32_t c = cnt[w][t];
+      cnt[w][t] = run;
+      run += c;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kSortItems; ++r) {
+    const uint32_t e = first + 32u * r;
+    if (e < k) {
+      const uint32_t pos = cnt[warp][rank[r] >> 16] + (rank[r] & 0xFFFFu);
+#pragma unroll
+      for (int w = 0; w < K; ++w) key_out.w[w][pos] = key_in.w[w][e];
+      val_out[pos] = val_in[e];
+    }
+  }
+}
+
+// ----------------------------------------------------------------- lcp ---
+constexpr uint32_t kBlockPos = 1024;  // lcp positions of a block
+constexpr uint32_t kPlanes = 9;       // bits of an lcp (at most kMaxFields)
+constexpr uint32_t kNoLcp = (1u << kPlanes) - 1;  // beyond the last: never smaller
+
+// Lanes whose value, given as bit planes, is below x.
+template <class Planes>
+__device__ __forceinline__ uint32_t below(const Planes &plane, uint32_t x) {
+  uint32_t lt = 0, eq = kAll;
+#pragma unroll
+  for (int b = kPlanes - 1; b >= 0; --b) {
+    const uint32_t bit = plane(b), want = (x >> b & 1u) ? kAll : 0u;
+    lt |= eq & want & ~bit;
+    eq &= ~(want ^ bit);
+  }
+  return lt;
+}
+
+__device__ __forceinline__ uint32_t top_bit(uint32_t m) { return 31u - (uint32_t)__clz((int)m); }
+__device__ __forceinline__ uint32_t low_bit(uint32_t m) { return (uint32_t)__ffs((int)m) - 1u; }
+
+// A block's 1,024 lcps for searches: in shared memory, the bit planes of every
+// warp's 32 values and (row 32) of the 32 warps' minima.  Positions are
+// relative to the block.  (Planes of the own warp and the minima in registers
+// left room for one block per SM instead of two: 38 against 34 us at 1M.)
+using LcpPlanes = uint32_t[33][kPlanes];
+
+struct BlockLcps {
+  const uint32_t (*planes)[kPlanes];
+
+  // planes_, wmin: shared memory; ends with a block barrier.
+  __device__ __forceinline__ BlockLcps(uint32_t v, LcpPlanes &planes_, uint32_t *wmin)
+      : planes(planes_) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    put(v, planes_[warp], lane);
+    const uint32_t m = __reduce_min_sync(kAll, v);
+    if (lane == 0) wmin[warp] = m;
+    __syncthreads();
+    if (warp == 0) put(wmin[lane], planes_[32], lane);
+    __syncthreads();
+  }
+  static __device__ __forceinline__ void put(uint32_t v, uint32_t *row, uint32_t lane) {
+    uint32_t mine = 0;
+#pragma unroll
+    for (uint32_t b = 0; b < kPlanes; ++b) {
+      const uint32_t set = __ballot_sync(kAll, v >> b & 1u);
+      mine = lane == b ? set : mine;
+    }
+    if (lane < kPlanes) row[lane] = mine;
+  }
+  __device__ __forceinline__ uint32_t in_warp(uint32_t w, uint32_t x) const {
+    return below([&](int b) { return planes[w][b]; }, x);
+  }
+  __device__ __forceinline__ uint32_t warps(uint32_t x) const {  // with a value below x
+    return in_warp(32u, x);
+  }
+  // First position >= q (q < 1,024) with a value below x, or -1.
+  __device__ __forceinline__ int32_t first_from(uint32_t q, uint32_t x) const {
+    const uint32_t w = q >> 5, here = in_warp(w, x) & (kAll << (q & 31u));
+    if (here) return (int32_t)(32u * w + low_bit(here));
+    const uint32_t later = warps(x) & ~((2u << w) - 1u);
+    if (!later) return -1;
+    const uint32_t w2 = low_bit(later);
+    return (int32_t)(32u * w2 + low_bit(in_warp(w2, x)));
+  }
+};
+
+// What the blocks around it tell a block about each value v (row v, column
+// block): last / first, the nearest position before / after the block with a
+// smaller lcp (-1: none); open, the position that names the interval of value
+// v that runs into the block (-1: none does, or it has no v yet).
+struct Carries {
+  int32_t *last, *first, *open;
+  uint32_t blocks;
+};
+
+// lcps, and per block and value: last / first position with a smaller lcp (-1:
+// none), and the first with this one after the last smaller one (-1: none).
+template <int K>
+__global__ void __launch_bounds__(kBlockPos, 2)
+    lcp_kernel(KeyWords key, uint32_t n, uint32_t fields, uint32_t bits,
+               uint16_t *__restrict__ L, Carries c) {
+  __shared__ LcpPlanes planes;
+  __shared__ uint32_t wmin[32];
+  const uint32_t base = blockIdx.x * kBlockPos, j = base + threadIdx.x;
+  uint32_t v = kNoLcp;
+  if (j < n) {
+    v = fields;
+    bool differ = false;
+#pragma unroll
+    for (int w = 0; w < K; ++w) {
+      const uint64_t x = key.w[w][j] ^ key.w[w][j + 1];
+      if (!differ && x) {
+        v = min(fields, (w * 64u + (uint32_t)__clzll((long long)x)) / bits);
+        differ = true;
+      }
+    }
+    L[j] = (uint16_t)v;
+  }
+  const BlockLcps bl(v, planes, wmin);
+  if (threadIdx.x <= fields) {
+    const uint32_t x = threadIdx.x;
+    const uint32_t ws = bl.warps(x);
+    int32_t last = -1, first = -1;
+    if (ws) {
+      const uint32_t w1 = top_bit(ws), w0 = low_bit(ws);
+      last = (int32_t)(32u * w1 + top_bit(bl.in_warp(w1, x)));
+      first = (int32_t)(32u * w0 + low_bit(bl.in_warp(w0, x)));
+    }
+    const int32_t open =
+        last + 1 < (int32_t)kBlockPos ? bl.first_from((uint32_t)(last + 1), x + 1u) : -1;
+    const size_t at = (size_t)x * c.blocks + blockIdx.x;
+    c.last[at] = last < 0 ? -1 : (int32_t)base + last;
+    c.first[at] = first < 0 ? -1 : (int32_t)base + first;
+    c.open[at] = open < 0 ? -1 : (int32_t)base + open;
+  }
+}
+
+// Row v: from each block's own answers to what the blocks before it (last,
+// open) and after it (first) tell it, in place.  One warp per row and
+// direction; the loads of kAhead chunks of 32 blocks are in flight together.
+constexpr uint32_t kAhead = 8;
+
+__device__ __forceinline__ void carry_forward(int32_t *last, int32_t *open, uint32_t blocks,
+                                              uint32_t lane) {
+  int32_t run_last = -1, run_open = -1;
+  for (uint32_t c0 = 0; c0 < blocks; c0 += 32u * kAhead) {
+    int32_t ls[kAhead], os[kAhead];
+#pragma unroll
+    for (uint32_t i = 0; i < kAhead; ++i) {
+      const uint32_t b = c0 + 32u * i + lane;
+      ls[i] = b < blocks ? last[b] : -1;
+      os[i] = b < blocks ? open[b] : -1;
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < kAhead; ++i) {
+      const uint32_t b = c0 + 32u * i + lane;
+      const int32_t l = ls[i], o = os[i];
+      // blocks with a smaller lcp start afresh; the others keep what is open
+      const uint32_t resets = __ballot_sync(kAll, l >= 0), opens = __ballot_sync(kAll, o >= 0);
+      const uint32_t lower = (1u << lane) - 1u;
+      const uint32_t r = resets & lower;
+      const uint32_t from = r ? top_bit(r) : 0u;  // the last reset before this block
+      const uint32_t since = opens & lower & (r ? kAll << from : kAll);
+      const int32_t l_from = __shfl_sync(kAll, l, from);
+      const int32_t o_first = __shfl_sync(kAll, o, since ? low_bit(since) : 0u);
+      const int32_t in_last = r ? l_from : run_last;
+      const int32_t in_open = !r && run_open >= 0 ? run_open : since ? o_first : -1;
+      if (b < blocks) {
+        last[b] = in_last;
+        open[b] = in_open;
+      }
+      // the state after this chunk's last block
+      const int32_t out_last = l >= 0 ? l : in_last;
+      const int32_t out_open = l >= 0 ? o : in_open >= 0 ? in_open : o;
+      run_last = __shfl_sync(kAll, out_last, 31);
+      run_open = __shfl_sync(kAll, out_open, 31);
+    }
+  }
+}
+
+__device__ __forceinline__ void carry_backward(int32_t *first, uint32_t blocks, uint32_t lane) {
+  int32_t run = -1;
+  const uint32_t step = 32u * kAhead;
+  for (uint32_t c0 = (blocks - 1u) / step * step;; c0 -= step) {
+    int32_t fs[kAhead];
+#pragma unroll
+    for (uint32_t i = 0; i < kAhead; ++i) {
+      const uint32_t b = c0 + 32u * i + lane;
+      fs[i] = b < blocks ? first[b] : -1;
+    }
+#pragma unroll
+    for (int i = kAhead - 1; i >= 0; --i) {
+      const uint32_t b = c0 + 32u * i + lane;
+      const int32_t f = fs[i];
+      const uint32_t have = __ballot_sync(kAll, f >= 0) & ~((2u << lane) - 1u);
+      const int32_t near = __shfl_sync(kAll, f, have ? low_bit(have) : 0u);
+      if (b < blocks) first[b] = have ? near : run;
+      const int32_t out = f >= 0 ? f : have ? near : run;
+      run = __shfl_sync(kAll, out, 0);
+    }
+    if (c0 == 0u) break;
+  }
+}
+
+__global__ void __launch_bounds__(64) carry_kernel(Carries c) {
+  const size_t row = (size_t)blockIdx.x * c.blocks;
+  const uint32_t lane = threadIdx.x & 31u;
+  if (threadIdx.x < 32u) carry_forward(c.last + row, c.open + row, c.blocks, lane);
+  else carry_backward(c.first + row, c.blocks, lane);
+}
+
+// Node numbering: position q names an interval iff bit q & 31 of mask[q >> 5]
+// is set; its rank is base[q >> 10] + before[q >> 5] + the set bits below it.
+struct NodeRanks {
+  uint32_t *mask, *before, *base;
+};
+
+__device__ __forceinline__ uint32_t node_rank(const NodeRanks &nr, uint32_t q) {
+  return nr.base[q >> 10] + nr.before[q >> 5] + __popc(nr.mask[q >> 5] & ((1u << (q & 31u)) - 1u));
+}
+
+// For each lcp position: rep, the position that names its interval; where
+// that is the position itself and the value at least 1, also PS and NS, the
+// previous and next strictly smaller positions.
+__global__ void __launch_bounds__(kBlockPos, 2)
+    intervals_kernel(const uint16_t *__restrict__ L, uint32_t n, Carries c,
+                     int32_t *__restrict__ ps_out, int32_t *__restrict__ ns_out,
+                     uint32_t *__restrict__ rep_out, NodeRanks nr) {
+  __shared__ LcpPlanes planes;
+  __shared__ uint32_t wmin[32];
+  __shared__ uint32_t sums[32];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t base = blockIdx.x * kBlockPos, j = base + threadIdx.x;
+  const uint32_t v = j < n ? L[j] : kNoLcp;
+  const BlockLcps bl(v, planes, wmin);
+  bool names = false;
+  if (j < n) {
+    const uint32_t lt = bl.in_warp(warp, v), ltw = bl.warps(v);
+    const uint32_t left = lt & ((1u << lane) - 1u), leftw = ltw & ((1u << warp) - 1u);
+    const size_t at = (size_t)v * c.blocks + blockIdx.x;
+    int32_t ps, rep;
+    if (left || leftw) {
+      const uint32_t w = left ? warp : top_bit(leftw);
+      const uint32_t q = 32u * w + top_bit(left ? left : bl.in_warp(w, v));
+      ps = (int32_t)(base + q);
+      // the first position after PS with a value of at most v (j at the latest)
+      rep = (int32_t)base + bl.first_from(q + 1u, v + 1u);
+    } else {
+      ps = c.last[at];
+      rep = c.open[at];
+      if (rep < 0) rep = (int32_t)base + bl.first_from(0u, v + 1u);
+    }
+    rep_out[j] = (uint32_t)rep;
+    names = rep == (int32_t)j && v >= 1u;
+    if (names) {
+      const uint32_t right = lt & ~((2u << lane) - 1u), rightw = ltw & ~((2u << warp) - 1u);
+      int32_t ns;
+      if (right) ns = (int32_t)(base + 32u * warp + low_bit(right));
+      else if (rightw) {
+        const uint32_t w = low_bit(rightw);
+        ns = (int32_t)(base + 32u * w + low_bit(bl.in_warp(w, v)));
+      } else {
+        ns = c.first[at];
+      }
+      ps_out[j] = ps;
+      ns_out[j] = ns;
+    }
+  }
+  const uint32_t mask = __ballot_sync(kAll, names);
+  const uint32_t x = block_exclusive(lane == 0 ? (uint32_t)__popc(mask) : 0u, sums);
+  if (lane == 0 && j < n) {
+    nr.mask[j >> 5] = mask;
+    nr.before[j >> 5] = x;
+  }
+  if (threadIdx.x == kBlockPos - 1u) nr.base[blockIdx.x] = x;
+}
+
+// Exclusive prefix sum of n counts in place and their total, one block (each
+// thread scans a contiguous chunk).
+__global__ void __launch_bounds__(1024)
+    scan_counts_kernel(uint32_t *__restrict__ a, uint32_t n, uint32_t *__restrict__ total) {
+  __shared__ uint32_t sums[32];
+  const uint32_t chunk = (n + 1023u) / 1024u;
+  const uint32_t lo = min(n, threadIdx.x * chunk), hi = min(n, lo + chunk);
+  uint32_t s = 0;
+  for (uint32_t i = lo; i < hi; ++i) s += a[i];
+  uint32_t run = block_exclusive(s, sums);
+  if (threadIdx.x == 1023u) *total = run + s;
   for (uint32_t i = lo; i < hi; ++i) {
     const uint32_t v = a[i];
     a[i] = run;
     run += v;
   }
-  if (t == 1023 && total) *total = part[1023];
 }
 
-// Stable scatter of one digit pass: elements keep their order within a
-// digit.  A tile is processed in rounds of 256 elements; within a round the
-// rank of an element among equal digits is (earlier rounds) + (earlier
-// warps of this round) + (earlier lanes of its warp, from __match_any_sync).
-__global__ void digit_scatter_kernel(KeyWords key_in, const uint32_t *__restrict__ val_in,
-                                     uint32_t k, uint32_t words, uint32_t dword, uint32_t shift,
-                                     uint32_t nblocks, const uint32_t *__restrict__ offsets,
-                                     KeyWords key_out, uint32_t *__restrict__ val_out) {
-  constexpr int kWarps = kSortThreads / 32;
-  __shared__ uint32_t running[256];
-  __shared__ uint32_t wc[kWarps][256];
-  const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
-  running[t] = offsets[t * nblocks + blockIdx.x];
-  const uint32_t base = blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortItems; ++r) {
-    for (int w = 0; w < kWarps; ++w) wc[w][t] = 0;
-    __syncthreads();
-    const uint32_t e = base + r * kSortThreads + t;
-    const bool live = e < k;
-    const uint32_t active = __ballot_sync(0xFFFFFFFFu, live);
-    uint64_t kv[kMaxWords] = {0, 0, 0, 0};
-    uint32_t vv = 0, d = 0, rank = 0;
-    if (live) {
-      for (uint32_t w = 0; w < words; ++w) kv[w] = key_in.w[w][e];
-      vv = val_in[e];
-      d = (uint32_t)(key_in.w[dword][e] >> shift) & 0xFFu;
-      const uint32_t peers = __match_any_sync(active, d);
-      rank = __popc(peers & ((1u << lane) - 1u));
-      if (rank == 0) wc[warp][d] = __popc(peers);
-    }
-    __syncthreads();
-    {  // thread t owns digit t: exclusive prefix over warps, then advance
-      uint32_t run = running[t];
-      for (int w = 0; w < kWarps; ++w) {
-        const uint32_t c = wc[w][t];
-        wc[w][t] = run;
-        run += c;
-      }
-      running[t] = run;
-    }
-    __syncthreads();
-    if (live) {
-      const uint32_t pos = wc[warp][d] + rank;
-      for (uint32_t w = 0; w < words; ++w) key_out.w[w][pos] = kv[w];
-      val_out[pos] = vv;
-    }
-    __syncthreads();
-  }
-}
-
-// ----------------------------------------------------------------- lcp ---
-__global__ void lcp_kernel(KeyWords key, uint32_t k, uint32_t words, uint32_t fields,
-                           uint32_t bits, int32_t *__restrict__ L) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j + 1 >= k) return;
-  uint32_t same = fields;
-  for (uint32_t w = 0; w < words; ++w) {
-    const uint64_t x = key.w[w][j] ^ key.w[w][j + 1];
-    if (x) {
-      same = (w * 64 + (uint32_t)__clzll((long long)x)) / bits;
-      break;
-    }
-  }
-  L[j] = (int32_t)min(same, fields);
-}
-
-// ------------------------------------------------- nearest smaller values ---
-// Levels of a 32-ary tree of minima over L (level 0 = L itself).
-struct MinTree {
-  int32_t *lvl[8];
-  uint32_t len[8];
-  int levels;
+struct FieldTimes {
+  int64_t t[kMaxFields];
 };
 
-__global__ void min_level_kernel(const int32_t *__restrict__ in, uint32_t n,
-                                 int32_t *__restrict__ out) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t m = (n + 31) / 32;
-  if (i >= m) return;
-  int32_t v = INT32_MAX;
-  for (uint32_t q = i * 32; q < min(n, i * 32 + 32); ++q) v = min(v, in[q]);
-  out[i] = v;
-}
-
-// Nearest index q < j (dir < 0) or q > j (dir > 0) with L[q] < x, or -1.
-__device__ int32_t nearest_below(const MinTree &mt, uint32_t j, int32_t x, int dir) {
-  int level = 0;
-  int64_t cur = j;  // exclusive bound at the current level
-  int64_t found = -1;
-  while (true) {
-    const int32_t *a = mt.lvl[level];
-    const int64_t n = mt.len[level];
-    if (dir < 0) {
-      const int64_t start = (cur / 32) * 32;
-      for (int64_t q = cur - 1; q >= start; --q)
-        if (a[q] < x) { found = q; break; }
-      if (found >= 0 || start == 0 || level + 1 >= mt.levels) break;
-      cur = start / 32;
-    } else {
-      const int64_t end = n < (cur / 32) * 32 + 32 ? n : (cur / 32) * 32 + 32;
-      for (int64_t q = cur + 1; q < end; ++q)
-        if (a[q] < x) { found = q; break; }
-      if (found >= 0 || end >= n || level + 1 >= mt.levels) break;
-      cur = end / 32 - 1;
-      // the next level is searched strictly after index cur (this block)
-    }
-    ++level;
-  }
-  if (found < 0) return -1;
-  while (level > 0) {  // descend into the block that holds the minimum
-    --level;
-    const int32_t *a = mt.lvl[level];
-    const int64_t n = mt.len[level];
-    const int64_t lo = found * 32, hi = n < lo + 32 ? n : lo + 32;
-    int64_t pick = -1;
-    if (dir < 0) {
-      for (int64_t q = hi - 1; q >= lo; --q)
-        if (a[q] < x) { pick = q; break; }
-    } else {
-      for (int64_t q = lo; q < hi; ++q)
-        if (a[q] < x) { pick = q; break; }
-    }
-    found = pick;
-  }
-  return (int32_t)found;
-}
-
-// For each lcp position: PS (previous strictly smaller), NS (next strictly
-// smaller) and the interval link (previous position with an equal value
-// and only larger ones between, else itself).
-__global__ void smaller_values_kernel(MinTree mt, uint32_t n, int32_t *__restrict__ ps,
-                                      int32_t *__restrict__ ns, int32_t *__restrict__ link) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const int32_t v = mt.lvl[0][j];
-  ps[j] = nearest_below(mt, j, v, -1);
-  ns[j] = nearest_below(mt, j, v, +1);
-  const int32_t pse = nearest_below(mt, j, v + 1, -1);  // previous smaller-or-equal
-  link[j] = (pse >= 0 && mt.lvl[0][pse] == v) ? pse : (int32_t)j;
-}
-
-__global__ void jump_kernel(const int32_t *__restrict__ in, uint32_t n,
-                            int32_t *__restrict__ out) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < n) out[j] = in[in[j]];
-}
-
-__global__ void rep_flags_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ rep,
-                                 uint32_t n, uint32_t *__restrict__ flag) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < n) flag[j] = (rep[j] == (int32_t)j && L[j] >= 1) ? 1u : 0u;
-}
-
-// Node ids: 0 the root, 1 + id[j] the interval named by position j, then the
+// Node ids: 0 the root, 1 + rank of the naming position an interval, then the
 // leaves in sorted order.
-__global__ void internal_nodes_kernel(const int32_t *__restrict__ L,
-                                      const int32_t *__restrict__ rep,
-                                      const int32_t *__restrict__ ps,
-                                      const int32_t *__restrict__ ns,
-                                      const uint32_t *__restrict__ id, uint32_t n,
-                                      const int64_t *__restrict__ times,
-                                      int64_t *__restrict__ parent, int64_t *__restrict__ time) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n || rep[j] != (int32_t)j || L[j] < 1) return;
-  const uint32_t node = 1 + id[j];
-  const int32_t a = ps[j], b = ns[j];
-  const int32_t La = a >= 0 ? L[a] : -1, Lb = b >= 0 ? L[b] : -1;
-  int64_t par = 0;
-  if (La > 0 || Lb > 0) par = 1 + id[rep[La >= Lb ? a : b]];
-  parent[node] = par;
-  time[node] = times[L[j] - 1];
-}
-
-__global__ void leaves_kernel(const int32_t *__restrict__ L, const int32_t *__restrict__ rep,
-                              const uint32_t *__restrict__ id, const uint32_t *__restrict__ val,
-                              uint32_t k, uint32_t internal, int64_t T,
-                              int64_t *__restrict__ parent, int64_t *__restrict__ time,
-                              uint32_t *__restrict__ leaf_of_sample) {
+__global__ void nodes_kernel(const uint16_t *__restrict__ L, uint32_t k,
+                             const int32_t *__restrict__ ps, const int32_t *__restrict__ ns,
+                             const uint32_t *__restrict__ rep, NodeRanks nr,
+                             const uint32_t *__restrict__ val,
+                             const uint32_t *__restrict__ internal,
+                             const __grid_constant__ FieldTimes times, int64_t T,
+                             int64_t *__restrict__ parent, int64_t *__restrict__ time,
+                             uint32_t *__restrict__ leaf_of_sample) {
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= k) return;
-  const int32_t La = p >= 1 ? L[p - 1] : -1, Lb = p + 1 < k ? L[p] : -1;
+  const uint32_t n = k - 1u;
+  const uint32_t total = *internal;
+  if (p == 0) {
+    parent[0] = -1;
+    time[0] = -1;
+  }
+  const int32_t Lp = p < n ? (int32_t)L[p] : -1;
+  if (p < n && (nr.mask[p >> 5] >> (p & 31u) & 1u)) {
+    const uint32_t node = 1u + node_rank(nr, p);
+    const int32_t a = ps[p], b = ns[p];
+    const int32_t La = a >= 0 ? (int32_t)L[a] : -1, Lb = b >= 0 ? (int32_t)L[b] : -1;
+    int64_t par = 0;
+    if (La > 0 || Lb > 0) par = 1 + (int64_t)node_rank(nr, rep[La >= Lb ? a : b]);
+    parent[node] = par;
+    time[node] = times.t[Lp - 1];
+  }
+  const int32_t La = p >= 1u ? (int32_t)L[p - 1u] : -1;
   int64_t par = 0;
-  if (La > 0 || Lb > 0) par = 1 + id[rep[La >= Lb ? p - 1 : p]];
-  const uint32_t node = 1 + internal + p;
+  if (La > 0 || Lp > 0) par = 1 + (int64_t)node_rank(nr, rep[La >= Lp ? p - 1u : p]);
+  const uint32_t node = 1u + total + p;
   parent[node] = par;
   time[node] = T;
   leaf_of_sample[val[p]] = node;
 }
 
-__global__ void root_kernel(int64_t *__restrict__ parent, int64_t *__restrict__ time) {
-  parent[0] = -1;
-  time[0] = -1;
-}
-
 inline uint32_t blocks_for(uint64_t n, uint32_t threads) {
   return (uint32_t)((n + threads - 1) / threads);
+}
+
+// Device memory of the current device that a kernel can read in place.
+bool readable_here(const void *ptr) {
+  int dev = 0;
+  cudaPointerAttributes attr;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&attr, ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return attr.type == cudaMemoryTypeDevice && attr.device == dev && ((uintptr_t)ptr & 7u) == 0;
+}
+
+// Keys of k surfaces, sorted: key[*cur], val[*cur].
+template <int K>
+cudaError_t sort_keys(const KeyPlan &kp, const uint64_t *surf, uint32_t k, KeyWords (&key)[2],
+                      uint32_t *(&val)[2], uint32_t *hist, uint32_t *digits, int *cur,
+                      cudaStream_t st) {
+  // over the significant bits only (the top fields * bits, rounded up to whole
+  // 8-bit digits, which then never straddle two key words)
+  const uint32_t passes = (kp.fields * kp.bits + 7) / 8;
+  *cur = 0;
+  make_keys_kernel<K><<<blocks_for(k, 128), 128, 0, st>>>(kp, surf, k, key[0], val[0]);
+  if (K == 1 && k <= kSmallSort) {
+    // the limit for every k: other threads launch too
+    const cudaError_t e =
+        cudaFuncSetAttribute(small_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)small_sort_smem(kSmallSort));
+    if (e != cudaSuccess) return e;
+    small_sort_kernel<<<1, 1024, small_sort_smem(k), st>>>(key[0].w[0], k, passes, key[1].w[0], val[1]);
+    *cur = 1;
+    return cudaGetLastError();
+  }
+  const uint32_t ntiles = blocks_for(k, kSortTile);
+  for (uint32_t i = 0; i < passes; ++i) {
+    const uint32_t top = 8 * (passes - 1 - i);  // digit's first bit from the top
+    const uint32_t dword = top / 64, shift = 64 - top % 64 - 8;
+    digit_histogram_kernel<<<ntiles, kSortThreads, 0, st>>>(key[*cur].w[dword], k, shift, ntiles,
+                                                            hist);
+    digit_scan_kernel<<<256, 256, 0, st>>>(hist, ntiles, digits);
+    digit_scatter_kernel<K><<<ntiles, kSortThreads, 0, st>>>(
+        key[*cur], val[*cur], k, dword, shift, ntiles, hist, digits, key[1 - *cur],
+        val[1 - *cur]);
+    *cur = 1 - *cur;
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -353,122 +734,103 @@ int hsga_reconstruct(const uint64_t *surf, uint32_t k, uint32_t surface_words, u
   KeyPlan kp{};
   kp.fields = (uint32_t)order.size();
   kp.bits = b;
-  kp.words = K;
-  std::vector<int64_t> times(kp.fields > 0 ? kp.fields : 1, -1);
+  FieldTimes times{};
   for (uint32_t j = 0; j < kp.fields; ++j) {
     kp.src[j] = order[j] * b;
-    times[j] = dep[order[j]] * (int64_t)kk;
+    times.t[j] = dep[order[j]] * (int64_t)kk;
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
   AllocHooks al = current_allocator();
-  const uint32_t nblocks = blocks_for(k, kSortTile);
+  const uint32_t ntiles = blocks_for(k, kSortTile);
   const uint32_t n = k - 1;  // lcp positions
-  // scratch
-  std::vector<void *> held;
-  auto alloc = [&](size_t bytes) {
-    void *p = device_alloc(al, bytes < 256 ? 256 : bytes, st);
-    held.push_back(p);
-    return p;
-  };
-  KeyWords key[2] = {};
-  for (int h = 0; h < 2; ++h)
-    for (uint32_t w = 0; w < K; ++w) key[h].w[w] = (uint64_t *)alloc(8ull * k);
-  uint32_t *val[2] = {(uint32_t *)alloc(4ull * k), (uint32_t *)alloc(4ull * k)};
-  uint32_t *hist = (uint32_t *)alloc(4ull * 256 * nblocks);
-  uint64_t *dsurf = (uint64_t *)alloc(8ull * k * K);
-  int64_t *dtimes = (int64_t *)alloc(8ull * times.size());
-  int32_t *L = (int32_t *)alloc(4ull * (n + 1));
-  int32_t *ps = (int32_t *)alloc(4ull * (n + 1));
-  int32_t *ns = (int32_t *)alloc(4ull * (n + 1));
-  int32_t *link[2] = {(int32_t *)alloc(4ull * (n + 1)), (int32_t *)alloc(4ull * (n + 1))};
-  uint32_t *id = (uint32_t *)alloc(4ull * (n + 1));
-  uint32_t *total = (uint32_t *)alloc(4);
+  const uint32_t nblocks = blocks_for(n, kBlockPos);
   const bool dev_out = device_pointer(parent_out);
-  int64_t *dparent = dev_out ? parent_out : (int64_t *)alloc(8 * need_nodes);
-  int64_t *dtime = dev_out ? time_out : (int64_t *)alloc(8 * need_nodes);
-  uint32_t *dleaf = dev_out ? leaf_of_sample : (uint32_t *)alloc(4ull * k);
-  MinTree mt{};
-  {
-    uint32_t len = n;
-    mt.lvl[0] = L;
-    mt.len[0] = len;
-    mt.levels = 1;
-    while (len > 32 && mt.levels < 8) {
-      len = (len + 31) / 32;
-      mt.lvl[mt.levels] = (int32_t *)alloc(4ull * len);
-      mt.len[mt.levels] = len;
-      ++mt.levels;
-    }
+  const bool in_place = readable_here(surf);
+  // scratch: one allocation, carved up
+  size_t bytes = 0;
+  const auto take = [&](size_t want) {
+    const size_t at = bytes;
+    bytes += (want + 255u) & ~(size_t)255u;
+    return at;
+  };
+  size_t at_key[2][kMaxWords] = {}, at_val[2];
+  for (int h = 0; h < 2; ++h) {
+    for (uint32_t w = 0; w < K; ++w) at_key[h][w] = take(8ull * k);
+    at_val[h] = take(4ull * k);
   }
-  int status = HSGA_OK;
-  for (void *p : held)
-    if (!p) status = HSGA_ERR_OOM;
+  const size_t at_hist = take(4ull * 256 * ntiles), at_digits = take(4 * 256);
+  const size_t at_surf = in_place ? 0 : take(8ull * k * K);
+  const size_t at_L = take(2ull * n);
+  const uint32_t rows = kp.fields + 1;
+  const size_t at_carry = take(12ull * rows * nblocks);
+  const size_t at_ps = take(4ull * n), at_ns = take(4ull * n), at_rep = take(4ull * n);
+  const size_t at_mask = take(4ull * 32 * nblocks), at_before = take(4ull * 32 * nblocks);
+  const size_t at_base = take(4ull * nblocks), at_total = take(4);
+  const size_t at_parent = dev_out ? 0 : take(8 * need_nodes);
+  const size_t at_time = dev_out ? 0 : take(8 * need_nodes);
+  const size_t at_leaf = dev_out ? 0 : take(4ull * k);
+  unsigned char *const mem = (unsigned char *)device_alloc(al, bytes, st);
+  if (!mem) return HSGA_ERR_OOM;
+  KeyWords key[2] = {};
+  uint32_t *val[2];
+  for (int h = 0; h < 2; ++h) {
+    for (uint32_t w = 0; w < K; ++w) key[h].w[w] = (uint64_t *)(mem + at_key[h][w]);
+    val[h] = (uint32_t *)(mem + at_val[h]);
+  }
+  uint16_t *const L = (uint16_t *)(mem + at_L);
+  int32_t *const carry = (int32_t *)(mem + at_carry);
+  const size_t per = (size_t)rows * nblocks;
+  const Carries carries{carry, carry + per, carry + 2 * per, nblocks};
+  uint32_t *const hist = (uint32_t *)(mem + at_hist), *const digits = (uint32_t *)(mem + at_digits);
+  int32_t *const ps = (int32_t *)(mem + at_ps), *const ns = (int32_t *)(mem + at_ns);
+  uint32_t *const rep = (uint32_t *)(mem + at_rep), *const total = (uint32_t *)(mem + at_total);
+  const NodeRanks nr{(uint32_t *)(mem + at_mask), (uint32_t *)(mem + at_before),
+                     (uint32_t *)(mem + at_base)};
+  int64_t *const dparent = dev_out ? parent_out : (int64_t *)(mem + at_parent);
+  int64_t *const dtime = dev_out ? time_out : (int64_t *)(mem + at_time);
+  uint32_t *const dleaf = dev_out ? leaf_of_sample : (uint32_t *)(mem + at_leaf);
   cudaError_t e = cudaSuccess;
-  uint32_t internal = 0;
-  if (status == HSGA_OK) {
-    e = cudaMemcpyAsync(dsurf, surf, 8ull * k * K, cudaMemcpyDefault, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(dtimes, times.data(), 8 * times.size(), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-      make_keys_kernel<<<blocks_for(k, 256), 256, 0, st>>>(kp, dsurf, k, key[0], val[0]);
-      // sort over the significant bits only (the top fields * bits, rounded
-      // up to whole 8-bit digits, which then never straddle two key words)
-      const uint32_t passes = (kp.fields * b + 7) / 8;
-      int cur = 0;
-      for (uint32_t ps_i = 0; ps_i < passes; ++ps_i) {
-        const uint32_t top = 8 * (passes - 1 - ps_i);  // digit's first bit from the top
-        const uint32_t dword = top / 64, shift = 64 - top % 64 - 8;
-        digit_histogram_kernel<<<nblocks, kSortThreads, 0, st>>>(key[cur].w[dword], k, shift,
-                                                                 nblocks, hist);
-        exclusive_scan_kernel<<<1, 1024, 0, st>>>(hist, 256 * nblocks, nullptr);
-        digit_scatter_kernel<<<nblocks, kSortThreads, 0, st>>>(key[cur], val[cur], k, K, dword,
-                                                               shift, nblocks, hist,
-                                                               key[1 - cur], val[1 - cur]);
-        cur = 1 - cur;
-      }
-      root_kernel<<<1, 1, 0, st>>>(dparent, dtime);
-      if (n > 0) {
-        lcp_kernel<<<blocks_for(n, 256), 256, 0, st>>>(key[cur], k, K, kp.fields, b, L);
-        for (int l = 1; l < mt.levels; ++l)
-          min_level_kernel<<<blocks_for(mt.len[l], 256), 256, 0, st>>>(mt.lvl[l - 1],
-                                                                       mt.len[l - 1], mt.lvl[l]);
-        smaller_values_kernel<<<blocks_for(n, 256), 256, 0, st>>>(mt, n, ps, ns, link[0]);
-        int lc = 0;
-        for (uint32_t span = 1; span < n; span <<= 1) {
-          jump_kernel<<<blocks_for(n, 256), 256, 0, st>>>(link[lc], n, link[1 - lc]);
-          lc = 1 - lc;
-        }
-        rep_flags_kernel<<<blocks_for(n, 256), 256, 0, st>>>(L, link[lc], n, id);
-        exclusive_scan_kernel<<<1, 1024, 0, st>>>(id, n, total);
-        e = cudaMemcpyAsync(&internal, total, 4, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e == cudaSuccess) {
-          internal_nodes_kernel<<<blocks_for(n, 256), 256, 0, st>>>(L, link[lc], ps, ns, id, n,
-                                                                    dtimes, dparent, dtime);
-          leaves_kernel<<<blocks_for(k, 256), 256, 0, st>>>(L, link[lc], id, val[cur], k,
-                                                            internal, (int64_t)generations,
-                                                            dparent, dtime, dleaf);
-        }
-      } else {
-        leaves_kernel<<<1, 32, 0, st>>>(L, link[0], id, val[cur], k, 0, (int64_t)generations,
-                                        dparent, dtime, dleaf);
-      }
-      if (e == cudaSuccess) e = cudaGetLastError();
-    }
-    const uint32_t nodes = 1 + internal + k;
-    if (e == cudaSuccess && !dev_out) {
-      e = cudaMemcpyAsync(parent_out, dparent, 8ull * nodes, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(time_out, dtime, 8ull * nodes, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(leaf_of_sample, dleaf, 4ull * k, cudaMemcpyDeviceToHost, st);
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) status = HSGA_ERR_CUDA;
-    *n_nodes = nodes;
+  const uint64_t *dsurf = surf;
+  if (!in_place) {
+    e = cudaMemcpyAsync(mem + at_surf, surf, 8ull * k * K, cudaMemcpyDefault, st);
+    dsurf = (const uint64_t *)(mem + at_surf);
   }
-  for (void *p : held)
-    if (p) device_free(al, p, st);
-  cudaStreamSynchronize(st);
-  return status;
+  int cur = 0;
+  if (e == cudaSuccess)
+    e = K == 1   ? sort_keys<1>(kp, dsurf, k, key, val, hist, digits, &cur, st)
+        : K == 2 ? sort_keys<2>(kp, dsurf, k, key, val, hist, digits, &cur, st)
+                 : sort_keys<4>(kp, dsurf, k, key, val, hist, digits, &cur, st);
+  if (e == cudaSuccess) {
+    if (n > 0) {
+      if (K == 1)
+        lcp_kernel<1><<<nblocks, kBlockPos, 0, st>>>(key[cur], n, kp.fields, b, L, carries);
+      else if (K == 2)
+        lcp_kernel<2><<<nblocks, kBlockPos, 0, st>>>(key[cur], n, kp.fields, b, L, carries);
+      else
+        lcp_kernel<4><<<nblocks, kBlockPos, 0, st>>>(key[cur], n, kp.fields, b, L, carries);
+      carry_kernel<<<rows, 64, 0, st>>>(carries);
+      intervals_kernel<<<nblocks, kBlockPos, 0, st>>>(L, n, carries, ps, ns, rep, nr);
+    }
+    scan_counts_kernel<<<1, 1024, 0, st>>>(nr.base, n > 0 ? nblocks : 0u, total);
+    nodes_kernel<<<blocks_for(k, 256), 256, 0, st>>>(L, k, ps, ns, rep, nr, val[cur],
+                                                     total, times, (int64_t)generations, dparent,
+                                                     dtime, dleaf);
+    e = cudaGetLastError();
+  }
+  uint32_t internal = 0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&internal, total, 4, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  const uint32_t nodes = 1 + internal + k;
+  if (e == cudaSuccess && !dev_out) {
+    e = cudaMemcpyAsync(parent_out, dparent, 8ull * nodes, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(time_out, dtime, 8ull * nodes, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(leaf_of_sample, dleaf, 4ull * k, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  }
+  if (e != cudaSuccess) cudaStreamSynchronize(st);  // the scratch may still be in use
+  device_free(al, mem, st);
+  *n_nodes = nodes;
+  return e == cudaSuccess ? HSGA_OK : HSGA_ERR_CUDA;
 }
