@@ -934,8 +934,13 @@ cudaError_t launch_step_resident(const RunParams &p, const ResidentPlan &plan, u
                                  uint32_t ngen, bool premigrated, uint32_t *t, uint64_t *s,
                                  uint64_t *rec, int *err, cudaStream_t stream) {
   ResidentFn fn = pick(p, plan.tile);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)plan.smem);
+  // the device's limit, whatever the plan: other threads launch other tiles
+  int dev = 0, limit = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
   if (e != cudaSuccess) return e;
   RunParams pp = p;
   ResidentTile tile = plan.tile;

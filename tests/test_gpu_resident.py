@@ -74,3 +74,28 @@ def test_records_are_never_torn(hb, policy):
                 g.sync()
             x, y = a.population(), b.population()
             assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
+
+
+def test_tiles_of_two_sizes_from_two_threads(hb):
+    """Each launch gets its own tile's shared memory, whatever another thread
+    launches the same kernel with."""
+    import threading
+    shapes, failed = [(76, 128), (150, 200)], []
+
+    def steps(rows, cols):
+        try:
+            with hb.Grid(kernel=hb.KERNEL_RESIDENT, rows=rows, cols=cols, n=32, tournament=2,
+                         policy="tilted", bits=1, seed=1) as g:
+                g.set_population(*inputs.random_population(g.agents, seed=1), 0)
+                for _ in range(2000):
+                    g.run(1)
+                g.sync()
+        except Exception as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=steps, args=s) for s in shapes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
