@@ -521,10 +521,24 @@ int advance(hsga_grid *g, uint64_t n) {
       done += m;
     }
   } else {
+    // moves of the generations to come, in the record buffer (64 bytes per
+    // island) that streamed steps have no other use for; nothing outlives the call
+    uint16_t *const moves = (uint16_t *)g->rec;
+    uint8_t *const leave = (uint8_t *)(moves + 8 * (size_t)g->p.islands);
     for (uint64_t k = 0; k < n && e == cudaSuccess; ++k) {
       const uint64_t G = g->G + k;
       const bool do_mig = migrates(g->p, G) && !(g->premigrated && k == 0);
-      e = launch_step_streamed(g->p, g->splan, (uint32_t)G, do_mig, g->trait[g->cur], g->surf[g->cur],
+      Moves mv;
+      if (g->splan.moves_ahead) {
+        const size_t even = (k & 1) ? g->p.islands : 0, odd = g->p.islands - even;
+        if (do_mig && k >= 2) mv.now = moves + 4 * even;
+        if (k >= 1 && k + 1 < n && migrates(g->p, G + 1)) {
+          mv.next = moves + 4 * odd;
+          mv.leave_next = leave + odd;
+        }
+        if (k + 2 < n && migrates(g->p, G + 2)) mv.leave_after = leave + even;
+      }
+      e = launch_step_streamed(g->p, g->splan, (uint32_t)G, do_mig, mv, g->trait[g->cur], g->surf[g->cur],
                                g->trait[1 - g->cur], g->surf[1 - g->cur], g->err, g->stream);
       g->cur = 1 - g->cur;
       g->launches++;

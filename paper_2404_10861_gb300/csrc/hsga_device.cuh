@@ -206,6 +206,24 @@ __device__ __forceinline__ Words4 philox_rk(const RunParams &p, uint32_t c0, uin
   return Words4{c0, c1, c2, c3};
 }
 
+// The same with the round keys of any holder of them.
+template <class Keys>
+__device__ __forceinline__ Words4 philox_keys(const Keys &k, uint32_t c0, uint32_t c1, uint32_t c2,
+                                              uint32_t c3) {
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    const uint64_t p0 = (uint64_t)c0 * kPhiloxM0;
+    const uint64_t p1 = (uint64_t)c2 * kPhiloxM1;
+    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.rk0[r];
+    const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.rk1[r];
+    c0 = n0;
+    c1 = (uint32_t)p1;
+    c2 = n2;
+    c3 = (uint32_t)p0;
+  }
+  return Words4{c0, c1, c2, c3};
+}
+
 // Per-generation deposit parameters: a whole synchronous generation shares
 // T, hence the site.  A b-bit field never straddles the two 32-bit halves
 // of the surface (b divides 32), so each insert is one bit-select per half:

@@ -11,16 +11,29 @@
 namespace hsga {
 namespace {
 
-constexpr int kFlatBlocksPerSM = 5;         // 20 warps
 constexpr int kFlatMaxSmem = 160 * 1024;  // limit set on the kernels; one block uses far less
 
-template <int K, bool T2, int NN, bool FLT>
-__global__ void __launch_bounds__(kFlatThreads, kFlatBlocksPerSM)
+// LARGE: the instance for grids that a launch takes long over.  Integer fitness
+// with at most one surface word is bound by issue and has later generations'
+// migration worked out ahead (hsga_moves.cuh; 500x500 islands of 8 24.1 us
+// against 28.0, 512x1024 of 24 69.6 against 73.3); binary32 fitness and wide
+// surfaces gain nothing from that (256x512 of 32 with two words 29.9 against
+// 28.9).
+template <int K, bool FLT>
+constexpr bool kFlatAhead = K <= 1 && !FLT;
+
+// 20 warps per SM at least; 28 fit by themselves where a tournament of 2 and
+// narrow surfaces leave the registers, and planning must not take them away.
+template <int K, bool T2, bool FLT, bool LARGE>
+constexpr int kFlatBlocksPerSM = LARGE && T2 && !FLT && K <= 2 ? 7 : 5;
+
+template <int K, bool T2, int NN, bool FLT, bool LARGE>
+__global__ void __launch_bounds__(kFlatThreads, (kFlatBlocksPerSM<K, T2, FLT, LARGE>))
     step_flat_kernel(RunParams p, FlatDeposit<K> dep, uint32_t G, uint32_t group, int migrate,
-                     int bulk,
-                     const uint32_t *__restrict__ tin, const uint64_t *__restrict__ sin,
-                     uint32_t *__restrict__ tout, uint64_t *__restrict__ sout,
-                     int *__restrict__ err) {
+                     int bulk, int back, Moves mv, const uint32_t *__restrict__ tin,
+                     const uint64_t *__restrict__ sin, uint32_t *__restrict__ tout,
+                     uint64_t *__restrict__ sout, int *__restrict__ err) {
+  constexpr bool AHEAD = LARGE && kFlatAhead<K, FLT>;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[kFlatWarps];
   const uint32_t lane = threadIdx.x & 31u, wib = __shfl_sync(kFull, threadIdx.x >> 5, 0);
@@ -37,28 +50,45 @@ __global__ void __launch_bounds__(kFlatThreads, kFlatBlocksPerSM)
   __syncwarp();
   const uint32_t groups = (p.islands + group - 1) / group;
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  for (uint32_t grp = blockIdx.x * kFlatWarps + wib; grp < groups; grp += gridDim.x * kFlatWarps) {
-    if (!flat_group<K, T2, NN, FLT>(p, p, dep, migrate != 0, bulk != 0, grp * group, group, G, tin,
-                                    sin, tout, sout, st)) {
-      // give up: record the timeout, wait (bounded) for the copy, leave
+  const uint32_t warp = blockIdx.x * kFlatWarps + wib, nwarps = gridDim.x * kFlatWarps;
+  const bool planned = AHEAD && mv.now != nullptr;
+  const auto first_of = [&](uint32_t grp) { 
+    return (LARGE && back ? groups - 1u - grp : grp) * group;
+  };
+  const auto move_of = [&](uint32_t grp) {
+    return planned && grp < groups
+               ? load_move(mv, first_of(grp), min(group, p.islands - first_of(grp)))
+               : 0u;
+  };
+  uint32_t next = move_of(warp);
+  [[maybe_unused]] Planner planner(p, mv, warp, nwarps);
+  for (uint32_t grp = warp; grp < groups; grp += nwarps) {
+    const uint32_t move = next;
+    next = move_of(grp + nwarps);
+    if (!flat_group<K, T2, NN, FLT, LARGE>(p, p, dep, migrate != 0, bulk != 0, first_of(grp),
+                                           group, G, planned, move, tin, sin, tout, sout, st)) {
+      // give up: record the timeout, wait (bounded) for the copy, leave (once
+      // the moves that later launches read are written)
       if (lane == 0) {
         atomicCAS(err, 0, kDevErrWaitTimeout);
         mbar_wait(st.bar, st.phase);
       }
       __syncwarp();
-      return;
+      break;
     }
+    if constexpr (AHEAD) planner.template visit<NN>(p, p, mv, G, group);
   }
+  if constexpr (AHEAD) planner.template rest<NN>(p, p, mv, G);
 }
 
 // Resident blocks and the shared memory to ask for per block: padded so that
 // no further block fits on an SM, since the next launch, scheduled early,
 // would park one there beside the running ones.
-template <int K, bool T2, int NN, bool FLT>
+template <int K, bool T2, int NN, bool FLT, bool LARGE>
 bool flat_plan(const RunParams &p, StreamPlan *out) {
-  const auto fn = step_flat_kernel<K, T2, NN, FLT>;
   const size_t need = kFlatWarps * flat_stage_bytes(p.n, K);
   int dev = 0, sms = 0, per_sm = 0, sm_smem = 0, reserved = 0;
+  const auto fn = step_flat_kernel<K, T2, NN, FLT, LARGE>;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
@@ -88,6 +118,11 @@ bool flat_plan(const RunParams &p, StreamPlan *out) {
     }
   }
   out->blocks = sms * per_sm;
+  out->back = LARGE && planes_exceed_l2(p);
+  // ahead only if the warps take at least two groups each (one: 128x256 of 48)
+  out->moves_ahead =
+      LARGE && kFlatAhead<K, FLT> && p.islands / (uint32_t)out->group >= 2u * warps;
+  out->large = kFlatAhead<K, FLT> ? out->moves_ahead : out->back;
   out->smem = pad > used && pad * per_sm <= (size_t)sm_smem && pad <= kFlatMaxSmem
                   ? pad - (size_t)reserved
                   : need;
@@ -96,8 +131,9 @@ bool flat_plan(const RunParams &p, StreamPlan *out) {
 
 template <int K, bool T2, int NN, bool FLT>
 cudaError_t launch_flat_t(const RunParams &p, const StreamPlan &plan, const FlatDeposit<K> &dep,
-                          uint32_t G, bool do_mig, const uint32_t *tin, const uint64_t *sin,
-                          uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream) {
+                          uint32_t G, bool do_mig, const Moves &mv, const uint32_t *tin,
+                          const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
+                          cudaStream_t stream) {
   const uint32_t groups = (p.islands + plan.group - 1) / plan.group;
   const uint32_t need = (groups + kFlatWarps - 1) / kFlatWarps;
   cudaLaunchConfig_t cfg = {};
@@ -111,8 +147,12 @@ cudaError_t launch_flat_t(const RunParams &p, const StreamPlan &plan, const Flat
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const int bulk = (((uintptr_t)tin | (uintptr_t)sin | (uintptr_t)sout) & 15u) == 0 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, step_flat_kernel<K, T2, NN, FLT>, p, dep, G,
-                            (uint32_t)plan.group, do_mig ? 1 : 0, bulk, tin, sin, tout, sout, err);
+  const int back = plan.back && (G & 1u) ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg,
+                            plan.large ? step_flat_kernel<K, T2, NN, FLT, true>
+                                       : step_flat_kernel<K, T2, NN, FLT, false>,
+                            p, dep, G, (uint32_t)plan.group, do_mig ? 1 : 0, bulk, back, mv, tin,
+                            sin, tout, sout, err);
 }
 
 // Calls F::run<K, T2, NN, FLT>(args...) for a configuration.
@@ -142,16 +182,17 @@ auto flat_pick_words(const RunParams &p, A &&...args) {
 struct Plan {
   template <int K, bool T2, int NN, bool FLT>
   static bool run(const RunParams &p, StreamPlan *out) {
-    return flat_plan<K, T2, NN, FLT>(p, out);
+    return flat_plan<K, T2, NN, FLT, true>(p, out) &&
+           (out->large || flat_plan<K, T2, NN, FLT, false>(p, out));
   }
 };
 
 struct Launch {
   template <int K, bool T2, int NN, bool FLT>
   static cudaError_t run(const RunParams &p, const StreamPlan &plan, uint32_t G, bool do_mig,
-                         const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
+                         const Moves &mv, const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
                          int *err, cudaStream_t stream) {
-    return launch_flat_t<K, T2, NN, FLT>(p, plan, flat_deposit<K>(p, G), G, do_mig, tin, sin,
+    return launch_flat_t<K, T2, NN, FLT>(p, plan, flat_deposit<K>(p, G), G, do_mig, mv, tin, sin,
                                          tout, sout, err, stream);
   }
 };
@@ -163,9 +204,9 @@ bool flat_stream_plan(const RunParams &p, StreamPlan *out) {
 }
 
 cudaError_t launch_step_flat(const RunParams &p, const StreamPlan &plan, uint32_t G, bool do_mig,
-                             const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
-                             uint64_t *sout, int *err, cudaStream_t stream) {
-  return flat_pick_words<Launch>(p, plan, G, do_mig, tin, sin, tout, sout, err, stream);
+                             const Moves &mv, const uint32_t *tin, const uint64_t *sin,
+                             uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream) {
+  return flat_pick_words<Launch>(p, plan, G, do_mig, mv, tin, sin, tout, sout, err, stream);
 }
 
 }  // namespace hsga

@@ -17,15 +17,16 @@
 // us per generation, here and on the kernels before it (a lane per agent in
 // registers; for binary32 fitness and wide surfaces a warp per island after
 // two migration launches): 128x256 islands of 48 8.7 (18.5), of 17 5.5
-// (10.3), of 64 with tournament 5 21.3 (43.0); 500x500 of 32, tournament 5,
-// binary32 94 (110); 256x512 of 32 with four surface words 54.6 (66.2), of
+// (10.3), of 64 with tournament 5 21.4 (43.0); 500x500 of 32, tournament 5,
+// binary32 94.7 (110); 256x512 of 32 with four surface words 46.2 (66.2), of
 // which 44.5 are its 72 bytes per agent at the measured copy bandwidth; 20x20
-// of 32, binary32 3.5 (14.4).  Three children per lane in flight and 20 warps
+// of 32, binary32 3.4 (14.4).  Three children per lane in flight and 20 warps
 // per SM: 128x256x48 takes a fifth longer with four, a tenth with two (32
 // warps).  Bound by issue: 113 warp instructions per 32 children at n = 48, 51
 // of them on the ALU pipe (two cycles each).
 #pragma once
 
+#include "hsga_moves.cuh"
 #include "hsga_stage.cuh"
 
 namespace hsga {
@@ -46,23 +47,6 @@ __host__ __device__ __forceinline__ uint32_t flat_stage_bytes(uint32_t n, uint32
 struct RoundKeys {
   uint32_t rk0[10], rk1[10];
 };
-
-template <class Keys>
-__device__ __forceinline__ Words4 philox_keys(const Keys &k, uint32_t c0, uint32_t c1, uint32_t c2,
-                                              uint32_t c3) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint64_t p0 = (uint64_t)c0 * kPhiloxM0;
-    const uint64_t p1 = (uint64_t)c2 * kPhiloxM1;
-    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.rk0[r];
-    const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.rk1[r];
-    c0 = n0;
-    c1 = (uint32_t)p1;
-    c2 = n2;
-    c3 = (uint32_t)p0;
-  }
-  return Words4{c0, c1, c2, c3};
-}
 
 // What a generation writes into K-word surfaces, per 32-bit half as in
 // Deposit: half = (half & clear) | ((value << shift) & ~clear).
@@ -163,15 +147,26 @@ __device__ __forceinline__ void flat_heads(const Keys &keys, uint32_t n, uint32_
   st.x0 = (uint32_t)(((uint64_t)G * kPhiloxM1) >> 32) ^ keys.rk0[0];
 }
 
+// Children that the next generation finds in L2 (StreamPlan::back) are stored
+// as any other data (four words 46.2 against 47.9 us), others as data not read
+// again soon.
+template <bool KEEP, class T>
+__device__ __forceinline__ void flat_store(T *at, T value) {
+  if constexpr (KEEP) *at = value;
+  else __stcs(at, value);
+}
+
 // Advances `group` (<= kFlatGroup) islands from isl0 on (fewer at the end of the
 // grid) from the parent planes to the child planes.  K: surface words (0: no surface).  NN:
 // island size when known (32), else 0.  T2: the tournament size is exactly 2.
-// FLT: binary32 fitness.  bulk: the planes allow 16-byte bulk copies.
+// FLT: binary32 fitness.  planned: `move` is the lane's
+// migration move (0: none).  bulk: the planes allow 16-byte bulk copies.
 // Returns false (on every lane) when the copy did not arrive in time.
-template <int K, bool T2, int NN, bool FLT, class Keys>
+template <int K, bool T2, int NN, bool FLT, bool KEEP = false, class Keys>
 __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
                                            const FlatDeposit<K> &dep, bool migrate, bool bulk,
                                            uint32_t isl0, uint32_t group, uint32_t G,
+                                           bool planned, uint32_t move,
                                            const uint32_t *__restrict__ tin,
                                            const uint64_t *__restrict__ sin,
                                            uint32_t *__restrict__ tout,
@@ -205,7 +200,16 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
 #pragma unroll
   for (int w = 0; w < KS; ++w) is[w] = 0;
   bool arrive = false;
-  if (migrate) {
+  if (planned) {
+    if (move & kMoveLands) {
+      const size_t a = (size_t)neighbour(p, isl0 + (lane >> 2), lane & 3u) * n + (move >> 6 & 63u);
+      it = __ldg(tin + a);
+      if constexpr (K > 0) {
+#pragma unroll
+        for (int w = 0; w < KS; ++w) is[w] = __ldg(sin + a * K + w);
+      }
+    }
+  } else if (migrate) {
     if (lane < cnt) {
       const Words4 v = philox_keys(keys, kSlotImmigrant, isl0 + lane, G, kPurposeMigration);
       st.plan[lane] = uindex_nn<NN>(v.x, n) | (uindex_nn<NN>(v.y, n) << 8) |
@@ -265,8 +269,9 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
     st.phase ^= 1u;
   }
   __syncwarp();
-  if (migrate) {
+  if (planned || migrate) {
     const uint32_t d = lane & 3u;
+    uint32_t at = (move & kMoveLands) ? (lane >> 2) * n + (move & 63u) : kNoArrival;
     const uint32_t bits = (__ballot_sync(kFull, arrive) >> (lane & 28u)) & 0xFu;
     if (arrive) {
       const uint32_t pl = st.plan[lane >> 2];
@@ -275,13 +280,13 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
 #pragma unroll
       for (uint32_t e = 1; e < 4; ++e)
         if (e > d && (bits >> e & 1u) && ((pl >> (8u * e)) & 0xFFu) == sl) last = false;
-      if (last) {
-        const uint32_t a = (lane >> 2) * n + sl;
-        st.trait[a] = it;
-        if constexpr (K > 0) {
+      if (last) at = (lane >> 2) * n + sl;
+    }
+    if (at != kNoArrival) {
+      st.trait[at] = it;
+      if constexpr (K > 0) {
 #pragma unroll
-          for (int w2 = 0; w2 < KS; ++w2) st.surf[a * K + w2] = is[w2];
-        }
+        for (int w2 = 0; w2 < KS; ++w2) st.surf[at * K + w2] = is[w2];
       }
     }
     __syncwarp();
@@ -374,17 +379,17 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
 #pragma unroll
     for (uint32_t u = 0; u < U; ++u) {
       if (c0 + 32u * u + lane < total) {
-        __stcs(to + 32u * u, ct[u]);
-        if constexpr (K == 1) __stcs(so + 32u * u, cs[u][0]);
+        flat_store<KEEP>(to + 32u * u, ct[u]);
+        if constexpr (K == 1) flat_store<KEEP>(so + 32u * u, cs[u][0]);
         if constexpr (K == 2 || K == 4) {
           uint64_t *const o = so + 32u * u * K;
           if (bulk) {  // 16-byte aligned planes
 #pragma unroll
             for (int q = 0; q < KS; q += 2)
-              __stcs((ulonglong2 *)(o + q), make_ulonglong2(cs[u][q], cs[u][q + 1]));
+              flat_store<KEEP>((ulonglong2 *)(o + q), make_ulonglong2(cs[u][q], cs[u][q + 1]));
           } else {
 #pragma unroll
-            for (int q = 0; q < KS; ++q) __stcs(o + q, cs[u][q]);
+            for (int q = 0; q < KS; ++q) flat_store<KEEP>(o + q, cs[u][q]);
           }
         }
       }

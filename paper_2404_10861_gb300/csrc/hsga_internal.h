@@ -11,13 +11,15 @@
 namespace hsga {
 
 constexpr int kStagedThreads = 256;     // staged streamed kernel (n = 32) block: 8 warps
-// 24 resident warps per SM (<= 80 registers), each with one group staged:
-// us per generation at 16.8M agents / on 256x256 / 128x128 islands of 32, 24
-// warps and 1 stage 72.1 / 11.9 / 4.9, 24 and 2 72.6 / 12.2 / 5.1, 16 and 2
-// 72.4 / 11.9 / 6.3, 16 and 3 74.2 / 12.1 / 6.3, 32 and 1 72.1 / 11.2 / 5.6
-// (but tournament 5 on 500x500 69.7 against 65.1: 64 registers spill).
-constexpr int kStagedBlocksPerSM = 3;
-constexpr uint32_t kStagedStages = 1;   // groups in flight per warp
+// 16 resident warps per SM (<= 128 registers), a group of 8 islands each, all
+// of its children in flight: us per generation at 16.8M agents / tournament 5
+// on 500x500 islands / on 256x256 islands, 16 warps 67.3 / 60.8 / 11.2; 24 warps
+// with the children of 4 islands in flight 68.6 / 62.9 / 11.0, of 8 (80
+// registers spill) 68.2 / 69.2 / 10.7; 32 with 4 72.7 / 72.5 / 11.1; 16 with
+// groups of 16 in two halves 70.5 / 61.3 / 10.8.  Groups of 6 on 24 warps, before:
+// 71.7 / 65.7 / 11.9.
+constexpr int kStagedBlocksPerSM = 2;
+constexpr uint32_t kStagedStages = 2;   // most groups in flight per warp
 constexpr int kResidentThreads = 128;   // free-running, float and wide kernels: 4 warps
 constexpr uint64_t kWaitNs = 1000000000ull; // bounded device wait: 1 s
 
@@ -35,30 +37,53 @@ struct ResidentPlan {
   bool one_block = false;  // a plain launch of one block that holds the whole grid
 };
 
+// Migration moves of a streamed run, worked out ahead of their generation
+// (hsga_moves.cuh).  now: this generation's, [island][direction], or NULL: the
+// launch derives them.  next: written, from leave_next, for the next
+// generation; leave_after: written for the one after it; or NULL.
+struct Moves {
+  const uint16_t *now = nullptr;
+  uint16_t *next = nullptr;
+  const uint8_t *leave_next = nullptr;
+  uint8_t *leave_after = nullptr;
+};
+
 // err: the grid's device error word (bounded waits report timeouts there).
 // plan: from stream_plan for the same parameters.
 struct StreamPlan {
   int blocks = 0;   // resident blocks of the whole device
   size_t smem = 0;  // dynamic shared memory per block
   int group = 0;    // islands per warp visit
+  bool moves_ahead = false;  // launches of a run plan the migration of later ones
+  bool back = false;         // odd generations walk the islands from last to first
+  bool large = false;        // the flat kernel's instance for large grids
 };
 bool stream_plan(const RunParams &p, StreamPlan *out);
+
+// Whether parents and children do not fit in L2 together.  Then every other
+// generation walks the islands from last to first: it begins with the parents
+// that the one before wrote last and finds part of them in L2 (256x512 islands
+// of 32 with four surface words: 46.2 us per generation, 54.9 without; grids
+// that fit lose 1%).
+bool planes_exceed_l2(const RunParams &p);
 cudaError_t launch_step_streamed(const RunParams &p, const StreamPlan &plan, uint32_t G,
-                                 bool do_mig, const uint32_t *tin, const uint64_t *sin,
-                                 uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream);
+                                 bool do_mig, const Moves &mv, const uint32_t *tin,
+                                 const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
+                                 cudaStream_t stream);
 
 // The same generation for 32-agent islands with the parents staged in shared
 // memory by bulk asynchronous copies (hsga_staged.cu); waits report
 // timeouts in err.
-cudaError_t launch_step_staged(const RunParams &p, uint32_t G, bool do_mig, const uint32_t *tin,
-                               const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
-                               cudaStream_t stream);
+bool staged_stream_plan(const RunParams &p, StreamPlan *out);
+cudaError_t launch_step_staged(const RunParams &p, const StreamPlan &plan, uint32_t G, bool do_mig,
+                               const Moves &mv, const uint32_t *tin, const uint64_t *sin,
+                               uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream);
 
 // The same generation for any island size, fitness model and surface width
 // (hsga_flat.cu).
 bool flat_stream_plan(const RunParams &p, StreamPlan *out);
 cudaError_t launch_step_flat(const RunParams &p, const StreamPlan &plan, uint32_t G, bool do_mig,
-                             const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
+                             const Moves &mv, const uint32_t *tin, const uint64_t *sin, uint32_t *tout,
                              uint64_t *sout, int *err, cudaStream_t stream);
 
 // Chooses the resident tiles.  Returns false when the grid does not fit in

@@ -122,16 +122,17 @@ __device__ __forceinline__ void land(uint32_t slot, uint32_t src, uint32_t it, u
   }
 }
 
-// --------------------------------------------- island groups (streaming) ---
-// A warp advances groups of kGroup consecutive islands.  The group's
-// migration draws take one warp-wide Philox evaluation: lane 5p+r (r < 4)
-// evaluates the emigrant block of the neighbour in direction r of island
-// isl0+p and gathers that emigrant's genome from the parent planes when it is
-// aimed at isl0+p; lane 5p+4 evaluates the placement block of isl0+p and
-// turns it into a landing plan: byte 3-d holds the slot where the direction-d
-// immigrant lands, or 0xFF when it does not arrive.  Later arrivals overwrite
-// earlier ones, and the reversed byte order makes the lowest matching byte
-// the latest direction, so slots shared by several arrivals need no pass.
+// ---------------------------------------------------- island groups ---
+// Up to kGroup consecutive islands by one warp, one at a time (the islands left
+// over when the staged kernel's groups are cut).  Their migration draws take one
+// warp-wide Philox evaluation: lane 5p+r (r < 4) evaluates the emigrant block of
+// the neighbour in direction r of island isl0+p and gathers that emigrant's
+// genome from the parent planes when it is aimed at isl0+p; lane 5p+4 evaluates
+// the placement block of isl0+p and turns it into a landing plan: byte 3-d
+// holds the slot where the direction-d immigrant lands, or 0xFF when it does
+// not arrive.  Later arrivals overwrite earlier ones, and the reversed byte
+// order makes the lowest matching byte the latest direction, so slots shared
+// by several arrivals need no pass.
 constexpr uint32_t kGroup = 6;  // 6 islands x 5 blocks = 30 of 32 lanes
 
 struct GroupMigration {
@@ -238,7 +239,7 @@ __device__ __forceinline__ void store_island(const RunParams &p, uint32_t isl,
   }
 }
 
-// The last, partial group: islands one at a time.
+// Up to kGroup islands from isl0 on, one at a time.
 template <int AP, bool TRACKED, bool T2, bool RK = true>
 __device__ __noinline__ void partial_group(const RunParams &p, const Deposit &dep, uint32_t G,
                                            bool do_mig, uint32_t isl0,
@@ -248,7 +249,7 @@ __device__ __noinline__ void partial_group(const RunParams &p, const Deposit &de
                                            uint64_t *__restrict__ sout) {
   GroupMigration gm;
   if (do_mig) group_migration<TRACKED, RK>(p, isl0, G, tin, sin, gm);
-  for (uint32_t k = 0; isl0 + k < p.islands; ++k) {
+  for (uint32_t k = 0; k < kGroup && isl0 + k < p.islands; ++k) {
     uint32_t pt[AP], ct[AP];
     uint64_t ps[AP], cs[AP];
     load_island<AP, TRACKED>(p, isl0 + k, tin, sin, pt, ps);

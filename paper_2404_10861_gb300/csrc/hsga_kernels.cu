@@ -20,16 +20,26 @@ namespace hsga {
 // kernel of their own, which plans its launches itself.
 static bool staged_shape(const RunParams &p) { return p.n == 32 && p.words == 1 && !p.flt; }
 
+bool planes_exceed_l2(const RunParams &p) {
+  int dev = 0, l2 = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+    return false;
+  const uint64_t genome = 4u + 8u * (p.policy == HSGA_NONE ? 0u : p.words);
+  return 2u * genome * p.n * p.islands > (uint64_t)l2;
+}
+
 bool stream_plan(const RunParams &p, StreamPlan *out) {
-  return staged_shape(p) || flat_stream_plan(p, out);
+  return staged_shape(p) ? staged_stream_plan(p, out) : flat_stream_plan(p, out);
 }
 
 cudaError_t launch_step_streamed(const RunParams &p, const StreamPlan &plan, uint32_t G,
-                                 bool do_mig, const uint32_t *tin, const uint64_t *sin,
-                                 uint32_t *tout, uint64_t *sout, int *err, cudaStream_t stream) {
+                                 bool do_mig, const Moves &mv, const uint32_t *tin,
+                                 const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
+                                 cudaStream_t stream) {
   if (staged_shape(p))
-    return launch_step_staged(p, G, do_mig, tin, sin, tout, sout, err, stream);
-  return launch_step_flat(p, plan, G, do_mig, tin, sin, tout, sout, err, stream);
+    return launch_step_staged(p, plan, G, do_mig, mv, tin, sin, tout, sout, err, stream);
+  return launch_step_flat(p, plan, G, do_mig, mv, tin, sin, tout, sout, err, stream);
 }
 
 // --------------------------------------------------- explicit a1 + a2 ---

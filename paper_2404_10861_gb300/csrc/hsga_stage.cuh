@@ -2,26 +2,28 @@
 // asynchronous copies, shared by the single-run staged generation kernel
 // (hsga_staged.cu).
 //
-// A warp owns a ring of kStagedStages stages; a stage holds one group of six
-// 32-agent islands: 768 bytes of traits, then 1,536 bytes of surfaces, each
-// contiguous in the island-major planes, copied by one lane with
-// cp.async.bulk and completing on the stage's mbarrier.  The helpers below
-// are the barrier and copy primitives, the landing of a group's immigrants
-// into a stage, and one child's replication from a stage.
+// A warp owns a ring of up to kStagedStages stages; a stage holds one group of
+// eight 32-agent islands: 1,024 bytes of traits, then 2,048 bytes of surfaces,
+// each contiguous in the island-major planes, copied by one lane with
+// cp.async.bulk and completing on the stage's mbarrier.  The helpers below are
+// the barrier and copy primitives, a group's immigrants, and its replication
+// from a stage.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include "hsga_internal.h"
 #include "hsga_island.cuh"
+#include "hsga_moves.cuh"
 
 namespace hsga {
 
-
 constexpr uint32_t kStagedWarps = kStagedThreads / 32;
-constexpr uint32_t kStageAgents = kGroup * 32;
-constexpr uint32_t kTraitBytes = kStageAgents * 4;  // 768
-constexpr uint32_t kSurfBytes = kStageAgents * 8;   // 1536
+constexpr uint32_t kStageGroup = 8;  // islands per stage
+constexpr uint32_t kStageWords = kStageGroup / 8;
+constexpr uint32_t kStageAgents = kStageGroup * 32;
+constexpr uint32_t kTraitBytes = kStageAgents * 4;  // 1,024
+constexpr uint32_t kSurfBytes = kStageAgents * 8;   // 2,048
 constexpr uint32_t kMaxPolls = 1u << 24;
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
@@ -89,27 +91,74 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   return false;
 }
 
-// a2 for a staged group: lane 5p+r (r < 4) holds the immigrant of island p
-// from direction r when it arrives; the landing plan of island p (lane 5p+4,
-// byte 3-d: slot of direction d, 0xFF: none) says where.  The lane stores it
-// unless a later direction lands on the same slot.
+// A lane's immigrants to a staged group, lane 4i + d of word a the one of
+// island 8a + i from direction d: the agent of the group that it overwrites
+// (none: kNoArrival) and its genome.
+constexpr uint32_t kNoArrival = 0xFFFFFFFFu;
+struct Arrivals {
+  uint32_t at[kStageWords], it[kStageWords];
+  uint64_t is[kStageWords];
+};
+
+// a1 and a2 derived here, for all of the group's islands.
 template <bool TRACKED>
-__device__ __forceinline__ void land_staged(const GroupMigration &gm, uint32_t lane,
-                                            uint32_t *tr, uint64_t *sr) {
-  const uint32_t pi = lane / 5u, role = lane - 5u * pi;
-  const uint32_t plan = __shfl_sync(kFull, gm.plan, min(5u * pi + 4u, 31u));
-  if (lane < 5u * kGroup && role < 4u) {
-    const uint32_t sh = 8u * (3u - role);
-    const uint32_t slot = (plan >> sh) & 0xFFu;
-    // bytes of later directions (below byte 3-role) kept, the rest all ones
-    const uint32_t later = plan | ~((1u << sh) - 1u);
-    const uint32_t x = later ^ (slot * 0x01010101u);
-    const bool overwritten = ((x - 0x01010101u) & ~x & 0x80808080u) != 0u;
-    if (slot != 0xFFu && !overwritten) {
-      tr[pi * 32u + slot] = gm.it;
-      if constexpr (TRACKED) sr[pi * 32u + slot] = gm.is;
+__device__ __forceinline__ void derive_arrivals(const RunParams &p, uint32_t isl0, uint32_t G,
+                                                const uint32_t *__restrict__ tin,
+                                                const uint64_t *__restrict__ sin, Arrivals &r) {
+  const uint32_t lane = threadIdx.x & 31u, d = lane & 3u;
+  const Words4 v = philox_rk(p, kSlotImmigrant, isl0 + min(lane, kStageGroup - 1u), G,
+                             kPurposeMigration);
+  const uint32_t plan =
+      v.x >> 27 | (v.y >> 27) << 8 | (v.z >> 27) << 16 | (v.w >> 27) << 24;
+#pragma unroll
+  for (uint32_t a = 0; a < kStageWords; ++a) {
+    const uint32_t i = 8u * a + (lane >> 2);
+    const uint32_t src = neighbour(p, isl0 + i, d);
+    const Words4 m = philox_rk(p, kSlotEmigrant, src, G, kPurposeMigration);
+    const bool arrive = (m.y >> 30) == (d ^ 2u);
+    r.at[a] = kNoArrival;
+    if (arrive) {
+      const uint32_t x = src * 32u + (m.x >> 27);
+      r.it[a] = __ldg(tin + x);
+      if constexpr (TRACKED) r.is[a] = __ldg(sin + x);
+    }
+    const uint32_t to = __shfl_sync(kFull, plan, i);
+    const uint32_t bits = (__ballot_sync(kFull, arrive) >> (lane & 28u)) & 0xFu;
+    const uint32_t slot = (to >> (8u * d)) & 0xFFu;
+    bool lands = arrive;
+#pragma unroll
+    for (uint32_t e = 1; e < 4; ++e)  // the latest of N, E, S, W wins a shared slot
+      lands = lands && !(e > d && (bits >> e & 1u) && ((to >> (8u * e)) & 0xFFu) == slot);
+    if (lands) r.at[a] = 32u * i + slot;
+  }
+}
+
+// The same from the lane's planned moves.
+template <bool TRACKED>
+__device__ __forceinline__ void planned_arrivals(const RunParams &p,
+                                                 const uint32_t (&move)[kStageWords],
+                                                 uint32_t isl0, const uint32_t *__restrict__ tin,
+                                                 const uint64_t *__restrict__ sin, Arrivals &r) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (uint32_t a = 0; a < kStageWords; ++a) {
+    const uint32_t i = 8u * a + (lane >> 2);
+    r.at[a] = kNoArrival;
+    if (move[a] & kMoveLands) {
+      const uint32_t x = neighbour(p, isl0 + i, lane & 3u) * 32u + (move[a] >> 6 & 31u);
+      r.at[a] = 32u * i + (move[a] & 31u);
+      r.it[a] = __ldg(tin + x);
+      if constexpr (TRACKED) r.is[a] = __ldg(sin + x);
     }
   }
+}
+
+// The lane's planned moves of a group.
+__device__ __forceinline__ void load_moves(const Moves &mv, uint32_t isl0,
+                                           uint32_t (&move)[kStageWords]) {
+#pragma unroll
+  for (uint32_t a = 0; a < kStageWords; ++a)
+    move[a] = mv.now[(size_t)isl0 * 4u + 32u * a + (threadIdx.x & 31u)];
 }
 
 // a3-a6 of child `lane` of every island of a staged group (parents of island
@@ -118,22 +167,22 @@ __device__ __forceinline__ void land_staged(const GroupMigration &gm, uint32_t l
 // compiler, which would otherwise finish one island before it reads the next.
 template <bool TRACKED, bool T2, bool TWO, bool DEL, class More>
 __device__ __forceinline__ void replicate_group(const RunParams &p, const Deposit &dep,
-                                                const Words4 (&w)[kGroup], const uint32_t *tr,
+                                                const Words4 (&w)[kStageGroup], const uint32_t *tr,
                                                 const uint64_t *sr, uint32_t *to, uint64_t *so,
                                                 const More &more) {
-  uint32_t best[kGroup], fbest[kGroup];
-  uint64_t cs[kGroup];
+  uint32_t best[kStageGroup], fbest[kStageGroup];
+  uint64_t cs[kStageGroup];
 #pragma unroll
-  for (uint32_t i = 0; i < kGroup; ++i) {
+  for (uint32_t i = 0; i < kStageGroup; ++i) {
     best[i] = w[i].x >> 27;
     fbest[i] = tr[32u * i + best[i]];
   }
   if (T2 || p.tournament >= 2) {
-    uint32_t fc[kGroup];
+    uint32_t fc[kStageGroup];
 #pragma unroll
-    for (uint32_t i = 0; i < kGroup; ++i) fc[i] = tr[32u * i + (w[i].y >> 27)];
+    for (uint32_t i = 0; i < kStageGroup; ++i) fc[i] = tr[32u * i + (w[i].y >> 27)];
 #pragma unroll
-    for (uint32_t i = 0; i < kGroup; ++i) {
+    for (uint32_t i = 0; i < kStageGroup; ++i) {
       best[i] = fc[i] > fbest[i] ? w[i].y >> 27 : best[i];
       fbest[i] = max(fc[i], fbest[i]);
     }
@@ -141,7 +190,7 @@ __device__ __forceinline__ void replicate_group(const RunParams &p, const Deposi
   if constexpr (!T2) {
     for (uint32_t c0 = 2; c0 < p.tournament; c0 += 4) {
 #pragma unroll
-      for (uint32_t i = 0; i < kGroup; ++i) {
+      for (uint32_t i = 0; i < kStageGroup; ++i) {
         const Words4 e = more(i, (c0 - 2) / 4);
         const uint32_t ew[4] = {e.x >> 27, e.y >> 27, e.z >> 27, e.w >> 27};
         uint32_t fc[4];
@@ -158,18 +207,17 @@ __device__ __forceinline__ void replicate_group(const RunParams &p, const Deposi
   }
   if constexpr (TRACKED) {
 #pragma unroll
-    for (uint32_t i = 0; i < kGroup; ++i) cs[i] = sr[32u * i + best[i]];
+    for (uint32_t i = 0; i < kStageGroup; ++i) cs[i] = sr[32u * i + best[i]];
   }
 #pragma unroll
-  for (uint32_t i = 0; i < kGroup; ++i) {
+  for (uint32_t i = 0; i < kStageGroup; ++i) {
     __stcs(to + 32u * i, mutate<DEL>(p, fbest[i], w[i].z));
     if constexpr (TRACKED) __stcs(so + 32u * i, deposit_into<TWO>(dep, cs[i], w[i].w));
   }
 }
 
 constexpr uint32_t kStageBytes = kTraitBytes + kSurfBytes;  // 2304 per group
-constexpr uint32_t kStages = kStagedStages;
-constexpr size_t kRingBytes = (size_t)kStagedWarps * kStages * kStageBytes;
+constexpr size_t kRingBytes = (size_t)kStagedWarps * kStagedStages * kStageBytes;
 
 // Shared memory requested per block: the ring, padded so that one block
 // more than kStagedBlocksPerSM does not fit on an SM.  Otherwise the next

@@ -4,29 +4,30 @@
 // One launch advances one synchronous generation of the whole grid (steps
 // a1-a6 of the paper's cycle, section "Asynchronous Island-model Genetic
 // Algorithm": migration, then evaluation, tournament selection, mutation and
-// the surface update).  A persistent grid of warps walks the islands in
-// groups of six (the group of the island-group helpers: six islands' five
-// migration blocks fill 30 lanes of one warp-wide Philox evaluation).  Each
-// warp stages a group's parents in shared memory; one lane copies them in
-// with cp.async.bulk (768 bytes of traits and 1,536 bytes of surfaces, both
+// the surface update).  A persistent grid of warps walks the islands in groups
+// of eight (four directions of eight islands fill a warp's lanes).  Each warp
+// stages a group's parents in shared memory; one lane copies them in with
+// cp.async.bulk (1,024 bytes of traits and 2,048 bytes of surfaces, both
 // contiguous in the island-major planes), completing on the stage's mbarrier,
 // while the group's replication draws are evaluated.  The bytes in flight
 // cost no registers, and the tournament reads the parents from shared memory:
 // two 4-byte loads for the candidates' fitness and one 8-byte load for the
-// winner's surface per child.  Immigrants are gathered from the neighbours'
-// parent planes one group ahead and land with one shared-memory store each
-// (the latest of N, E, S, W wins a shared slot).  Children go straight to the
-// child planes with streaming stores.
+// winner's surface per child (warp shuffles of the fitness in their place:
+// 70.4 against 65.6 us with a tournament of 5).  Immigrants are gathered from
+// the neighbours' parent planes one group ahead and land with one shared-memory
+// store each.  Children go straight to the child planes with streaming stores.
 //
 // Of the replication blocks' first three rounds only two products depend on
-// the island, one of them the same on every lane (lane_head).
+// the island, one of them the same on every lane (lane_head).  Where warps take
+// several groups, a launch works out the migration of the two generations after
+// it between its groups and finds its own worked out (hsga_moves.cuh).
 //
-// What bounds it, per generation at 16.8M agents (copies of the kernel that
-// skip work): without loads and stores 69 us, without migration 64-71, both
-// together 47, everything 72.1; 92 warp instructions per island, 21 of them
-// migration, at 0.56 instructions per cycle and scheduler.  Before: 75.2 us
-// (tournament 5 on 500x500 islands 71.8, now 64.5-65.1), each island's reads
-// behind the stores of the one before it and the gather's latency exposed.
+// What bounds it, per generation at 16.8M agents: 66.0 us, of which 59.4 are
+// its 24 bytes per agent at the measured copy bandwidth; half of the issue
+// slots are taken.  Groups of six, each deriving its own migration: 71.7, and 69
+// without any load or store; before the reads of a group came ahead of its
+// stores: 75.2.  Tournament 5 on 500x500 islands 60.8 (65.7, 71.8), untracked
+// 16.8M 53-55 (60.0), 256x256 islands 11.2 (11.9); these are bound by issue.
 //
 // Consecutive generations overlap at the launch boundary (programmatic
 // dependent launch): a launch lets the next one be scheduled as soon as it
@@ -44,38 +45,49 @@
 namespace hsga {
 namespace {
 
+struct StagedLaunch {
+  uint32_t G;
+  uint32_t back;    // walk the groups from the last to the first
+  uint32_t stages;  // groups staged per warp, 1 .. kStagedStages
+  Moves mv;
+};
+
 template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG>
 __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
-    step_staged_kernel(RunParams p, Deposit dep, uint32_t G, const uint32_t *__restrict__ tin,
+    step_staged_kernel(RunParams p, Deposit dep, StagedLaunch l, const uint32_t *__restrict__ tin,
                        const uint64_t *__restrict__ sin, uint32_t *__restrict__ tout,
                        uint64_t *__restrict__ sout, int *__restrict__ err) {
+  const uint32_t G = l.G, stages = l.stages;
+  const Moves &mv = l.mv;
   extern __shared__ __align__(128) unsigned char s_ring[];  // the ring (kRingBytes), padded
-  __shared__ __align__(8) uint64_t s_bar[kStagedWarps][kStages];
+  __shared__ __align__(8) uint64_t s_bar[kStagedWarps][kStagedStages];
   const uint32_t lane = threadIdx.x & 31u, wib = __shfl_sync(kFull, threadIdx.x >> 5, 0);
   const uint32_t warp = blockIdx.x * kStagedWarps + wib;
   const uint32_t nwarps = gridDim.x * kStagedWarps;
-  const uint32_t nfull = p.islands / kGroup;
-  unsigned char *ring = s_ring + (size_t)wib * kStages * kStageBytes;
+  const uint32_t nfull = p.islands / kStageGroup;
+  unsigned char *ring = s_ring + (size_t)wib * kStagedStages * kStageBytes;
   uint64_t *bar = s_bar[wib];
   constexpr uint32_t kTx = kTraitBytes + (TRACKED ? kSurfBytes : 0u);
 
-  // stage st holds a group's traits (768 B) then its surfaces (1,536 B)
-  auto issue = [&](uint32_t grp, uint32_t st) {  // one lane
+  // stage st holds a group's traits (1,024 B) then its surfaces (2,048 B)
+  auto issue = [&](uint32_t isl0, uint32_t st) {  // one lane
     unsigned char *dst = ring + st * kStageBytes;
     proxy_fence();
     mbar_expect_tx(&bar[st], kTx);
-    bulk_load(dst, tin + (size_t)grp * kStageAgents, kTraitBytes, &bar[st]);
+    bulk_load(dst, tin + (size_t)isl0 * 32u, kTraitBytes, &bar[st]);
     if constexpr (TRACKED)
-      bulk_load(dst + kTraitBytes, sin + (size_t)grp * kStageAgents, kSurfBytes, &bar[st]);
+      bulk_load(dst + kTraitBytes, sin + (size_t)isl0 * 32u, kSurfBytes, &bar[st]);
   };
 
   // the next launch may be scheduled now; it waits below for this one
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (lane == 0) {
 #pragma unroll
-    for (uint32_t st = 0; st < kStages; ++st) mbar_init(&bar[st], 1);
+    for (uint32_t st = 0; st < stages; ++st) mbar_init(&bar[st], 1);
     mbar_init_fence();
   }
+  const uint32_t first = (l.back ? nfull - 1u - warp : warp) * kStageGroup;
+  const uint32_t skip = l.back ? 0u - nwarps * kStageGroup : nwarps * kStageGroup;
   const LaneHead head = lane_head(p, lane, G, kPurposeReplicate);
   [[maybe_unused]] LaneHead head2;  // candidates 2-5
   if constexpr (!T2) head2 = lane_head(p, lane, G, kPurposeReplicate + 1u);
@@ -84,51 +96,74 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (lane == 0) {
 #pragma unroll
-    for (uint32_t st = 0; st < kStages; ++st)
-      if (warp + st * nwarps < nfull) issue(warp + st * nwarps, st);
+    for (uint32_t st = 0; st < stages; ++st)
+      if (warp + st * nwarps < nfull) issue(first + st * skip, st);
   }
   __syncwarp();
 
   // The immigrants of a group are gathered while the group before it is
   // replicated: the gather's latency, with nothing to hide it, made up a
   // third of a generation on L2-resident grids.
-  GroupMigration next_gm{};
+  Arrivals next;
+  uint32_t move[kStageWords] = {};  // planned, of the group after the next
   if constexpr (MIG) {
-    if (warp < nfull) group_migration<TRACKED, true, 32>(p, warp * kGroup, G, tin, sin, next_gm);
-  }
-  uint32_t st = 0, phase = 0;  // ring position of the k-th group and its phase parity
-  for (uint32_t grp = warp; grp < nfull; grp += nwarps) {
-    const uint32_t isl0 = grp * kGroup;
-    const GroupMigration gm = next_gm;
-    if constexpr (MIG) {
-      if (grp + nwarps < nfull)
-        group_migration<TRACKED, true, 32>(p, isl0 + nwarps * kGroup, G, tin, sin, next_gm);
+    if (warp < nfull) {
+      const uint32_t isl0 = first;
+      if (mv.now) {
+        load_moves(mv, isl0, move);
+        planned_arrivals<TRACKED>(p, move, isl0, tin, sin, next);
+        if (warp + nwarps < nfull) load_moves(mv, isl0 + skip, move);
+      } else {
+        derive_arrivals<TRACKED>(p, isl0, G, tin, sin, next);
+      }
     }
-    Words4 w[kGroup];
+  }
+  Planner planner(p, mv, warp, nwarps);
+  uint32_t st = 0, phase = 0;  // ring position of the k-th group and its phase parity
+  uint32_t isl0 = first;
+  for (uint32_t grp = warp; grp < nfull; grp += nwarps, isl0 += skip) {
+    const Arrivals in = next;
+    if constexpr (MIG) {
+      if (grp + nwarps < nfull) {
+        if (mv.now) {
+          planned_arrivals<TRACKED>(p, move, isl0 + skip, tin, sin, next);
+          if (grp + 2u * nwarps < nfull) load_moves(mv, isl0 + 2u * skip, move);
+        } else {
+          derive_arrivals<TRACKED>(p, isl0 + skip, G, tin, sin, next);
+        }
+      }
+    }
+    Words4 w[kStageGroup];
 #pragma unroll
-    for (uint32_t i = 0; i < kGroup; ++i) w[i] = lane_tail(p, head, isl0 + i);
+    for (uint32_t i = 0; i < kStageGroup; ++i) w[i] = lane_tail(p, head, isl0 + i);
     if (!__all_sync(kFull, mbar_wait(&bar[st], phase))) {
       // give up: record the timeout, wait (bounded) for this warp's copies
       // still in flight (the groups issued into the ring from this one on),
-      // leave
+      // leave (once the moves that later launches read are written)
       if (lane == 0) {
         atomicCAS(err, 0, kDevErrWaitTimeout);
         uint32_t s2 = st, ph2 = phase;
-        for (uint32_t j = 0; j < kStages && grp + j * nwarps < nfull; ++j) {
+        for (uint32_t j = 0; j < stages && grp + j * nwarps < nfull; ++j) {
           mbar_wait(&bar[s2], ph2);
-          if (++s2 == kStages) {
+          if (++s2 == stages) {
             s2 = 0;
             ph2 ^= 1u;
           }
         }
       }
       __syncwarp();
-      return;
+      break;
     }
     uint32_t *tr = (uint32_t *)(ring + st * kStageBytes);
     uint64_t *sr = (uint64_t *)(ring + st * kStageBytes + kTraitBytes);
     if constexpr (MIG) {
-      land_staged<TRACKED>(gm, lane, tr, sr);
+#pragma unroll
+      for (uint32_t a = 0; a < kStageWords; ++a) {
+        if (in.at[a] != kNoArrival) {
+          tr[in.at[a]] = in.it[a];
+          if constexpr (TRACKED) sr[in.at[a]] = in.is[a];
+        }
+      }
       __syncwarp();
     }
     uint32_t *to = tout + (size_t)isl0 * 32u + lane;
@@ -139,15 +174,18 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
                         : philox_rk(p, lane, isl0 + i, G, kPurposeReplicate + 1 + q);
         });
     __syncwarp();  // every lane is done with this stage before it is refilled
-    if (lane == 0 && grp + kStages * nwarps < nfull) issue(grp + kStages * nwarps, st);
-    if (++st == kStages) {
+    if (lane == 0 && grp + stages * nwarps < nfull) issue(isl0 + stages * skip, st);
+    planner.visit<32>(p, p, mv, G, kStageGroup);
+    if (++st == stages) {
       st = 0;
       phase ^= 1u;
     }
   }
-  // the last, partial group (fewer than six islands) on the register path
-  if (p.islands % kGroup != 0u && warp == nfull % nwarps)
-    partial_group<1, TRACKED, T2>(p, dep, G, MIG, nfull * kGroup, tin, sin, tout, sout);
+  planner.rest<32>(p, p, mv, G);
+  // the last islands, too few for a group, on the register path
+  if (warp == nfull % nwarps)
+    for (uint32_t i = nfull * kStageGroup; i < p.islands; i += kGroup)
+      partial_group<1, TRACKED, T2>(p, dep, G, MIG, i, tin, sin, tout, sout);
 }
 
 template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG>
@@ -169,10 +207,10 @@ int staged_blocks() {
 }
 
 template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG>
-void launch_staged_t(const RunParams &p, const Deposit &dep, uint32_t G, const uint32_t *tin,
-                     const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
-                     cudaStream_t stream) {
-  const uint32_t groups = (p.islands + kGroup - 1) / kGroup;
+void launch_staged_t(const RunParams &p, const Deposit &dep, const StagedLaunch &l,
+                     const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
+                     int *err, cudaStream_t stream) {
+  const uint32_t groups = (p.islands + kStageGroup - 1) / kStageGroup;
   const uint32_t need = (groups + kStagedWarps - 1) / kStagedWarps;
   int b = staged_blocks<TRACKED, T2, TWO, DEL, MIG>();
   if ((uint32_t)b > need) b = (int)need;
@@ -186,20 +224,20 @@ void launch_staged_t(const RunParams &p, const Deposit &dep, uint32_t G, const u
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, step_staged_kernel<TRACKED, T2, TWO, DEL, MIG>, p, dep, G, tin, sin,
+  cudaLaunchKernelEx(&cfg, step_staged_kernel<TRACKED, T2, TWO, DEL, MIG>, p, dep, l, tin, sin,
                      tout, sout, err);
 }
 
 template <bool TRACKED, bool T2>
-void launch_staged_m(const RunParams &p, const Deposit &dep, uint32_t G, bool mig,
+void launch_staged_m(const RunParams &p, const Deposit &dep, const StagedLaunch &l, bool mig,
                      const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
                      int *err, cudaStream_t stream) {
-#define HSGA_STAGED(TWO_, DEL_)                                                            \
-  if (mig)                                                                                 \
-    launch_staged_t<TRACKED, T2, TWO_, DEL_, true>(p, dep, G, tin, sin, tout, sout, err,   \
-                                                   stream);                                \
-  else                                                                                     \
-    launch_staged_t<TRACKED, T2, TWO_, DEL_, false>(p, dep, G, tin, sin, tout, sout, err,  \
+#define HSGA_STAGED(TWO_, DEL_)                                                               \
+  if (mig)                                                                                    \
+    launch_staged_t<TRACKED, T2, TWO_, DEL_, true>(p, dep, l, tin, sin, tout, sout, err,      \
+                                                   stream);                                   \
+  else                                                                                        \
+    launch_staged_t<TRACKED, T2, TWO_, DEL_, false>(p, dep, l, tin, sin, tout, sout, err,     \
                                                     stream);
   if (TRACKED && dep.two) {
     HSGA_STAGED(true, true)
@@ -213,19 +251,36 @@ void launch_staged_m(const RunParams &p, const Deposit &dep, uint32_t G, bool mi
 
 }  // namespace
 
-cudaError_t launch_step_staged(const RunParams &p, uint32_t G, bool do_mig, const uint32_t *tin,
+// Launches plan ahead where a warp takes at least two groups: with one, planning
+// would lengthen every warp's only visit.
+bool staged_stream_plan(const RunParams &p, StreamPlan *out) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  out->moves_ahead =
+      p.islands / kStageGroup >= 2u * kStagedWarps * kStagedBlocksPerSM * (uint32_t)sms;
+  out->back = planes_exceed_l2(p);
+  return true;
+}
+
+cudaError_t launch_step_staged(const RunParams &p, const StreamPlan &plan, uint32_t G,
+                               bool do_mig, const Moves &mv, const uint32_t *tin,
                                const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
                                cudaStream_t stream) {
   if (p.n != 32) return cudaErrorInvalidValue;
   const Deposit dep = deposit_for(p, G);
-  const bool tracked = p.policy != HSGA_NONE;
-  const bool t2 = p.tournament == 2;
+  const bool tracked = p.policy != HSGA_NONE, t2 = p.tournament == 2;
+  // a second group staged ahead pays where memory is the limit: 16.8M agents
+  // 66.0 against 67.3 us, but untracked 54.5 against 52.7, tournament 5 on
+  // 500x500 islands 61.6 against 60.8, 256x256 islands 11.5 against 11.2
+  const StagedLaunch l{G, plan.back && (G & 1u) ? 1u : 0u, tracked && t2 && plan.back ? 2u : 1u,
+                       mv};
   if (tracked) {
-    if (t2) launch_staged_m<true, true>(p, dep, G, do_mig, tin, sin, tout, sout, err, stream);
-    else launch_staged_m<true, false>(p, dep, G, do_mig, tin, sin, tout, sout, err, stream);
+    if (t2) launch_staged_m<true, true>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
+    else launch_staged_m<true, false>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
   } else {
-    if (t2) launch_staged_m<false, true>(p, dep, G, do_mig, tin, sin, tout, sout, err, stream);
-    else launch_staged_m<false, false>(p, dep, G, do_mig, tin, sin, tout, sout, err, stream);
+    if (t2) launch_staged_m<false, true>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
+    else launch_staged_m<false, false>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
   }
   return cudaGetLastError();
 }
