@@ -22,10 +22,11 @@ constexpr int kFlatMaxSmem = 160 * 1024;  // limit set on the kernels; one block
 template <int K, bool FLT>
 constexpr bool kFlatAhead = K <= 1 && !FLT;
 
-// 20 warps per SM at least; 28 fit by themselves where a tournament of 2 and
-// narrow surfaces leave the registers, and planning must not take them away.
+// Warps per SM: 28 fit by themselves where a tournament of 2 and narrow surfaces
+// leave the registers, and planning must not take them away; 16 for larger
+// tournaments and binary32 (hsga_flat.cuh has the alternatives' times).
 template <int K, bool T2, bool FLT, bool LARGE>
-constexpr int kFlatBlocksPerSM = LARGE && T2 && !FLT && K <= 2 ? 7 : 5;
+constexpr int kFlatBlocksPerSM = LARGE && T2 && !FLT && K <= 2 ? 7 : T2 || (K >= 2 && !FLT) ? 5 : 4;
 
 template <int K, bool T2, int NN, bool FLT, bool LARGE>
 __global__ void __launch_bounds__(kFlatThreads, (kFlatBlocksPerSM<K, T2, FLT, LARGE>))

@@ -18,12 +18,23 @@
 // registers; for binary32 fitness and wide surfaces a warp per island after
 // two migration launches): 128x256 islands of 48 8.7 (18.5), of 17 5.5
 // (10.3), of 64 with tournament 5 21.4 (43.0); 500x500 of 32, tournament 5,
-// binary32 94.7 (110); 256x512 of 32 with four surface words 46.2 (66.2), of
+// binary32 89.7 (110); 256x512 of 32 with four surface words 46.1 (66.2), of
 // which 44.5 are its 72 bytes per agent at the measured copy bandwidth; 20x20
-// of 32, binary32 3.4 (14.4).  Three children per lane in flight and 20 warps
-// per SM: 128x256x48 takes a fifth longer with four, a tenth with two (32
-// warps).  Bound by issue: 113 warp instructions per 32 children at n = 48, 51
-// of them on the ALU pipe (two cycles each).
+// of 32, binary32 3.1 (14.4).
+//
+// Children in flight against warps per SM, us: integer, tournament 2: three
+// children and 20-28 warps (128x256x48 takes a fifth longer with four, a tenth
+// with two and 32 warps).  Larger tournaments hold more blocks at once: 64 agents,
+// tournament 5, three children and 16 warps 19.3, 20 warps 21.4, 24 22.7, two
+// children and 28 warps 20.2.  binary32: four and 16 warps 89.7, three and 16
+// 91.2, 20 94.6, two and 32 96.4, four and 12 97.3.  Two surface words: two
+// children 25.5, three 27.4.  (Closing the mutating children up over the lanes
+// before their amounts are drawn: 89.2, but 3.3 on 20x20; generator heads for
+// the second tournament block as well: 64 agents 21.9 for 21.4.)
+//
+// Bound by issue, but for four words: 113 warp instructions per 32 children at
+// n = 48, 51 of them on the ALU pipe (two cycles each); binary32 274, 129 on
+// the ALU and 85 on the multiplier pipe, which binds three blocks a child.
 #pragma once
 
 #include "hsga_moves.cuh"
@@ -32,7 +43,9 @@
 namespace hsga {
 
 constexpr uint32_t kFlatGroup = 8;    // most islands per warp visit
-constexpr uint32_t kFlatUnroll = 3;   // children per lane in flight
+// Children per lane in flight.
+template <int K, bool T2, bool FLT>
+constexpr uint32_t kFlatUnroll = FLT ? 4 : T2 && K >= 2 ? 2 : 3;
 constexpr int kFlatThreads = 128;
 constexpr uint32_t kFlatWarps = kFlatThreads / 32;
 
@@ -172,6 +185,7 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
                                            uint32_t *__restrict__ tout,
                                            uint64_t *__restrict__ sout, FlatStage &st) {
   constexpr int KS = K > 0 ? K : 1;
+  constexpr uint32_t U0 = kFlatUnroll<K, T2, FLT>;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t n = NN ? (uint32_t)NN : p.n;
   const uint32_t cnt = min(group, p.islands - isl0), total = cnt * n;
@@ -257,12 +271,12 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
     return Words4{a0, a1, a2, a3};
   };
   // the first round's draws, while the copy and the gather are in flight
-  uint32_t isl_first[kFlatUnroll], slot_first[kFlatUnroll];
-  Words4 w_first[kFlatUnroll];
-  const bool early = total > 32u * (kFlatUnroll - 1u);
+  uint32_t isl_first[U0], slot_first[U0];
+  Words4 w_first[U0];
+  const bool early = total > 32u * (U0 - 1u);
   if (early) {
 #pragma unroll
-    for (uint32_t u = 0; u < kFlatUnroll; ++u) w_first[u] = draw(0, u, isl_first[u], slot_first[u]);
+    for (uint32_t u = 0; u < U0; ++u) w_first[u] = draw(0, u, isl_first[u], slot_first[u]);
   }
   if (copy) {
     if (!__all_sync(kFull, mbar_wait(st.bar, st.phase))) return false;
@@ -405,13 +419,13 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
   };
   uint32_t c0 = 0;
   if (early) {
-    children(Count<kFlatUnroll>{}, 0u, isl_first, slot_first, w_first);
-    c0 = 32u * kFlatUnroll;
+    children(Count<U0>{}, 0u, isl_first, slot_first, w_first);
+    c0 = 32u * U0;
   }
-  // full rounds, then the remainder in halves: no lane works beyond the last
+  // full rounds, then the remainder (at most three) in smaller ones: no lane works beyond the last
   // 32 children (a fixed unroll wastes 2 of 8 rounds at n = 24)
-  for (; total > c0 + 32u * (kFlatUnroll - 1u); c0 += 32u * kFlatUnroll)
-    round(Count<kFlatUnroll>{}, c0);
+  for (; total > c0 + 32u * (U0 - 1u); c0 += 32u * U0)
+    round(Count<U0>{}, c0);
   if (total > c0 + 32u) {
     round(Count<2>{}, c0);
     c0 += 64u;
