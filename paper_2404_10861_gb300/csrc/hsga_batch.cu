@@ -39,12 +39,15 @@ struct WorkItem {
   uint32_t run, isl0;
 };
 
-constexpr int kBatchBlocksPerSM = 5;  // 20 warps (<= 96 registers)
+// 16 warps (<= 128 registers, the runs' round keys among them): 104 ms for a
+// 16-run mix; 20 warps, where they spill, 111; 12 warps 110.
+constexpr int kBatchBlocksPerSM = 4;
 
 __global__ void __launch_bounds__(kFlatThreads, kBatchBlocksPerSM)
     batch_step_kernel(const BatchRun *__restrict__ runs, const WorkItem *__restrict__ items,
                       uint32_t n_items, const uint32_t *__restrict__ tick_base,
-                      uint32_t tick_off, uint32_t stage_bytes, int *__restrict__ err) {
+                      uint32_t tick_off, uint32_t stage_bytes, uint32_t may_back,
+                      int *__restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[kFlatWarps];
   const uint32_t lane = threadIdx.x & 31u, wib = __shfl_sync(kFull, threadIdx.x >> 5, 0);
@@ -63,7 +66,11 @@ __global__ void __launch_bounds__(kFlatThreads, kBatchBlocksPerSM)
   const uint32_t nwarps = gridDim.x * kFlatWarps;
   uint32_t i = blockIdx.x * kFlatWarps + wib;
   uint32_t phase = 0;
-  WorkItem w = i < n_items ? items[i] : WorkItem{0u, 0u};
+  // odd ticks walk the list backwards where the planes exceed L2: the last
+  // children written are the first parents read
+  const bool back = may_back != 0u && par != 0u;
+  const auto item = [&](uint32_t k) { return items[back ? n_items - 1u - k : k]; };
+  WorkItem w = i < n_items ? item(i) : WorkItem{0u, 0u};
   while (i < n_items) {
     const uint32_t run = w.run;
     const BatchRun &R = runs[run];
@@ -91,7 +98,7 @@ __global__ void __launch_bounds__(kFlatThreads, kBatchBlocksPerSM)
     do {
       const uint32_t isl0 = w.isl0;
       i += nwarps;
-      if (i < n_items) w = items[i];
+      if (i < n_items) w = item(i);
       const bool ok = t2 ? flat_group<1, true, 0, false>(p, keys, dep, do_mig, bulk, isl0,
                                                          kFlatGroup, G, false, 0u, tin, sin, tout, sout, st)
                          : flat_group<1, false, 0, false>(p, keys, dep, do_mig, bulk, isl0,
@@ -149,6 +156,7 @@ struct hsga_batch {
   // (finishing tick, items up to and including that run)
   std::vector<std::pair<uint64_t, uint32_t>> prefix;
   uint32_t stage_bytes = 0;  // shared memory per warp for the largest island in the list
+  uint32_t back = 0;         // odd ticks walk the list backwards
   int most_per_sm = 1;       // blocks that an SM keeps resident with it
   int per_sm = 0;            // blocks per SM that ticks are launched with
   std::map<int, int> tuned;  // per_sm by log4 of the item count
@@ -217,14 +225,17 @@ cudaError_t rebuild_items(hsga_batch *b) {
   b->h_items.clear();
   b->prefix.clear();
   uint32_t n_max = 1;
+  uint64_t agents = 0;
   for (uint32_t r : order) {
     const HostRun &R = b->runs[r];
+    agents += R.agents;
     n_max = std::max(n_max, R.p.n);
     for (uint32_t i0 = 0; i0 < R.p.islands; i0 += kFlatGroup)
       b->h_items.push_back(WorkItem{r, i0});
     b->prefix.push_back({R.start_tick + R.budget, (uint32_t)b->h_items.size()});
   }
   b->stage_bytes = flat_stage_bytes(n_max, 1);
+  b->back = exceeds_l2(24u * agents) ? 1u : 0u;  // both planes of 12-byte genomes
   int per_sm = 0;
   cudaError_t e = cudaFuncSetAttribute(batch_step_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
@@ -286,7 +297,7 @@ cudaError_t launch_tick(hsga_batch *b, uint32_t off) {
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, batch_step_kernel, (const BatchRun *)b->d_runs,
                             (const WorkItem *)b->d_items, b->n_items,
-                            (const uint32_t *)b->d_tick, off, b->stage_bytes,
+                            (const uint32_t *)b->d_tick, off, b->stage_bytes, b->back,
                             (int *)(b->d_tick + 1));
 }
 

@@ -66,6 +66,7 @@ bool stream_plan(const RunParams &p, StreamPlan *out);
 // of 32 with four surface words: 46.2 us per generation, 54.9 without; grids
 // that fit lose 1%).
 bool planes_exceed_l2(const RunParams &p);
+bool exceeds_l2(uint64_t bytes);
 cudaError_t launch_step_streamed(const RunParams &p, const StreamPlan &plan, uint32_t G,
                                  bool do_mig, const Moves &mv, const uint32_t *tin,
                                  const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,

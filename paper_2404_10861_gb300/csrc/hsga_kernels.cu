@@ -20,13 +20,16 @@ namespace hsga {
 // kernel of their own, which plans its launches itself.
 static bool staged_shape(const RunParams &p) { return p.n == 32 && p.words == 1 && !p.flt; }
 
-bool planes_exceed_l2(const RunParams &p) {
+bool exceeds_l2(uint64_t bytes) {
   int dev = 0, l2 = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
-    return false;
+  return cudaGetDevice(&dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) == cudaSuccess &&
+         bytes > (uint64_t)l2;
+}
+
+bool planes_exceed_l2(const RunParams &p) {
   const uint64_t genome = 4u + 8u * (p.policy == HSGA_NONE ? 0u : p.words);
-  return 2u * genome * p.n * p.islands > (uint64_t)l2;
+  return exceeds_l2(2u * genome * p.n * p.islands);
 }
 
 bool stream_plan(const RunParams &p, StreamPlan *out) {
