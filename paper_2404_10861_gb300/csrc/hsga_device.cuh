@@ -174,8 +174,8 @@ struct RunParams {
   uint32_t flt;            // binary32 fitness with Gaussian mutation amounts
   float gscale;            // float(sigma / sqrt(24 + 1/12) / 2^24)
   FastDiv cols_div;        // island -> (row, column)
-  uint32_t n_recip;        // floor(2^16 / n) + 1: agent of a few islands -> island
   uint32_t rk0[10], rk1[10];  // Philox round keys k + r * (W0, W1)
+  uint32_t n_recip;        // floor(2^16 / n) + 1: agent of a few islands -> island
 };
 
 inline void set_round_keys(RunParams &p) {
