@@ -19,6 +19,7 @@ constexpr int kStagedThreads = 256;     // staged streamed kernel (n = 32) block
 // groups of 16 in two halves 70.5 / 61.3 / 10.8.  Groups of 6 on 24 warps, before:
 // 71.7 / 65.7 / 11.9.
 constexpr int kStagedBlocksPerSM = 2;
+constexpr int kSmallStagedBlocksPerSM = 3;  // groups of four islands: 24 warps
 constexpr uint32_t kStagedStages = 2;   // most groups in flight per warp
 constexpr int kResidentThreads = 128;   // free-running, float and wide kernels: 4 warps
 constexpr uint64_t kWaitNs = 1000000000ull; // bounded device wait: 1 s

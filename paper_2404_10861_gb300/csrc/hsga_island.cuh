@@ -242,14 +242,14 @@ __device__ __forceinline__ void store_island(const RunParams &p, uint32_t isl,
 // Up to kGroup islands from isl0 on, one at a time.
 template <int AP, bool TRACKED, bool T2, bool RK = true>
 __device__ __noinline__ void partial_group(const RunParams &p, const Deposit &dep, uint32_t G,
-                                           bool do_mig, uint32_t isl0,
+                                           bool do_mig, uint32_t isl0, uint32_t count,
                                            const uint32_t *__restrict__ tin,
                                            const uint64_t *__restrict__ sin,
                                            uint32_t *__restrict__ tout,
                                            uint64_t *__restrict__ sout) {
   GroupMigration gm;
   if (do_mig) group_migration<TRACKED, RK>(p, isl0, G, tin, sin, gm);
-  for (uint32_t k = 0; k < kGroup && isl0 + k < p.islands; ++k) {
+  for (uint32_t k = 0; k < count; ++k) {
     uint32_t pt[AP], ct[AP];
     uint64_t ps[AP], cs[AP];
     load_island<AP, TRACKED>(p, isl0 + k, tin, sin, pt, ps);

@@ -883,6 +883,12 @@ uint32_t threads_for(uint32_t I, uint32_t n) {
 // block, 0.69 in 16; 30 islands: 0.84 and 0.68).
 constexpr uint32_t kOneBlockAgents = 768;
 
+// Tiles of one island poll again just before their neighbours' records arrive
+// once they spread over most of the device: 10x12 islands in 120 tiles 1.33 us
+// per generation, in 60 tiles of two 1.12; 12x12 0.94 and 0.73; 8x12 in 96
+// tiles 0.70.
+constexpr uint32_t kMostSingles = 96;
+
 bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
   int dev = 0, sms = 0, coop = 0, smem = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
@@ -912,6 +918,7 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
       const uint32_t most_c = (uint32_t)sms / tiles_r;
       const uint32_t tc = (p.cols + most_c - 1) / most_c;
       if (bytes((uint64_t)tr * tc) > (uint32_t)smem) continue;
+      if (tr * tc == 1u && p.islands > kMostSingles) continue;
       const double edge = (p.rows > tr ? 2.0 * tc : 0.0) + (p.cols > tc ? 2.0 * tr : 0.0);
       const double cost = (double)tr * tc * p.n / 32.0 + 0.1 * edge;
       if (cost < best) {

@@ -19,11 +19,12 @@
 namespace hsga {
 
 constexpr uint32_t kStagedWarps = kStagedThreads / 32;
-constexpr uint32_t kStageGroup = 8;  // islands per stage
-constexpr uint32_t kStageWords = kStageGroup / 8;
-constexpr uint32_t kStageAgents = kStageGroup * 32;
-constexpr uint32_t kTraitBytes = kStageAgents * 4;  // 1,024
-constexpr uint32_t kSurfBytes = kStageAgents * 8;   // 2,048
+// Islands per stage: eight; four on grids that so take one round of groups.
+constexpr uint32_t kStageGroup = 8, kSmallStageGroup = 4;
+template <uint32_t GR>
+constexpr uint32_t kTraitBytes = GR * 32 * 4;
+template <uint32_t GR>
+constexpr uint32_t kSurfBytes = GR * 32 * 8;
 constexpr uint32_t kMaxPolls = 1u << 24;
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
@@ -91,98 +92,84 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   return false;
 }
 
-// A lane's immigrants to a staged group, lane 4i + d of word a the one of
-// island 8a + i from direction d: the agent of the group that it overwrites
-// (none: kNoArrival) and its genome.
+// A lane's immigrant to a staged group of GR islands, lane 4i + d the one of
+// island i from direction d: the agent of the group that it overwrites (none:
+// kNoArrival) and its genome.
 constexpr uint32_t kNoArrival = 0xFFFFFFFFu;
-struct Arrivals {
-  uint32_t at[kStageWords], it[kStageWords];
-  uint64_t is[kStageWords];
+struct Arrival {
+  uint32_t at, it;
+  uint64_t is;
 };
 
-// a1 and a2 derived here, for all of the group's islands.
-template <bool TRACKED>
-__device__ __forceinline__ void derive_arrivals(const RunParams &p, uint32_t isl0, uint32_t G,
-                                                const uint32_t *__restrict__ tin,
-                                                const uint64_t *__restrict__ sin, Arrivals &r) {
-  const uint32_t lane = threadIdx.x & 31u, d = lane & 3u;
-  const Words4 v = philox_rk(p, kSlotImmigrant, isl0 + min(lane, kStageGroup - 1u), G,
-                             kPurposeMigration);
+// a1 and a2 derived here.
+template <bool TRACKED, uint32_t GR>
+__device__ __forceinline__ Arrival derive_arrival(const RunParams &p, uint32_t isl0, uint32_t G,
+                                                  const uint32_t *__restrict__ tin,
+                                                  const uint64_t *__restrict__ sin) {
+  const uint32_t lane = threadIdx.x & 31u, d = lane & 3u, i = min(lane >> 2, GR - 1u);
+  const Words4 v =
+      philox_rk(p, kSlotImmigrant, isl0 + min(lane, GR - 1u), G, kPurposeMigration);
   const uint32_t plan =
       v.x >> 27 | (v.y >> 27) << 8 | (v.z >> 27) << 16 | (v.w >> 27) << 24;
-#pragma unroll
-  for (uint32_t a = 0; a < kStageWords; ++a) {
-    const uint32_t i = 8u * a + (lane >> 2);
-    const uint32_t src = neighbour(p, isl0 + i, d);
-    const Words4 m = philox_rk(p, kSlotEmigrant, src, G, kPurposeMigration);
-    const bool arrive = (m.y >> 30) == (d ^ 2u);
-    r.at[a] = kNoArrival;
-    if (arrive) {
-      const uint32_t x = src * 32u + (m.x >> 27);
-      r.it[a] = __ldg(tin + x);
-      if constexpr (TRACKED) r.is[a] = __ldg(sin + x);
-    }
-    const uint32_t to = __shfl_sync(kFull, plan, i);
-    const uint32_t bits = (__ballot_sync(kFull, arrive) >> (lane & 28u)) & 0xFu;
-    const uint32_t slot = (to >> (8u * d)) & 0xFFu;
-    bool lands = arrive;
-#pragma unroll
-    for (uint32_t e = 1; e < 4; ++e)  // the latest of N, E, S, W wins a shared slot
-      lands = lands && !(e > d && (bits >> e & 1u) && ((to >> (8u * e)) & 0xFFu) == slot);
-    if (lands) r.at[a] = 32u * i + slot;
+  const uint32_t src = neighbour(p, isl0 + i, d);
+  const Words4 m = philox_rk(p, kSlotEmigrant, src, G, kPurposeMigration);
+  const bool arrive = lane < 4u * GR && (m.y >> 30) == (d ^ 2u);
+  Arrival r{kNoArrival, 0u, 0ull};
+  if (arrive) {
+    const uint32_t x = src * 32u + (m.x >> 27);
+    r.it = __ldg(tin + x);
+    if constexpr (TRACKED) r.is = __ldg(sin + x);
   }
+  const uint32_t to = __shfl_sync(kFull, plan, i);
+  const uint32_t bits = (__ballot_sync(kFull, arrive) >> (lane & 28u)) & 0xFu;
+  const uint32_t slot = (to >> (8u * d)) & 0xFFu;
+  bool lands = arrive;
+#pragma unroll
+  for (uint32_t e = 1; e < 4; ++e)  // the latest of N, E, S, W wins a shared slot
+    lands = lands && !(e > d && (bits >> e & 1u) && ((to >> (8u * e)) & 0xFFu) == slot);
+  if (lands) r.at = 32u * i + slot;
+  return r;
 }
 
-// The same from the lane's planned moves.
+// The same from the lane's planned move (0: none).
 template <bool TRACKED>
-__device__ __forceinline__ void planned_arrivals(const RunParams &p,
-                                                 const uint32_t (&move)[kStageWords],
-                                                 uint32_t isl0, const uint32_t *__restrict__ tin,
-                                                 const uint64_t *__restrict__ sin, Arrivals &r) {
-  const uint32_t lane = threadIdx.x & 31u;
-#pragma unroll
-  for (uint32_t a = 0; a < kStageWords; ++a) {
-    const uint32_t i = 8u * a + (lane >> 2);
-    r.at[a] = kNoArrival;
-    if (move[a] & kMoveLands) {
-      const uint32_t x = neighbour(p, isl0 + i, lane & 3u) * 32u + (move[a] >> 6 & 31u);
-      r.at[a] = 32u * i + (move[a] & 31u);
-      r.it[a] = __ldg(tin + x);
-      if constexpr (TRACKED) r.is[a] = __ldg(sin + x);
-    }
+__device__ __forceinline__ Arrival planned_arrival(const RunParams &p, uint32_t move,
+                                                   uint32_t isl0,
+                                                   const uint32_t *__restrict__ tin,
+                                                   const uint64_t *__restrict__ sin) {
+  const uint32_t lane = threadIdx.x & 31u, i = lane >> 2;
+  Arrival r{kNoArrival, 0u, 0ull};
+  if (move & kMoveLands) {
+    const uint32_t x = neighbour(p, isl0 + i, lane & 3u) * 32u + (move >> 6 & 31u);
+    r.at = 32u * i + (move & 31u);
+    r.it = __ldg(tin + x);
+    if constexpr (TRACKED) r.is = __ldg(sin + x);
   }
-}
-
-// The lane's planned moves of a group.
-__device__ __forceinline__ void load_moves(const Moves &mv, uint32_t isl0,
-                                           uint32_t (&move)[kStageWords]) {
-#pragma unroll
-  for (uint32_t a = 0; a < kStageWords; ++a)
-    move[a] = mv.now[(size_t)isl0 * 4u + 32u * a + (threadIdx.x & 31u)];
+  return r;
 }
 
 // a3-a6 of child `lane` of every island of a staged group (parents of island
 // i at tr + 32 i, sr + 32 i), stored to to + 32 i, so + 32 i.  All of the
 // group's reads come before its first store: the stores order memory for the
 // compiler, which would otherwise finish one island before it reads the next.
-template <bool TRACKED, bool T2, bool TWO, bool DEL, class More>
+template <bool TRACKED, bool T2, bool TWO, bool DEL, uint32_t GR, class More>
 __device__ __forceinline__ void replicate_group(const RunParams &p, const Deposit &dep,
-                                                const Words4 (&w)[kStageGroup], const uint32_t *tr,
+                                                const Words4 (&w)[GR], const uint32_t *tr,
                                                 const uint64_t *sr, uint32_t *to, uint64_t *so,
                                                 const More &more) {
-  uint32_t best[kStageGroup], fbest[kStageGroup];
-  uint64_t cs[kStageGroup];
+  uint32_t best[GR], fbest[GR];
+  uint64_t cs[GR];
 #pragma unroll
-  for (uint32_t i = 0; i < kStageGroup; ++i) {
+  for (uint32_t i = 0; i < GR; ++i) {
     best[i] = w[i].x >> 27;
     fbest[i] = tr[32u * i + best[i]];
   }
   if (T2 || p.tournament >= 2) {
-    uint32_t fc[kStageGroup];
+    uint32_t fc[GR];
 #pragma unroll
-    for (uint32_t i = 0; i < kStageGroup; ++i) fc[i] = tr[32u * i + (w[i].y >> 27)];
+    for (uint32_t i = 0; i < GR; ++i) fc[i] = tr[32u * i + (w[i].y >> 27)];
 #pragma unroll
-    for (uint32_t i = 0; i < kStageGroup; ++i) {
+    for (uint32_t i = 0; i < GR; ++i) {
       best[i] = fc[i] > fbest[i] ? w[i].y >> 27 : best[i];
       fbest[i] = max(fc[i], fbest[i]);
     }
@@ -190,7 +177,7 @@ __device__ __forceinline__ void replicate_group(const RunParams &p, const Deposi
   if constexpr (!T2) {
     for (uint32_t c0 = 2; c0 < p.tournament; c0 += 4) {
 #pragma unroll
-      for (uint32_t i = 0; i < kStageGroup; ++i) {
+      for (uint32_t i = 0; i < GR; ++i) {
         const Words4 e = more(i, (c0 - 2) / 4);
         const uint32_t ew[4] = {e.x >> 27, e.y >> 27, e.z >> 27, e.w >> 27};
         uint32_t fc[4];
@@ -207,25 +194,30 @@ __device__ __forceinline__ void replicate_group(const RunParams &p, const Deposi
   }
   if constexpr (TRACKED) {
 #pragma unroll
-    for (uint32_t i = 0; i < kStageGroup; ++i) cs[i] = sr[32u * i + best[i]];
+    for (uint32_t i = 0; i < GR; ++i) cs[i] = sr[32u * i + best[i]];
   }
 #pragma unroll
-  for (uint32_t i = 0; i < kStageGroup; ++i) {
+  for (uint32_t i = 0; i < GR; ++i) {
     __stcs(to + 32u * i, mutate<DEL>(p, fbest[i], w[i].z));
     if constexpr (TRACKED) __stcs(so + 32u * i, deposit_into<TWO>(dep, cs[i], w[i].w));
   }
 }
 
-constexpr uint32_t kStageBytes = kTraitBytes + kSurfBytes;  // 2304 per group
-constexpr size_t kRingBytes = (size_t)kStagedWarps * kStagedStages * kStageBytes;
+template <uint32_t GR>
+constexpr uint32_t kStageBytes = kTraitBytes<GR> + kSurfBytes<GR>;
+template <uint32_t GR>
+constexpr size_t kRingBytes = (size_t)kStagedWarps * kStagedStages * kStageBytes<GR>;
+template <uint32_t GR>
+constexpr int kStagedBlocks = GR == kStageGroup ? kStagedBlocksPerSM : kSmallStagedBlocksPerSM;
 
 // Shared memory requested per block: the ring, padded so that one block
-// more than kStagedBlocksPerSM does not fit on an SM.  Otherwise the next
+// more than kStagedBlocks does not fit on an SM.  Otherwise the next
 // generation's launch, scheduled early by programmatic dependent launch,
 // parks a block in the free slot that competes with the running blocks for
 // issue slots until it may start (107 us per generation at 16.8M agents
 // with a free slot, 75.3 us without).
-inline size_t staged_smem_bytes() {
+template <uint32_t GR>
+size_t staged_smem_bytes() {
   static size_t bytes = 0;
   if (bytes == 0) {
     int dev = 0, per_sm = 0, per_block = 0, reserved = 0;
@@ -233,10 +225,10 @@ inline size_t staged_smem_bytes() {
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    size_t pad = (size_t)per_sm / (kStagedBlocksPerSM + 1) + 128;
+    size_t pad = (size_t)per_sm / (kStagedBlocks<GR> + 1) + 128;
     pad = pad > (size_t)reserved ? pad - (size_t)reserved : pad;
-    size_t b = kRingBytes > pad ? kRingBytes : pad;
-    if (per_block > 0 && b > (size_t)per_block - 1024) b = kRingBytes;  // no room to pad
+    size_t b = kRingBytes<GR> > pad ? kRingBytes<GR> : pad;
+    if (per_block > 0 && b > (size_t)per_block - 1024) b = kRingBytes<GR>;  // no room to pad
     bytes = (b + 127) & ~(size_t)127;
   }
   return bytes;

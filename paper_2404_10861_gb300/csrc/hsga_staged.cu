@@ -52,8 +52,8 @@ struct StagedLaunch {
   Moves mv;
 };
 
-template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG>
-__global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
+template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG, uint32_t GR>
+__global__ void __launch_bounds__(kStagedThreads, (kStagedBlocks<GR>))
     step_staged_kernel(RunParams p, Deposit dep, StagedLaunch l, const uint32_t *__restrict__ tin,
                        const uint64_t *__restrict__ sin, uint32_t *__restrict__ tout,
                        uint64_t *__restrict__ sout, int *__restrict__ err) {
@@ -64,19 +64,19 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
   const uint32_t lane = threadIdx.x & 31u, wib = __shfl_sync(kFull, threadIdx.x >> 5, 0);
   const uint32_t warp = blockIdx.x * kStagedWarps + wib;
   const uint32_t nwarps = gridDim.x * kStagedWarps;
-  const uint32_t nfull = p.islands / kStageGroup;
-  unsigned char *ring = s_ring + (size_t)wib * kStagedStages * kStageBytes;
+  const uint32_t nfull = p.islands / GR;
+  unsigned char *ring = s_ring + (size_t)wib * kStagedStages * kStageBytes<GR>;
   uint64_t *bar = s_bar[wib];
-  constexpr uint32_t kTx = kTraitBytes + (TRACKED ? kSurfBytes : 0u);
+  constexpr uint32_t kTx = kTraitBytes<GR> + (TRACKED ? kSurfBytes<GR> : 0u);
 
   // stage st holds a group's traits (1,024 B) then its surfaces (2,048 B)
   auto issue = [&](uint32_t isl0, uint32_t st) {  // one lane
-    unsigned char *dst = ring + st * kStageBytes;
+    unsigned char *dst = ring + st * kStageBytes<GR>;
     proxy_fence();
     mbar_expect_tx(&bar[st], kTx);
-    bulk_load(dst, tin + (size_t)isl0 * 32u, kTraitBytes, &bar[st]);
+    bulk_load(dst, tin + (size_t)isl0 * 32u, kTraitBytes<GR>, &bar[st]);
     if constexpr (TRACKED)
-      bulk_load(dst + kTraitBytes, sin + (size_t)isl0 * 32u, kSurfBytes, &bar[st]);
+      bulk_load(dst + kTraitBytes<GR>, sin + (size_t)isl0 * 32u, kSurfBytes<GR>, &bar[st]);
   };
 
   // the next launch may be scheduled now; it waits below for this one
@@ -86,8 +86,8 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
     for (uint32_t st = 0; st < stages; ++st) mbar_init(&bar[st], 1);
     mbar_init_fence();
   }
-  const uint32_t first = (l.back ? nfull - 1u - warp : warp) * kStageGroup;
-  const uint32_t skip = l.back ? 0u - nwarps * kStageGroup : nwarps * kStageGroup;
+  const uint32_t first = (l.back ? nfull - 1u - warp : warp) * GR;
+  const uint32_t skip = l.back ? 0u - nwarps * GR : nwarps * GR;
   const LaneHead head = lane_head(p, lane, G, kPurposeReplicate);
   [[maybe_unused]] LaneHead head2;  // candidates 2-5
   if constexpr (!T2) head2 = lane_head(p, lane, G, kPurposeReplicate + 1u);
@@ -104,38 +104,40 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
   // The immigrants of a group are gathered while the group before it is
   // replicated: the gather's latency, with nothing to hide it, made up a
   // third of a generation on L2-resident grids.
-  Arrivals next;
-  uint32_t move[kStageWords] = {};  // planned, of the group after the next
+  // Only groups of eight plan ahead: a round of smaller ones is too short.
+  constexpr bool PLAN = GR == kStageGroup;
+  const bool planned = PLAN && mv.now != nullptr;
+  Arrival next{kNoArrival, 0u, 0ull};
+  uint32_t move = 0;  // planned, of the group after the next
+  const auto load_of = [&](uint32_t isl) { return (uint32_t)mv.now[(size_t)isl * 4u + lane]; };
   if constexpr (MIG) {
     if (warp < nfull) {
-      const uint32_t isl0 = first;
-      if (mv.now) {
-        load_moves(mv, isl0, move);
-        planned_arrivals<TRACKED>(p, move, isl0, tin, sin, next);
-        if (warp + nwarps < nfull) load_moves(mv, isl0 + skip, move);
+      if (planned) {
+        next = planned_arrival<TRACKED>(p, load_of(first), first, tin, sin);
+        if (warp + nwarps < nfull) move = load_of(first + skip);
       } else {
-        derive_arrivals<TRACKED>(p, isl0, G, tin, sin, next);
+        next = derive_arrival<TRACKED, GR>(p, first, G, tin, sin);
       }
     }
   }
-  Planner planner(p, mv, warp, nwarps);
+  [[maybe_unused]] Planner planner(p, mv, warp, nwarps);
   uint32_t st = 0, phase = 0;  // ring position of the k-th group and its phase parity
   uint32_t isl0 = first;
   for (uint32_t grp = warp; grp < nfull; grp += nwarps, isl0 += skip) {
-    const Arrivals in = next;
+    const Arrival in = next;
     if constexpr (MIG) {
       if (grp + nwarps < nfull) {
-        if (mv.now) {
-          planned_arrivals<TRACKED>(p, move, isl0 + skip, tin, sin, next);
-          if (grp + 2u * nwarps < nfull) load_moves(mv, isl0 + 2u * skip, move);
+        if (planned) {
+          next = planned_arrival<TRACKED>(p, move, isl0 + skip, tin, sin);
+          if (grp + 2u * nwarps < nfull) move = load_of(isl0 + 2u * skip);
         } else {
-          derive_arrivals<TRACKED>(p, isl0 + skip, G, tin, sin, next);
+          next = derive_arrival<TRACKED, GR>(p, isl0 + skip, G, tin, sin);
         }
       }
     }
-    Words4 w[kStageGroup];
+    Words4 w[GR];
 #pragma unroll
-    for (uint32_t i = 0; i < kStageGroup; ++i) w[i] = lane_tail(p, head, isl0 + i);
+    for (uint32_t i = 0; i < GR; ++i) w[i] = lane_tail(p, head, isl0 + i);
     if (!__all_sync(kFull, mbar_wait(&bar[st], phase))) {
       // give up: record the timeout, wait (bounded) for this warp's copies
       // still in flight (the groups issued into the ring from this one on),
@@ -154,91 +156,89 @@ __global__ void __launch_bounds__(kStagedThreads, kStagedBlocksPerSM)
       __syncwarp();
       break;
     }
-    uint32_t *tr = (uint32_t *)(ring + st * kStageBytes);
-    uint64_t *sr = (uint64_t *)(ring + st * kStageBytes + kTraitBytes);
+    uint32_t *tr = (uint32_t *)(ring + st * kStageBytes<GR>);
+    uint64_t *sr = (uint64_t *)(ring + st * kStageBytes<GR> + kTraitBytes<GR>);
     if constexpr (MIG) {
-#pragma unroll
-      for (uint32_t a = 0; a < kStageWords; ++a) {
-        if (in.at[a] != kNoArrival) {
-          tr[in.at[a]] = in.it[a];
-          if constexpr (TRACKED) sr[in.at[a]] = in.is[a];
-        }
+      if (in.at != kNoArrival) {
+        tr[in.at] = in.it;
+        if constexpr (TRACKED) sr[in.at] = in.is;
       }
       __syncwarp();
     }
     uint32_t *to = tout + (size_t)isl0 * 32u + lane;
     uint64_t *so = TRACKED ? sout + (size_t)isl0 * 32u + lane : sout;
-    replicate_group<TRACKED, T2, TWO, DEL>(
+    replicate_group<TRACKED, T2, TWO, DEL, GR>(
         p, dep, w, tr, sr, to, so, [&](uint32_t i, uint32_t q) {
           return q == 0 ? lane_tail(p, head2, isl0 + i)
                         : philox_rk(p, lane, isl0 + i, G, kPurposeReplicate + 1 + q);
         });
     __syncwarp();  // every lane is done with this stage before it is refilled
     if (lane == 0 && grp + stages * nwarps < nfull) issue(isl0 + stages * skip, st);
-    planner.visit<32>(p, p, mv, G, kStageGroup);
+    if constexpr (PLAN) planner.visit<32>(p, p, mv, G, GR);
     if (++st == stages) {
       st = 0;
       phase ^= 1u;
     }
   }
-  planner.rest<32>(p, p, mv, G);
-  // the last islands, too few for a group, on the register path
-  if (warp == nfull % nwarps)
-    for (uint32_t i = nfull * kStageGroup; i < p.islands; i += kGroup)
-      partial_group<1, TRACKED, T2>(p, dep, G, MIG, i, tin, sin, tout, sout);
+  if constexpr (PLAN) planner.rest<32>(p, p, mv, G);
+  // the last islands, too few for a group, on the register path, one to a warp
+  // (333x337 islands 16.2 us; all of them on one warp 18.5)
+  const uint32_t rest = nfull * GR + (nwarps - 1u - warp);
+  if (rest < p.islands)
+    partial_group<1, TRACKED, T2>(p, dep, G, MIG, rest, 1u, tin, sin, tout, sout);
 }
 
-template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG>
+template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG, uint32_t GR>
 int staged_blocks() {
   static int blocks = 0;
   if (blocks == 0) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t smem = staged_smem_bytes();
-    cudaFuncSetAttribute(step_staged_kernel<TRACKED, T2, TWO, DEL, MIG>,
+    const size_t smem = staged_smem_bytes<GR>();
+    cudaFuncSetAttribute(step_staged_kernel<TRACKED, T2, TWO, DEL, MIG, GR>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, step_staged_kernel<TRACKED, T2, TWO, DEL, MIG>, kStagedThreads, smem);
-    if (per_sm > kStagedBlocksPerSM) per_sm = kStagedBlocksPerSM;
+        &per_sm, step_staged_kernel<TRACKED, T2, TWO, DEL, MIG, GR>, kStagedThreads, smem);
+    if (per_sm > kStagedBlocks<GR>) per_sm = kStagedBlocks<GR>;
     blocks = sms * (per_sm > 0 ? per_sm : 1);
   }
   return blocks;
 }
 
-template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG>
+template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG, uint32_t GR>
 void launch_staged_t(const RunParams &p, const Deposit &dep, const StagedLaunch &l,
                      const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
                      int *err, cudaStream_t stream) {
-  const uint32_t groups = (p.islands + kStageGroup - 1) / kStageGroup;
+  const uint32_t groups = (p.islands + GR - 1) / GR;
   const uint32_t need = (groups + kStagedWarps - 1) / kStagedWarps;
-  int b = staged_blocks<TRACKED, T2, TWO, DEL, MIG>();
+  int b = staged_blocks<TRACKED, T2, TWO, DEL, MIG, GR>();
   if ((uint32_t)b > need) b = (int)need;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)b);
   cfg.blockDim = dim3(kStagedThreads);
-  cfg.dynamicSmemBytes = staged_smem_bytes();
+  cfg.dynamicSmemBytes = staged_smem_bytes<GR>();
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, step_staged_kernel<TRACKED, T2, TWO, DEL, MIG>, p, dep, l, tin, sin,
+  cudaLaunchKernelEx(&cfg, step_staged_kernel<TRACKED, T2, TWO, DEL, MIG, GR>, p, dep, l, tin, sin,
                      tout, sout, err);
 }
 
-template <bool TRACKED, bool T2>
+template <bool TRACKED, bool T2, uint32_t GR>
 void launch_staged_m(const RunParams &p, const Deposit &dep, const StagedLaunch &l, bool mig,
                      const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
                      int *err, cudaStream_t stream) {
 #define HSGA_STAGED(TWO_, DEL_)                                                               \
   if (mig)                                                                                    \
-    launch_staged_t<TRACKED, T2, TWO_, DEL_, true>(p, dep, l, tin, sin, tout, sout, err,      \
-                                                   stream);                                   \
+    launch_staged_t<TRACKED, T2, TWO_, DEL_, true, GR>(p, dep, l, tin, sin, tout, sout, err,  \
+                                                       stream);                               \
   else                                                                                        \
-    launch_staged_t<TRACKED, T2, TWO_, DEL_, false>(p, dep, l, tin, sin, tout, sout, err,     \
-                                                    stream);
+    launch_staged_t<TRACKED, T2, TWO_, DEL_, false, GR>(p, dep, l, tin, sin, tout, sout, err, \
+                                                        stream);
   if (TRACKED && dep.two) {
     HSGA_STAGED(true, true)
   } else if (p.has_del) {
@@ -247,6 +247,20 @@ void launch_staged_m(const RunParams &p, const Deposit &dep, const StagedLaunch 
     HSGA_STAGED(false, false)
   }
 #undef HSGA_STAGED
+}
+
+template <uint32_t GR>
+void launch_staged_g(const RunParams &p, const Deposit &dep, const StagedLaunch &l, bool mig,
+                     const uint32_t *tin, const uint64_t *sin, uint32_t *tout, uint64_t *sout,
+                     int *err, cudaStream_t stream) {
+  const bool t2 = p.tournament == 2;
+  if (p.policy != HSGA_NONE) {
+    if (t2) launch_staged_m<true, true, GR>(p, dep, l, mig, tin, sin, tout, sout, err, stream);
+    else launch_staged_m<true, false, GR>(p, dep, l, mig, tin, sin, tout, sout, err, stream);
+  } else {
+    if (t2) launch_staged_m<false, true, GR>(p, dep, l, mig, tin, sin, tout, sout, err, stream);
+    else launch_staged_m<false, false, GR>(p, dep, l, mig, tin, sin, tout, sout, err, stream);
+  }
 }
 
 }  // namespace
@@ -260,6 +274,12 @@ bool staged_stream_plan(const RunParams &p, StreamPlan *out) {
   out->moves_ahead =
       p.islands / kStageGroup >= 2u * kStagedWarps * kStagedBlocksPerSM * (uint32_t)sms;
   out->back = planes_exceed_l2(p);
+  // groups of four where they take one round of the warps: the generation is
+  // then one group's latency (16x16 islands 2.5 us, 3.0 with groups of eight;
+  // 64x63 with a tournament of 5 5.6 and 6.3)
+  const uint32_t one_round =
+      kSmallStageGroup * kStagedWarps * kSmallStagedBlocksPerSM * (uint32_t)sms;
+  out->group = (int)(p.islands <= one_round ? kSmallStageGroup : kStageGroup);
   return true;
 }
 
@@ -275,13 +295,10 @@ cudaError_t launch_step_staged(const RunParams &p, const StreamPlan &plan, uint3
   // 500x500 islands 61.6 against 60.8, 256x256 islands 11.5 against 11.2
   const StagedLaunch l{G, plan.back && (G & 1u) ? 1u : 0u, tracked && t2 && plan.back ? 2u : 1u,
                        mv};
-  if (tracked) {
-    if (t2) launch_staged_m<true, true>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
-    else launch_staged_m<true, false>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
-  } else {
-    if (t2) launch_staged_m<false, true>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
-    else launch_staged_m<false, false>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
-  }
+  if (plan.group == (int)kSmallStageGroup)
+    launch_staged_g<kSmallStageGroup>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
+  else
+    launch_staged_g<kStageGroup>(p, dep, l, do_mig, tin, sin, tout, sout, err, stream);
   return cudaGetLastError();
 }
 

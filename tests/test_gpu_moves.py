@@ -22,6 +22,9 @@ def hb():
 
 
 CASES = [
+    dict(rows=1, cols=3), dict(rows=7, cols=1, tournament=5), dict(rows=5, cols=6),  # groups of four
+    dict(rows=41, cols=59, policy="hybrid", bits=2), dict(rows=64, cols=228, p_del=0.2),
+    dict(rows=97, cols=151, policy="none", tournament=3),                  # one round of eight
     dict(rows=205, cols=191),                                              # groups of 32-agent islands
     dict(rows=2, cols=19501, interval=2, tournament=5, p_del=0.3),
     dict(rows=39003, cols=1, interval=3, policy="none", calls=(9,)),
