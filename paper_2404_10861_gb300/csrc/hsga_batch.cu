@@ -100,9 +100,9 @@ __global__ void __launch_bounds__(kFlatThreads, kBatchBlocksPerSM)
       i += nwarps;
       if (i < n_items) w = item(i);
       const bool ok = t2 ? flat_group<1, true, 0, false>(p, keys, dep, do_mig, bulk, isl0,
-                                                         kFlatGroup, G, false, 0u, tin, sin, tout, sout, st)
+                                                         kFlatGroup, G, false, 0u, false, tin, sin, tout, sout, st)
                          : flat_group<1, false, 0, false>(p, keys, dep, do_mig, bulk, isl0,
-                                                          kFlatGroup, G, false, 0u, tin, sin, tout, sout, st);
+                                                          kFlatGroup, G, false, 0u, false, tin, sin, tout, sout, st);
       if (!ok) {
         // give up: record the timeout, wait (bounded) for the copy, leave
         if (lane == 0) {

@@ -50,7 +50,11 @@ __global__ void __launch_bounds__(kFlatThreads, (kFlatBlocksPerSM<K, T2, FLT, LA
   flat_heads(p, n, G, st);
   __syncwarp();
   const uint32_t groups = (p.islands + group - 1) / group;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // On small grids the first group's draws come before the wait and overlap the
+  // launch before: 20x20 islands of 32, binary32 2.5 us, 3.1 with the wait first;
+  // 64x64 with four words 4.2 and 5.0; 128x256 of 48 8.0 and 8.7; 20x20 of 17 2.1
+  // and 2.6.  (Large ones lose 2% to the second copy of the loads.)
+  if constexpr (LARGE) asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t warp = blockIdx.x * kFlatWarps + wib, nwarps = gridDim.x * kFlatWarps;
   const bool planned = AHEAD && mv.now != nullptr;
   const auto first_of = [&](uint32_t grp) { 
@@ -67,7 +71,8 @@ __global__ void __launch_bounds__(kFlatThreads, (kFlatBlocksPerSM<K, T2, FLT, LA
     const uint32_t move = next;
     next = move_of(grp + nwarps);
     if (!flat_group<K, T2, NN, FLT, LARGE>(p, p, dep, migrate != 0, bulk != 0, first_of(grp),
-                                           group, G, planned, move, tin, sin, tout, sout, st)) {
+                                           group, G, planned, move, !LARGE && grp == warp, tin,
+                                           sin, tout, sout, st)) {
       // give up: record the timeout, wait (bounded) for the copy, leave (once
       // the moves that later launches read are written)
       if (lane == 0) {

@@ -16,11 +16,11 @@
 //
 // us per generation, here and on the kernels before it (a lane per agent in
 // registers; for binary32 fitness and wide surfaces a warp per island after
-// two migration launches): 128x256 islands of 48 8.7 (18.5), of 17 5.5
-// (10.3), of 64 with tournament 5 21.4 (43.0); 500x500 of 32, tournament 5,
+// two migration launches): 128x256 islands of 48 8.0 (18.5), of 17 4.5
+// (10.3), of 64 with tournament 5 18.8 (43.0); 500x500 of 32, tournament 5,
 // binary32 89.7 (110); 256x512 of 32 with four surface words 46.1 (66.2), of
 // which 44.5 are its 72 bytes per agent at the measured copy bandwidth; 20x20
-// of 32, binary32 3.1 (14.4).
+// of 32, binary32 2.5 (14.4).
 //
 // Children in flight against warps per SM, us: integer, tournament 2: three
 // children and 20-28 warps (128x256x48 takes a fifth longer with four, a tenth
@@ -173,13 +173,15 @@ __device__ __forceinline__ void flat_store(T *at, T value) {
 // grid) from the parent planes to the child planes.  K: surface words (0: no surface).  NN:
 // island size when known (32), else 0.  T2: the tournament size is exactly 2.
 // FLT: binary32 fitness.  planned: `move` is the lane's
-// migration move (0: none).  bulk: the planes allow 16-byte bulk copies.
+// migration move (0: none).  first: wait for the launch
+// before this one once the draws are done.  bulk: the planes allow 16-byte bulk
+// copies.
 // Returns false (on every lane) when the copy did not arrive in time.
 template <int K, bool T2, int NN, bool FLT, bool KEEP = false, class Keys>
 __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
                                            const FlatDeposit<K> &dep, bool migrate, bool bulk,
                                            uint32_t isl0, uint32_t group, uint32_t G,
-                                           bool planned, uint32_t move,
+                                           bool planned, uint32_t move, bool first,
                                            const uint32_t *__restrict__ tin,
                                            const uint64_t *__restrict__ sin,
                                            uint32_t *__restrict__ tout,
@@ -194,34 +196,42 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
     if constexpr (NN == 32) return c >> 5;
     else return (c * p.n_recip) >> 16;  // exact for c < kFlatGroup n, n <= 64
   };
-  // stage the parents (the previous group's reads are behind a warp barrier)
+  // stages the parents (the previous group's reads are behind a warp barrier)
   const bool copy = bulk && ((total | (uint32_t)base) & 3u) == 0u;  // whole 16-byte pieces
-  if (copy) {
-    if (lane == 0) {
-      proxy_fence();
-      mbar_expect_tx(st.bar, total * (4u + 8u * K));
-      bulk_load(st.trait, tin + base, 4u * total, st.bar);
-      if constexpr (K > 0) bulk_load(st.surf, sin + base * K, 8u * K * total, st.bar);
+  const auto stage = [&] {
+    if (copy) {
+      if (lane == 0) {
+        proxy_fence();
+        mbar_expect_tx(st.bar, total * (4u + 8u * K));
+        bulk_load(st.trait, tin + base, 4u * total, st.bar);
+        if constexpr (K > 0) bulk_load(st.surf, sin + base * K, 8u * K * total, st.bar);
+      }
+    } else {
+      for (uint32_t c = lane; c < total; c += 32u) st.trait[c] = __ldcs(tin + base + c);
+      if constexpr (K > 0)
+        for (uint32_t c = lane; c < total * K; c += 32u) st.surf[c] = __ldcs(sin + base * K + c);
     }
-  } else {
-    for (uint32_t c = lane; c < total; c += 32u) st.trait[c] = __ldcs(tin + base + c);
-    if constexpr (K > 0)
-      for (uint32_t c = lane; c < total * K; c += 32u) st.surf[c] = __ldcs(sin + base * K + c);
-  }
+  };
+  if (!first) stage();
   // a1, a2: draws, and the gather of the emigrants aimed at this group
-  uint32_t it = 0;
+  uint32_t it = 0, src = 0, src_slot = 0;
   uint64_t is[KS];
 #pragma unroll
   for (int w = 0; w < KS; ++w) is[w] = 0;
   bool arrive = false;
+  const auto gather = [&] {
+    const size_t a = (size_t)src * n + src_slot;
+    it = __ldg(tin + a);
+    if constexpr (K > 0) {
+#pragma unroll
+      for (int w = 0; w < KS; ++w) is[w] = __ldg(sin + a * K + w);
+    }
+  };
   if (planned) {
     if (move & kMoveLands) {
-      const size_t a = (size_t)neighbour(p, isl0 + (lane >> 2), lane & 3u) * n + (move >> 6 & 63u);
-      it = __ldg(tin + a);
-      if constexpr (K > 0) {
-#pragma unroll
-        for (int w = 0; w < KS; ++w) is[w] = __ldg(sin + a * K + w);
-      }
+      src = neighbour(p, isl0 + (lane >> 2), lane & 3u);
+      src_slot = move >> 6 & 63u;
+      gather();
     }
   } else if (migrate) {
     if (lane < cnt) {
@@ -231,17 +241,11 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
     }
     const uint32_t d = lane & 3u;
     const bool valid = (lane >> 2) < cnt;
-    const uint32_t src = neighbour(p, valid ? isl0 + (lane >> 2) : isl0, d);
+    src = neighbour(p, valid ? isl0 + (lane >> 2) : isl0, d);
     const Words4 m = philox_keys(keys, kSlotEmigrant, src, G, kPurposeMigration);
     arrive = valid && (m.y >> 30) == (d ^ 2u);
-    if (arrive) {
-      const size_t a = (size_t)src * n + uindex_nn<NN>(m.x, n);
-      it = __ldg(tin + a);
-      if constexpr (K > 0) {
-#pragma unroll
-        for (int w = 0; w < KS; ++w) is[w] = __ldg(sin + a * K + w);
-      }
-    }
+    src_slot = uindex_nn<NN>(m.x, n);
+    if (arrive && !first) gather();
   }
   if (lane < kFlatGroup) {
     const uint64_t u = (uint64_t)(st.x0 ^ (isl0 + lane)) * kPhiloxM0;
@@ -277,6 +281,11 @@ __device__ __forceinline__ bool flat_group(const RunParams &p, const Keys &keys,
   if (early) {
 #pragma unroll
     for (uint32_t u = 0; u < U0; ++u) w_first[u] = draw(0, u, isl_first[u], slot_first[u]);
+  }
+  if (first) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    stage();
+    if (arrive) gather();
   }
   if (copy) {
     if (!__all_sync(kFull, mbar_wait(st.bar, st.phase))) return false;

@@ -101,25 +101,17 @@ struct Arrival {
   uint64_t is;
 };
 
-// a1 and a2 derived here.
-template <bool TRACKED, uint32_t GR>
-__device__ __forceinline__ Arrival derive_arrival(const RunParams &p, uint32_t isl0, uint32_t G,
-                                                  const uint32_t *__restrict__ tin,
-                                                  const uint64_t *__restrict__ sin) {
+// The lane's move (hsga_moves.cuh; 0: none) derived here.
+template <uint32_t GR>
+__device__ __forceinline__ uint32_t derive_move(const RunParams &p, uint32_t isl0, uint32_t G) {
   const uint32_t lane = threadIdx.x & 31u, d = lane & 3u, i = min(lane >> 2, GR - 1u);
   const Words4 v =
       philox_rk(p, kSlotImmigrant, isl0 + min(lane, GR - 1u), G, kPurposeMigration);
   const uint32_t plan =
       v.x >> 27 | (v.y >> 27) << 8 | (v.z >> 27) << 16 | (v.w >> 27) << 24;
-  const uint32_t src = neighbour(p, isl0 + i, d);
-  const Words4 m = philox_rk(p, kSlotEmigrant, src, G, kPurposeMigration);
+  const Words4 m =
+      philox_rk(p, kSlotEmigrant, neighbour(p, isl0 + i, d), G, kPurposeMigration);
   const bool arrive = lane < 4u * GR && (m.y >> 30) == (d ^ 2u);
-  Arrival r{kNoArrival, 0u, 0ull};
-  if (arrive) {
-    const uint32_t x = src * 32u + (m.x >> 27);
-    r.it = __ldg(tin + x);
-    if constexpr (TRACKED) r.is = __ldg(sin + x);
-  }
   const uint32_t to = __shfl_sync(kFull, plan, i);
   const uint32_t bits = (__ballot_sync(kFull, arrive) >> (lane & 28u)) & 0xFu;
   const uint32_t slot = (to >> (8u * d)) & 0xFFu;
@@ -127,16 +119,14 @@ __device__ __forceinline__ Arrival derive_arrival(const RunParams &p, uint32_t i
 #pragma unroll
   for (uint32_t e = 1; e < 4; ++e)  // the latest of N, E, S, W wins a shared slot
     lands = lands && !(e > d && (bits >> e & 1u) && ((to >> (8u * e)) & 0xFFu) == slot);
-  if (lands) r.at = 32u * i + slot;
-  return r;
+  return lands ? kMoveLands | (m.x >> 27) << 6 | slot : 0u;
 }
 
-// The same from the lane's planned move (0: none).
+// The immigrant of the lane's move.
 template <bool TRACKED>
-__device__ __forceinline__ Arrival planned_arrival(const RunParams &p, uint32_t move,
-                                                   uint32_t isl0,
-                                                   const uint32_t *__restrict__ tin,
-                                                   const uint64_t *__restrict__ sin) {
+__device__ __forceinline__ Arrival arrival_of(const RunParams &p, uint32_t move, uint32_t isl0,
+                                              const uint32_t *__restrict__ tin,
+                                              const uint64_t *__restrict__ sin) {
   const uint32_t lane = threadIdx.x & 31u, i = lane >> 2;
   Arrival r{kNoArrival, 0u, 0ull};
   if (move & kMoveLands) {

@@ -22,17 +22,17 @@
 // several groups, a launch works out the migration of the two generations after
 // it between its groups and finds its own worked out (hsga_moves.cuh).
 //
-// What bounds it, per generation at 16.8M agents: 66.0 us, of which 59.4 are
+// What bounds it, per generation at 16.8M agents: 64.9 us, of which 59.4 are
 // its 24 bytes per agent at the measured copy bandwidth; half of the issue
 // slots are taken.  Groups of six, each deriving its own migration: 71.7, and 69
 // without any load or store; before the reads of a group came ahead of its
-// stores: 75.2.  Tournament 5 on 500x500 islands 60.8 (65.7, 71.8), untracked
-// 16.8M 53-55 (60.0), 256x256 islands 11.2 (11.9); these are bound by issue.
+// stores: 75.2.  Tournament 5 on 500x500 islands 59.8 (65.7, 71.8), untracked
+// 16.8M 54.2 (60.0), 256x256 islands 10.7 (11.9); these are bound by issue.
 //
 // Consecutive generations overlap at the launch boundary (programmatic
 // dependent launch): a launch lets the next one be scheduled as soon as it
-// starts, and the next one initialises its barriers and generator heads,
-// then waits (griddepcontrol.wait) for this launch to complete and its
+// starts, and the next one initialises its barriers and generator heads and
+// draws its first groups, then waits (griddepcontrol.wait) for this launch to complete and its
 // writes to be visible before it touches either population plane.
 //
 // Waits on a stage are bounded (1 s of %globaltimer): on expiry the warp
@@ -91,6 +91,22 @@ __global__ void __launch_bounds__(kStagedThreads, (kStagedBlocks<GR>))
   const LaneHead head = lane_head(p, lane, G, kPurposeReplicate);
   [[maybe_unused]] LaneHead head2;  // candidates 2-5
   if constexpr (!T2) head2 = lane_head(p, lane, G, kPurposeReplicate + 1u);
+  // Only groups of eight plan ahead: a round of smaller ones is too short.  The
+  // first group's draws come before the wait, beside the launch before: 16x16
+  // islands 2.0 us, 2.5 after it, 64x64 2.3 and 3.9 (tournament 5 4.2 and 5.6),
+  // 256x256 10.7 and 11.2, 16.8M agents 64.9 and 66.0.
+  constexpr bool PLAN = GR == kStageGroup;
+  const bool planned = PLAN && mv.now != nullptr;
+  const auto move_of = [&](uint32_t isl) {
+    return planned ? (uint32_t)mv.now[(size_t)isl * 4u + lane] : derive_move<GR>(p, isl, G);
+  };
+  uint32_t move = 0;  // the lane's in the next group to gather for
+  Words4 w[GR];
+  if (warp < nfull) {
+    if constexpr (MIG && !PLAN) move = move_of(first);
+#pragma unroll
+    for (uint32_t i = 0; i < GR; ++i) w[i] = lane_tail(p, head, first + i);
+  }
   // the previous launch (which wrote this launch's parents and read the
   // plane this one writes) has completed and its writes are visible
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -104,20 +120,12 @@ __global__ void __launch_bounds__(kStagedThreads, (kStagedBlocks<GR>))
   // The immigrants of a group are gathered while the group before it is
   // replicated: the gather's latency, with nothing to hide it, made up a
   // third of a generation on L2-resident grids.
-  // Only groups of eight plan ahead: a round of smaller ones is too short.
-  constexpr bool PLAN = GR == kStageGroup;
-  const bool planned = PLAN && mv.now != nullptr;
   Arrival next{kNoArrival, 0u, 0ull};
-  uint32_t move = 0;  // planned, of the group after the next
-  const auto load_of = [&](uint32_t isl) { return (uint32_t)mv.now[(size_t)isl * 4u + lane]; };
   if constexpr (MIG) {
     if (warp < nfull) {
-      if (planned) {
-        next = planned_arrival<TRACKED>(p, load_of(first), first, tin, sin);
-        if (warp + nwarps < nfull) move = load_of(first + skip);
-      } else {
-        next = derive_arrival<TRACKED, GR>(p, first, G, tin, sin);
-      }
+      if constexpr (PLAN) move = move_of(first);
+      next = arrival_of<TRACKED>(p, move, first, tin, sin);
+      if (planned && warp + nwarps < nfull) move = move_of(first + skip);
     }
   }
   [[maybe_unused]] Planner planner(p, mv, warp, nwarps);
@@ -127,17 +135,15 @@ __global__ void __launch_bounds__(kStagedThreads, (kStagedBlocks<GR>))
     const Arrival in = next;
     if constexpr (MIG) {
       if (grp + nwarps < nfull) {
-        if (planned) {
-          next = planned_arrival<TRACKED>(p, move, isl0 + skip, tin, sin);
-          if (grp + 2u * nwarps < nfull) move = load_of(isl0 + 2u * skip);
-        } else {
-          next = derive_arrival<TRACKED, GR>(p, isl0 + skip, G, tin, sin);
-        }
+        if (!planned) move = move_of(isl0 + skip);
+        next = arrival_of<TRACKED>(p, move, isl0 + skip, tin, sin);
+        if (planned && grp + 2u * nwarps < nfull) move = move_of(isl0 + 2u * skip);
       }
     }
-    Words4 w[GR];
+    if (grp != warp) {
 #pragma unroll
-    for (uint32_t i = 0; i < GR; ++i) w[i] = lane_tail(p, head, isl0 + i);
+      for (uint32_t i = 0; i < GR; ++i) w[i] = lane_tail(p, head, isl0 + i);
+    }
     if (!__all_sync(kFull, mbar_wait(&bar[st], phase))) {
       // give up: record the timeout, wait (bounded) for this warp's copies
       // still in flight (the groups issued into the ring from this one on),
@@ -275,8 +281,8 @@ bool staged_stream_plan(const RunParams &p, StreamPlan *out) {
       p.islands / kStageGroup >= 2u * kStagedWarps * kStagedBlocksPerSM * (uint32_t)sms;
   out->back = planes_exceed_l2(p);
   // groups of four where they take one round of the warps: the generation is
-  // then one group's latency (16x16 islands 2.5 us, 3.0 with groups of eight;
-  // 64x63 with a tournament of 5 5.6 and 6.3)
+  // then one group's latency (16x16 islands 2.5 us against 3.0 with groups of
+  // eight, both with their draws after the wait)
   const uint32_t one_round =
       kSmallStageGroup * kStagedWarps * kSmallStagedBlocksPerSM * (uint32_t)sms;
   out->group = (int)(p.islands <= one_round ? kSmallStageGroup : kStageGroup);
