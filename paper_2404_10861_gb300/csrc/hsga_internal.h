@@ -28,10 +28,12 @@ constexpr uint64_t kWaitNs = 1000000000ull; // bounded device wait: 1 s
 // last tile of a row or column may be smaller), tiles_c to a row of tiles.
 struct ResidentTile {
   uint32_t rows, cols, tiles_c;
+  uint32_t stride, slots;  // record slots per tile (0: one per island, in order), per buffer
+  uint32_t by_cols;        // consecutive blocks take the tiles of a column, not of a row
 };
 
 struct ResidentPlan {
-  ResidentTile tile{0, 0, 1};
+  ResidentTile tile{0, 0, 1, 0, 0, 0};
   int blocks = 0;          // one per tile
   int threads = 0;
   uint32_t smem = 0;       // dynamic shared memory per block

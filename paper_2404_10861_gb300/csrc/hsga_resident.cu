@@ -58,7 +58,18 @@ constexpr uint32_t group_warps(uint32_t kg) { return kg == 8u ? 16u : 32u; }
 constexpr uint32_t kSmallTile = 64; // largest tile of the small-tile kernel
 static_assert(kSmallTile >= 64, "larger tiles of 32-agent islands take groups of eight");
 constexpr uint32_t kChunk = 16;       // generations whose draws are tabulated together
-constexpr uint32_t kRemote = 1u << 31;  // neighbour in another tile: global record
+constexpr uint32_t kRemote = 1u << 31;  // neighbour in another tile: record slot
+
+// Slot of island g's record: a tile's islands one after another, tiles apart, so
+// that no 128-byte line is written by two tiles (stride 0: no room for that,
+// slots in island order).
+__device__ __forceinline__ uint32_t record_slot(const RunParams &p, const ResidentTile &t,
+                                                uint32_t g) {
+  if (t.stride == 0u) return g;
+  const uint32_t r = g / p.cols, c = g - r * p.cols;
+  const uint32_t tr = r / t.rows, tc = c / t.cols;
+  return (tr * t.tiles_c + tc) * t.stride + (r - tr * t.rows) * t.cols + c - tc * t.cols;
+}
 constexpr uint32_t kBuf1 = 1u << 31;    // migration word: record buffer 1
 
 __device__ __forceinline__ uint64_t ld_relaxed64(const uint64_t *p) {
@@ -157,6 +168,15 @@ __device__ __forceinline__ uint32_t migration_word(const RunParams &p, uint32_t 
   const uint32_t m = G / p.interval;
   if (m * p.interval != G) return 0u;
   return (m % 0x3FFFFFFFu + 1u) | ((m & 1u) ? kBuf1 : 0u);
+}
+
+// First row and column of this block's tile.
+__device__ __forceinline__ void tile_origin(const ResidentTile &t, uint32_t *r0, uint32_t *c0) {
+  const uint32_t tiles_r = gridDim.x / t.tiles_c;
+  const uint32_t r = t.by_cols ? blockIdx.x % tiles_r : blockIdx.x / t.tiles_c;
+  const uint32_t c = t.by_cols ? blockIdx.x / tiles_r : blockIdx.x - r * t.tiles_c;
+  *r0 = r * t.rows;
+  *c0 = c * t.cols;
 }
 
 template <bool B>
@@ -311,8 +331,8 @@ __global__ void __launch_bounds__(group_warps(KG) * 32, 1)
   const uint32_t tid = threadIdx.x, lane = tid & 31u, nthr = blockDim.x;
   const uint32_t warp = __shfl_sync(kFull, tid >> 5, 0), nwarp = nthr >> 5;
   // this block's tile: rows [r0, r0 + h), columns [c0, c0 + w)
-  const uint32_t tb = blockIdx.x / tile.tiles_c;
-  const uint32_t r0 = tb * tile.rows, c0 = (blockIdx.x - tb * tile.tiles_c) * tile.cols;
+  uint32_t r0, c0;
+  tile_origin(tile, &r0, &c0);
   const uint32_t h = min(tile.rows, p.rows - r0), w = min(tile.cols, p.cols - c0);
   const uint32_t I = h * w, agents = I * n;
   const uint32_t groups = (I + KG - 1u) / KG, IP = groups * KG;  // padded with idle islands
@@ -339,13 +359,13 @@ __global__ void __launch_bounds__(group_warps(KG) * 32, 1)
       if (i < I) {
         const uint32_t nb = neighbour(p, g, d);
         const uint32_t nr = nb / p.cols - r0, nc = nb % p.cols - c0;  // wraps if outside
-        loc = nr < h && nc < w ? nr * w + nc : (nb | kRemote);
+        loc = nr < h && nc < w ? nr * w + nc : (record_slot(p, tile, nb) | kRemote);
       }
       nbloc[4 * i + d] = loc;
       e |= loc & kRemote;
     }
     gisl[i] = i < I ? g : 0u;
-    edge[i] = e;
+    edge[i] = e ? record_slot(p, tile, g) | kRemote : 0u;
   }
   __syncthreads();
   for (uint32_t f = tid; f < IP * n; f += nthr) {
@@ -414,7 +434,8 @@ __global__ void __launch_bounds__(group_warps(KG) * 32, 1)
         const uint4 r = make_uint4(t[0], TRACKED ? t[n] : 0u, TRACKED ? t[2 * n] : 0u,
                                    (mw << 2) | (m.y >> 30));
         srec[(mw & kBuf1 ? IP : 0u) + i] = r;
-        if (edge[i]) st_record<TRACKED>(grec + (mw & kBuf1 ? p.islands : 0u) + gisl[i], r);
+        if (edge[i])
+          st_record<TRACKED>(grec + (mw & kBuf1 ? tile.slots : 0u) + (edge[i] & ~kRemote), r);
       }
       __syncthreads();
     }
@@ -453,7 +474,7 @@ __global__ void __launch_bounds__(group_warps(KG) * 32, 1)
           const bool mine = lane < 4u * KG;
           const uint32_t loc = single ? lane_loc : mine ? nbloc[4u * i0 + lane] : 0u;
           const uint32_t pl = mine ? plan[4u * (o * IP + i0) + lane] : 0u;
-          const uint4 *const in = grec + (mig & kBuf1 ? p.islands : 0u) + (loc & ~kRemote);
+          const uint4 *const in = grec + (mig & kBuf1 ? tile.slots : 0u) + (loc & ~kRemote);
           bool have = (loc & kRemote) == 0u;
           uint4 r = make_uint4(0, 0, 0, 0);
           if (have) r = srec[(mig & kBuf1 ? IP : 0u) + loc];
@@ -519,7 +540,8 @@ __global__ void __launch_bounds__(group_warps(KG) * 32, 1)
             const uint4 r = make_uint4(x[0], TRACKED ? x[n] : 0u, TRACKED ? x[2 * n] : 0u,
                                        (mig_next << 2) | (e >> 6));
             if (edge[i])
-              st_record<TRACKED>(grec + (mig_next & kBuf1 ? p.islands : 0u) + gisl[i], r);
+              st_record<TRACKED>(
+                  grec + (mig_next & kBuf1 ? tile.slots : 0u) + (edge[i] & ~kRemote), r);
             srec[(mig_next & kBuf1 ? IP : 0u) + i] = r;
           }
         }
@@ -613,7 +635,9 @@ __device__ __forceinline__ GenInfo gen_info(const RunParams &p, uint32_t G0, uin
   return gi;
 }
 
-template <bool TRACKED, bool T2, uint32_t KC>
+// ONE: the grid is one tile, and no record leaves the block (4x4 islands 0.487 us
+// per generation, 0.543 with the code for records and waits in place).
+template <bool TRACKED, bool T2, uint32_t KC, bool ONE>
 __global__ void __launch_bounds__(1024, 1)
     step_small_kernel(RunParams p, ResidentTile tile, uint32_t G0, uint32_t ngen, int premigrated,
                       uint32_t *__restrict__ tplane, uint64_t *__restrict__ splane,
@@ -622,8 +646,8 @@ __global__ void __launch_bounds__(1024, 1)
   constexpr uint32_t isz = TRACKED ? 384u : 128u;
   const uint32_t tid = threadIdx.x, lane = tid & 31u;
   const uint32_t warp = __shfl_sync(kFull, tid >> 5, 0);
-  const uint32_t tb = blockIdx.x / tile.tiles_c;
-  const uint32_t r0 = tb * tile.rows, c0 = (blockIdx.x - tb * tile.tiles_c) * tile.cols;
+  uint32_t r0, c0;
+  tile_origin(tile, &r0, &c0);
   const uint32_t h = min(tile.rows, p.rows - r0), w = min(tile.cols, p.cols - c0);
   const uint32_t I = h * w;
   // roles are laid out for a full tile; a cut-off tile has idle warps
@@ -643,7 +667,7 @@ __global__ void __launch_bounds__(1024, 1)
   const auto locate = [&](uint32_t li, uint32_t d) {
     const uint32_t nb = neighbour(p, global_index(li), d);
     const uint32_t nr = nb / p.cols - r0, nc = nb % p.cols - c0;  // wraps if outside
-    return nr < h && nc < w ? nr * w + nc : (nb | kRemote);
+    return nr < h && nc < w ? nr * w + nc : (record_slot(p, tile, nb) | kRemote);
   };
   if (tid == 0) *failed = ~0u;
   for (uint32_t f = tid; f < IF * 32u; f += blockDim.x) {
@@ -678,7 +702,8 @@ __global__ void __launch_bounds__(1024, 1)
 #pragma unroll
       for (uint32_t d = 0; d < 4; ++d) remote |= locate(i, d);
       if (remote & kRemote)
-        st_record<TRACKED>(grec + (mw & kBuf1 ? p.islands : 0u) + global_index(i), r);
+        st_record<TRACKED>(
+            grec + (mw & kBuf1 ? tile.slots : 0u) + record_slot(p, tile, global_index(i)), r);
     }
     block_barrier();
   }
@@ -688,6 +713,7 @@ __global__ void __launch_bounds__(1024, 1)
     const uint32_t i0 = warp * KC;
     uint32_t g[KC];
     bool on_edge[KC];
+    uint32_t slot[KC];  // of the record
 #pragma unroll
     for (uint32_t k = 0; k < KC; ++k) {
       const bool live = i0 + k < I;
@@ -697,7 +723,8 @@ __global__ void __launch_bounds__(1024, 1)
 #pragma unroll
         for (uint32_t d = 0; d < 4; ++d) remote |= locate(i0 + k, d);
       }
-      on_edge[k] = (remote & kRemote) != 0u;
+      on_edge[k] = !ONE && (remote & kRemote) != 0u;
+      slot[k] = on_edge[k] ? record_slot(p, tile, g[k]) : 0u;
     }
     for (uint32_t gen = 0; gen < ngen; ++gen) {
       const uint4 *const info = (const uint4 *)(gens + (gen & (2u * kGenBatch - 1u)));
@@ -731,7 +758,7 @@ __global__ void __launch_bounds__(1024, 1)
               if (((e ^ lane) & 31u) == 0u) {
                 r.w = (mig_next << 2) | (e >> 6);
                 if (on_edge[k])
-                  st_record<TRACKED>(grec + (mig_next & kBuf1 ? p.islands : 0u) + g[k], r);
+                  st_record<TRACKED>(grec + (mig_next & kBuf1 ? tile.slots : 0u) + slot[k], r);
                 srec[i0 + k] = r;
               }
             });
@@ -746,26 +773,26 @@ __global__ void __launch_bounds__(1024, 1)
     const uint32_t i0 = 8u * (warp - nchild), li = i0 + (lane >> 2);
     const bool mine = li < I;
     const uint32_t loc = mine ? locate(li, lane & 3u) : 0u;
-    const bool local = (loc & kRemote) == 0u;
+    const bool local = ONE || (loc & kRemote) == 0u;
     const uint4 *const near = srec + (local ? loc : 0u);
     const uint4 *const far = grec + (loc & ~kRemote);
     for (uint32_t gen = 0; gen < ngen; ++gen) {
       const uint32_t mig = gens[gen & (2u * kGenBatch - 1u)].mig;
       if (mig != 0u) {
         const uint32_t pl = mine ? plan[4u * ((gen % kRows) * IF + i0) + lane] : 0u;
-        const uint4 *const in = far + (mig & kBuf1 ? p.islands : 0u);
+        const uint4 *const in = far + (mig & kBuf1 ? tile.slots : 0u);
         uint4 r = make_uint4(0, 0, 0, 0);
         if (local) r = *near;
         bool have = local;
-        const bool ok = wait_warp(
-            [&] {
-              if (!have) {
-                r = ld_record<TRACKED>(in);
-                have = (r.w >> 2) == (mig & 0x3FFFFFFFu);
-              }
-              return have;
-            },
-            err, kWaitNs);
+        const bool ok = ONE || wait_warp(
+                                   [&] {
+                                     if (!have) {
+                                       r = ld_record<TRACKED>(in);
+                                       have = (r.w >> 2) == (mig & 0x3FFFFFFFu);
+                                     }
+                                     return have;
+                                   },
+                                   err, kWaitNs);
         if (ok) {
           const bool arrive = mine && ((r.w ^ lane) & 3u) == 2u;  // aimed back: d ^ 2
           const uint32_t later = __ballot_sync(kFull, arrive) >> (lane & 28u);
@@ -830,12 +857,12 @@ ResidentFn pick_group(const RunParams &p) {
   return t2 ? step_resident_kernel<false, true, NN, KG> : step_resident_kernel<false, false, NN, KG>;
 }
 
-template <uint32_t KC>
+template <uint32_t KC, bool ONE = false>
 ResidentFn pick_small(const RunParams &p) {
   const bool t2 = p.tournament == 2;
   if (p.policy != HSGA_NONE)
-    return t2 ? step_small_kernel<true, true, KC> : step_small_kernel<true, false, KC>;
-  return t2 ? step_small_kernel<false, true, KC> : step_small_kernel<false, false, KC>;
+    return t2 ? step_small_kernel<true, true, KC, ONE> : step_small_kernel<true, false, KC, ONE>;
+  return t2 ? step_small_kernel<false, true, KC, ONE> : step_small_kernel<false, false, KC, ONE>;
 }
 
 // Warps of a small-tile block of I islands with kc islands per child warp.
@@ -855,8 +882,9 @@ uint32_t small_kc(uint32_t I, uint32_t n) {
 // larger ones would leave most warps without one.
 uint32_t group_for(uint32_t I) { return I <= 32u ? 2u : I <= 64u ? 4u : kMaxGroup; }
 
-ResidentFn pick(const RunParams &p, const ResidentTile &t) {
+ResidentFn pick(const RunParams &p, const ResidentTile &t, bool one) {
   const uint32_t I = t.rows * t.cols, kg = group_for(I);
+  if (one && small_kc(I, p.n) == 1u) return pick_small<1, true>(p);
   switch (small_kc(I, p.n)) {
     case 1: return pick_small<1>(p);
     case 2: return pick_small<2>(p);
@@ -884,10 +912,13 @@ uint32_t threads_for(uint32_t I, uint32_t n) {
 constexpr uint32_t kOneBlockAgents = 768;
 
 // Tiles of one island poll again just before their neighbours' records arrive
-// once they spread over most of the device: 10x12 islands in 120 tiles 1.33 us
-// per generation, in 60 tiles of two 1.12; 12x12 0.94 and 0.73; 8x12 in 96
-// tiles 0.70.
+// once they spread over most of the device: 10x12 islands in 120 tiles 1.31 us
+// per generation, in 60 tiles of two 0.76; 12x12 0.94 and 0.73; 8x12 in 96
+// tiles 0.69.
 constexpr uint32_t kMostSingles = 96;
+
+// Islands of a tile up to which tiles keep their records apart.
+constexpr uint32_t kMostApart = 96;
 
 bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
   int dev = 0, sms = 0, coop = 0, smem = 0;
@@ -904,7 +935,7 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
     return padded > 65536 ? ~0u : tile_layout((uint32_t)padded, p.n, tracked).bytes;
   };
   if (!grid_only && (uint64_t)p.islands * p.n <= kOneBlockAgents) {
-    out->tile = ResidentTile{p.rows, p.cols, 1};
+    out->tile = ResidentTile{p.rows, p.cols, 1, 0, 0, 0};
     out->blocks = 1;
     out->one_block = true;
   } else {
@@ -920,11 +951,14 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
       if (bytes((uint64_t)tr * tc) > (uint32_t)smem) continue;
       if (tr * tc == 1u && p.islands > kMostSingles) continue;
       const double edge = (p.rows > tr ? 2.0 * tc : 0.0) + (p.cols > tc ? 2.0 * tr : 0.0);
-      const double cost = (double)tr * tc * p.n / 32.0 + 0.1 * edge;
+      double cost = (double)tr * tc * p.n / 32.0 + 0.1 * edge;
+      // small tiles (a warp or two per island) that all have the same size:
+      // 64x64 islands 1.35 us in tiles of 4x8, 1.42 in 5x6 with ones cut off
+      if (p.n == 32 && tr * tc <= kSmallTile && (p.rows % tr || p.cols % tc)) cost *= 1.1;
       if (cost < best) {
         best = cost;
         const uint32_t tiles_c = (p.cols + tc - 1) / tc;
-        out->tile = ResidentTile{tr, tc, tiles_c};
+        out->tile = ResidentTile{tr, tc, tiles_c, 0, 0, 0};
         out->blocks = (int)(tiles_r * tiles_c);
       }
     }
@@ -932,6 +966,20 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
     out->one_block = false;
   }
   const uint32_t I = out->tile.rows * out->tile.cols;
+  // record slots: two buffers of at most two slots per island
+  const uint64_t most = 2ull * p.islands, tiles = (uint64_t)out->blocks;
+  const uint32_t apart = (I + 7u) & ~7u;
+  // Slots apart: 64x64 islands 1.41 us against 1.57 in island order, 10x12 0.76
+  // and 1.09, 100x100 1.95 and 2.00; but large tiles 128x128 2.40 and 2.32.
+  out->tile.stride = I > kMostApart          ? 0u
+                     : tiles * apart <= most ? apart
+                     : tiles * I <= most     ? I
+                                             : 0u;
+  // Tiles down the columns: 64x64 islands 1.25 us against 1.35, 24x24 0.89 and
+  // 0.94, 32x128 1.18 and 1.26; tiles of one or two 16x16 0.81 and 0.73, large
+  // ones 100x100 1.98 and 1.95.
+  out->tile.by_cols = p.n == 32 && I > 2u && I <= kSmallTile ? 1u : 0u;
+  out->tile.slots = out->tile.stride ? (uint32_t)tiles * out->tile.stride : p.islands;
   out->threads = (int)threads_for(I, p.n);
   out->smem = bytes(I);
   return true;
@@ -940,7 +988,7 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
 cudaError_t launch_step_resident(const RunParams &p, const ResidentPlan &plan, uint32_t G0,
                                  uint32_t ngen, bool premigrated, uint32_t *t, uint64_t *s,
                                  uint64_t *rec, int *err, cudaStream_t stream) {
-  ResidentFn fn = pick(p, plan.tile);
+  ResidentFn fn = pick(p, plan.tile, plan.one_block);
   // the device's limit, whatever the plan: other threads launch other tiles
   int dev = 0, limit = 0;
   cudaError_t e = cudaGetDevice(&dev);
