@@ -38,6 +38,7 @@ struct ResidentPlan {
   int threads = 0;
   uint32_t smem = 0;       // dynamic shared memory per block
   bool one_block = false;  // a plain launch of one block that holds the whole grid
+  bool warp = false;       // an island per warp in registers (hsga_resident_warp.cu)
 };
 
 // Migration moves of a streamed run, worked out ahead of their generation
@@ -97,6 +98,11 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only = false
 cudaError_t launch_step_resident(const RunParams &p, const ResidentPlan &plan, uint32_t G0,
                                  uint32_t ngen, bool premigrated, uint32_t *t, uint64_t *s,
                                  uint64_t *rec, int *err, cudaStream_t stream);
+
+bool resident_warp_plan(const RunParams &p, ResidentPlan *out);
+cudaError_t launch_step_resident_warp(const RunParams &p, const ResidentPlan &plan, uint32_t G0,
+                                      uint32_t ngen, bool premigrated, uint32_t *t, uint64_t *s,
+                                      uint64_t *rec, int *err, cudaStream_t stream);
 
 cudaError_t launch_migrate(const RunParams &p, uint32_t G, uint32_t *t, uint64_t *s,
                            uint4 *rec, cudaStream_t stream);

@@ -921,6 +921,7 @@ constexpr uint32_t kMostSingles = 96;
 constexpr uint32_t kMostApart = 96;
 
 bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
+  if (resident_warp_plan(p, out)) return true;
   int dev = 0, sms = 0, coop = 0, smem = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -988,6 +989,8 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
 cudaError_t launch_step_resident(const RunParams &p, const ResidentPlan &plan, uint32_t G0,
                                  uint32_t ngen, bool premigrated, uint32_t *t, uint64_t *s,
                                  uint64_t *rec, int *err, cudaStream_t stream) {
+  if (plan.warp)
+    return launch_step_resident_warp(p, plan, G0, ngen, premigrated, t, s, rec, err, stream);
   ResidentFn fn = pick(p, plan.tile, plan.one_block);
   // the device's limit, whatever the plan: other threads launch other tiles
   int dev = 0, limit = 0;

@@ -29,6 +29,9 @@ SHAPES = [
     dict(rows=92, cols=76), dict(rows=47, cols=152),                    # 46, 47
     dict(rows=76, cols=128), dict(rows=95, cols=104),                   # 64, 65
     dict(rows=131, cols=149),                                           # tiles cut off both ways
+    dict(rows=2, cols=4, n=20, tournament=3), dict(rows=15, cols=15, n=22),   # a warp an island
+    dict(rows=7, cols=9, n=47, policy="hybrid", bits=2, interval=2), dict(rows=64, cols=64, n=31),
+    dict(rows=1, cols=7, n=33), dict(rows=33, cols=62, n=64, policy="none"),
     dict(rows=3, cols=400, n=1), dict(rows=40, cols=61, n=31), dict(rows=70, cols=71, n=33),
     dict(rows=97, cols=101, n=17, tournament=3), dict(rows=64, cols=77, n=64, tournament=5),
     dict(rows=90, cols=93, policy="none", p_del=0.1), dict(rows=20, cols=31, policy="none"),
