@@ -50,6 +50,9 @@ struct hsga_grid {
   uint64_t fossil_dropped = 0;
   uint32_t *fossil_words = nullptr;  // fossil_cap x 4
   uint32_t *fossil_where = nullptr;  // fossil_cap x 2
+  // its own: captured runs keep the pointer, and a later hsga_sample_surfaces
+  // of more genomes replaces sample_scratch
+  uint32_t *fossil_scratch = nullptr;
   // free-running migration: per-genome counters, last stamp seen per
   // (island, direction), optional take log
   bool async = false;     // either free-running mode
@@ -210,6 +213,13 @@ int fetch_device_error(hsga_grid *g) {
   return HSGA_OK;
 }
 
+void free_fossils(hsga_grid *g) {
+  dev_free(g->alloc, g->fossil_words, g->stream);
+  dev_free(g->alloc, g->fossil_where, g->stream);
+  dev_free(g->alloc, g->fossil_scratch, g->stream);
+  g->fossil_words = g->fossil_where = g->fossil_scratch = nullptr;
+}
+
 void free_grid(hsga_grid *g) {
   if (!g) return;
   for (int i = 0; i < 2; ++i) {
@@ -220,8 +230,7 @@ void free_grid(hsga_grid *g) {
   dev_free(g->alloc, g->wrec, g->stream);
   dev_free(g->alloc, g->err, g->stream);
   dev_free(g->alloc, g->sample_scratch, g->stream);
-  dev_free(g->alloc, g->fossil_words, g->stream);
-  dev_free(g->alloc, g->fossil_where, g->stream);
+  free_fossils(g);
   dev_free(g->alloc, g->tcount, g->stream);
   dev_free(g->alloc, g->seen, g->stream);
   dev_free(g->alloc, g->mail, g->stream);
@@ -449,11 +458,9 @@ int take_fossils(hsga_grid *g) {
     g->fossil_dropped += g->fossil_k;
     return HSGA_OK;
   }
-  const int r = ensure_sample_scratch(g, g->fossil_k);
-  if (r != HSGA_OK) return r;
   cudaError_t e = launch_sample(g->p, (uint32_t)g->G, g->fossil_k, g->trait[g->cur],
                                 g->surf[g->cur], g->fossil_words + 4 * (size_t)g->fossil_count,
-                                g->fossil_where + 2 * (size_t)g->fossil_count, g->sample_scratch,
+                                g->fossil_where + 2 * (size_t)g->fossil_count, g->fossil_scratch,
                                 g->stream, g->tcount);
   g->launches++;
   g->fossil_count += g->fossil_k;
@@ -556,28 +563,21 @@ int hsga_set_fossil_sampling(hsga_grid *g, uint64_t every, uint32_t k, uint32_t 
   if (!g) return HSGA_ERR_INVALID_ARG;
   if (g->wide && every) return HSGA_ERR_UNSUPPORTED;
   if (every && (k == 0 || k > g->p.islands || capacity < k)) return HSGA_ERR_INVALID_ARG;
-  dev_free(g->alloc, g->fossil_words, g->stream);
-  dev_free(g->alloc, g->fossil_where, g->stream);
-  g->fossil_words = g->fossil_where = nullptr;
+  free_fossils(g);
   g->fossil_every = 0;
   g->fossil_k = g->fossil_cap = g->fossil_count = 0;
   g->fossil_dropped = 0;
   if (!every) return HSGA_OK;
+  // all of it held from now on, so that a run under stream capture allocates
+  // nothing
+  const size_t scratch = sample_scratch_bytes(k);
   g->fossil_words = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * 4 * (size_t)capacity,
                                           g->stream);
   g->fossil_where = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * 2 * (size_t)capacity,
                                           g->stream);
-  if (!g->fossil_words || !g->fossil_where) {
-    dev_free(g->alloc, g->fossil_words, g->stream);
-    dev_free(g->alloc, g->fossil_where, g->stream);
-    g->fossil_words = g->fossil_where = nullptr;
-    return HSGA_ERR_OOM;
-  }
-  // held from now on, so that a run under stream capture allocates nothing
-  if (ensure_sample_scratch(g, k) != HSGA_OK) {
-    dev_free(g->alloc, g->fossil_words, g->stream);
-    dev_free(g->alloc, g->fossil_where, g->stream);
-    g->fossil_words = g->fossil_where = nullptr;
+  if (scratch) g->fossil_scratch = (uint32_t *)dev_alloc(g->alloc, scratch, g->stream);
+  if (!g->fossil_words || !g->fossil_where || (scratch && !g->fossil_scratch)) {
+    free_fossils(g);
     return HSGA_ERR_OOM;
   }
   g->fossil_every = every;
