@@ -40,7 +40,8 @@ struct hsga_grid {
   uint32_t *trait[2] = {nullptr, nullptr};
   uint64_t *surf[2] = {nullptr, nullptr};
   int cur = 0;
-  uint4 *rec = nullptr;      // migrant records, 64 B per island (two stamped 4-word slots)
+  uint4 *rec = nullptr;      // migrant records, 64 B per island, on a 16-byte boundary
+  void *rec_held = nullptr;  // the allocation that holds them
   int *err = nullptr;        // device error word
   uint32_t *sample_scratch = nullptr;
   size_t sample_scratch_bytes = 0;
@@ -91,6 +92,13 @@ void *dev_alloc(const Allocator &a, size_t bytes, cudaStream_t s) {
     return nullptr;
   }
   return p;
+}
+
+// Memory on a 16-byte boundary wherever a hook's starts; *held goes back to
+// dev_free.
+void *dev_alloc16(const Allocator &a, size_t bytes, cudaStream_t s, void **held) {
+  *held = dev_alloc(a, bytes + 15, s);
+  return (void *)(((uintptr_t)*held + 15) & ~(uintptr_t)15);
 }
 
 void dev_free(const Allocator &a, void *ptr, cudaStream_t s) {
@@ -226,7 +234,7 @@ void free_grid(hsga_grid *g) {
     dev_free(g->alloc, g->trait[i], g->stream);
     dev_free(g->alloc, g->surf[i], g->stream);
   }
-  dev_free(g->alloc, g->rec, g->stream);
+  dev_free(g->alloc, g->rec_held, g->stream);
   dev_free(g->alloc, g->wrec, g->stream);
   dev_free(g->alloc, g->err, g->stream);
   dev_free(g->alloc, g->sample_scratch, g->stream);
@@ -331,7 +339,8 @@ int hsga_init_grid(const hsga_config *cfg, void *cuda_stream, hsga_grid **out) {
     g->surf[i] = tracked ? (uint64_t *)dev_alloc(g->alloc, sizeof(uint64_t) * g->swords, g->stream)
                          : nullptr;
   }
-  g->rec = (uint4 *)dev_alloc(g->alloc, sizeof(uint4) * 4 * (size_t)g->p.islands, g->stream);
+  g->rec = (uint4 *)dev_alloc16(g->alloc, sizeof(uint4) * 4 * (size_t)g->p.islands, g->stream,
+                                &g->rec_held);
   g->async = cfg->migration_mode != HSGA_MIGRATION_SYNC;
   g->buffered = cfg->migration_mode == HSGA_MIGRATION_BUFFERED;
   if (g->async) {
