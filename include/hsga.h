@@ -196,8 +196,10 @@ typedef struct hsga_stats {
 typedef struct hsga_grid hsga_grid;
 
 /* Device allocator hooks (optional).  alloc returns device memory of at
- * least `bytes` bytes usable on `stream`, or NULL; free releases it.  Set
- * before hsga_init_grid; grids keep the hooks they were created with.
+ * least `bytes` bytes usable on `stream`, aligned to 8 bytes or more, or NULL;
+ * free releases it.  (Population planes that are not aligned to 16 bytes go
+ * without bulk copies.)  Set before hsga_init_grid; grids keep the hooks they
+ * were created with.
  * Passing NULL for both restores the default (cudaMallocAsync/cudaFreeAsync
  * on the grid's stream). */
 typedef void *(*hsga_alloc_fn)(size_t bytes, void *stream, void *ctx);

@@ -394,7 +394,9 @@ int hsga_init_grid(const hsga_config *cfg, void *cuda_stream, hsga_grid **out) {
       return HSGA_ERR_UNSUPPORTED;
     }
   }
-  if (!g->resident && !g->async && !stream_plan(g->p, &g->splan)) {
+  const bool aligned = (((uintptr_t)g->trait[0] | (uintptr_t)g->trait[1] |
+                         (uintptr_t)g->surf[0] | (uintptr_t)g->surf[1]) & 15u) == 0;
+  if (!g->resident && !g->async && !stream_plan(g->p, aligned, &g->splan)) {
     free_grid(g);
     return HSGA_ERR_CUDA;
   }

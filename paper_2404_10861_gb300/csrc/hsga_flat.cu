@@ -1,6 +1,6 @@
 // hsga_flat.cu -- streamed generation kernel for every island size, fitness
-// model and surface width that the staged kernel (32-agent integer islands
-// with one surface word) does not serve: one launch advances one synchronous
+// model, surface width and alignment that the staged kernel (32-agent integer
+// islands with one surface word) does not serve: one launch advances one synchronous
 // generation of the whole grid, steps a1-a6, a warp taking groups of eight
 // islands (hsga_flat.cuh).  Consecutive launches overlap by programmatic
 // dependent launch, as in the staged kernel.
@@ -168,7 +168,7 @@ auto flat_pick(const RunParams &p, A &&...args) {
   if (p.flt)  // general tournament path only
     return n32 ? F::template run<K, false, 32, true>(p, args...)
                : F::template run<K, false, 0, true>(p, args...);
-  if constexpr (K > 1) {  // 32-agent islands with at most one word: the staged kernel
+  if constexpr (K > 1) {  // aligned 32-agent islands with at most one word: the staged kernel
     if (n32)
       return t2 ? F::template run<K, true, 32, false>(p, args...)
                 : F::template run<K, false, 32, false>(p, args...);

@@ -61,8 +61,10 @@ struct StreamPlan {
   bool moves_ahead = false;  // launches of a run plan the migration of later ones
   bool back = false;         // odd generations walk the islands from last to first
   bool large = false;        // the flat kernel's instance for large grids
+  bool staged = false;       // the staged kernel, else the flat one
 };
-bool stream_plan(const RunParams &p, StreamPlan *out);
+// aligned: the population planes start on 16-byte boundaries.
+bool stream_plan(const RunParams &p, bool aligned, StreamPlan *out);
 
 // Whether parents and children do not fit in L2 together.  Then every other
 // generation walks the islands from last to first: it begins with the parents

@@ -17,8 +17,8 @@ namespace hsga {
 
 // ------------------------------------------------------ streamed step ---
 // 32-agent integer islands with one surface word (the paper's shape) have a
-// kernel of their own, which plans its launches itself.
-static bool staged_shape(const RunParams &p) { return p.n == 32 && p.words == 1 && !p.flt; }
+// kernel of their own, whose bulk copies need planes on 16-byte boundaries; it
+// and the flat kernel plan their launches themselves.
 
 bool exceeds_l2(uint64_t bytes) {
   int dev = 0, l2 = 0;
@@ -32,15 +32,16 @@ bool planes_exceed_l2(const RunParams &p) {
   return exceeds_l2(2u * genome * p.n * p.islands);
 }
 
-bool stream_plan(const RunParams &p, StreamPlan *out) {
-  return staged_shape(p) ? staged_stream_plan(p, out) : flat_stream_plan(p, out);
+bool stream_plan(const RunParams &p, bool aligned, StreamPlan *out) {
+  out->staged = p.n == 32 && p.words == 1 && !p.flt && aligned;
+  return out->staged ? staged_stream_plan(p, out) : flat_stream_plan(p, out);
 }
 
 cudaError_t launch_step_streamed(const RunParams &p, const StreamPlan &plan, uint32_t G,
                                  bool do_mig, const Moves &mv, const uint32_t *tin,
                                  const uint64_t *sin, uint32_t *tout, uint64_t *sout, int *err,
                                  cudaStream_t stream) {
-  if (staged_shape(p))
+  if (plan.staged)
     return launch_step_staged(p, plan, G, do_mig, mv, tin, sin, tout, sout, err, stream);
   return launch_step_flat(p, plan, G, do_mig, mv, tin, sin, tout, sout, err, stream);
 }

@@ -66,3 +66,10 @@ def check(hb, orc, gens=6, migrate=False, **kw):
     dict(rows=4, cols=4), dict(rows=11, cols=12, migrate=True)])
 def test_resident_grids(hb, orc, kw):
     check(hb, orc, kernel=hb.KERNEL_RESIDENT, **kw)
+
+
+@pytest.mark.parametrize("kw", [
+    dict(rows=9, cols=7), dict(rows=9, cols=7, policy="none", tournament=5),
+    dict(rows=181, cols=199, p_del=0.2), dict(rows=9, cols=7, policy="hybrid", bits=2)])
+def test_streamed_grids_of_32_agents(hb, orc, kw):
+    check(hb, orc, kernel=hb.KERNEL_STREAMED, **kw)
