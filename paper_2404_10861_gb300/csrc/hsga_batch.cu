@@ -557,10 +557,12 @@ int hsga_batch_sample(hsga_batch *b, uint32_t run, uint32_t k, uint32_t *out_wor
   uint32_t *scratch = scratch_bytes
                           ? (uint32_t *)device_alloc(b->alloc, scratch_bytes, b->stream)
                           : nullptr;
-  uint32_t *staging = (uint32_t *)device_alloc(b->alloc, sizeof(uint32_t) * 6 * k, b->stream);
+  void *held = nullptr;
+  uint32_t *staging =
+      (uint32_t *)device_alloc16(b->alloc, sizeof(uint32_t) * 6 * k, b->stream, &held);
   if ((scratch_bytes && !scratch) || !staging) {
     device_free(b->alloc, scratch, b->stream);
-    device_free(b->alloc, staging, b->stream);
+    device_free(b->alloc, held, b->stream);
     return HSGA_ERR_OOM;
   }
   cudaError_t e = launch_sample(R.p, (uint32_t)G, k, R.trait[par], R.surf[par], staging,
@@ -573,7 +575,7 @@ int hsga_batch_sample(hsga_batch *b, uint32_t run, uint32_t k, uint32_t *out_wor
     e = cudaMemcpyAsync(out_island_slot, staging + 4 * (size_t)k, sizeof(uint32_t) * 2 * k,
                         cudaMemcpyDefault, b->stream);
   device_free(b->alloc, scratch, b->stream);
-  device_free(b->alloc, staging, b->stream);
+  device_free(b->alloc, held, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   return e == cudaSuccess ? HSGA_OK : HSGA_ERR_CUDA;
 }

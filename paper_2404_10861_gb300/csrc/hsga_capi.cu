@@ -49,7 +49,8 @@ struct hsga_grid {
   uint64_t fossil_every = 0;
   uint32_t fossil_k = 0, fossil_cap = 0, fossil_count = 0;
   uint64_t fossil_dropped = 0;
-  uint32_t *fossil_words = nullptr;  // fossil_cap x 4
+  uint32_t *fossil_words = nullptr;  // fossil_cap x 4, on a 16-byte boundary
+  void *fossil_words_held = nullptr;
   uint32_t *fossil_where = nullptr;  // fossil_cap x 2
   // its own: captured runs keep the pointer, and a later hsga_sample_surfaces
   // of more genomes replaces sample_scratch
@@ -65,8 +66,8 @@ struct hsga_grid {
   // lane state {posts, taken, waiting, 0}
   uint64_t *mail = nullptr;
   uint32_t *ack = nullptr;
-  uint4 *inbuf = nullptr;
-  uint4 *chst = nullptr;
+  uint4 *inbuf = nullptr, *chst = nullptr;
+  void *inbuf_held = nullptr, *chst_held = nullptr;
   uint32_t *alog = nullptr;
   uint32_t alog_gens = 0;
   uint32_t octet_slice = 1;  // free-running: generations per octet visit
@@ -222,10 +223,11 @@ int fetch_device_error(hsga_grid *g) {
 }
 
 void free_fossils(hsga_grid *g) {
-  dev_free(g->alloc, g->fossil_words, g->stream);
+  dev_free(g->alloc, g->fossil_words_held, g->stream);
   dev_free(g->alloc, g->fossil_where, g->stream);
   dev_free(g->alloc, g->fossil_scratch, g->stream);
   g->fossil_words = g->fossil_where = g->fossil_scratch = nullptr;
+  g->fossil_words_held = nullptr;
 }
 
 void free_grid(hsga_grid *g) {
@@ -243,8 +245,8 @@ void free_grid(hsga_grid *g) {
   dev_free(g->alloc, g->seen, g->stream);
   dev_free(g->alloc, g->mail, g->stream);
   dev_free(g->alloc, g->ack, g->stream);
-  dev_free(g->alloc, g->inbuf, g->stream);
-  dev_free(g->alloc, g->chst, g->stream);
+  dev_free(g->alloc, g->inbuf_held, g->stream);
+  dev_free(g->alloc, g->chst_held, g->stream);
   dev_free(g->alloc, g->alog, g->stream);
   cudaStreamSynchronize(g->stream);
   delete g;
@@ -351,8 +353,8 @@ int hsga_init_grid(const hsga_config *cfg, void *cuda_stream, hsga_grid **out) {
     if (g->buffered) {
       g->mail = (uint64_t *)dev_alloc(g->alloc, sizeof(uint64_t) * 4 * C, g->stream);
       g->ack = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * C, g->stream);
-      g->inbuf = (uint4 *)dev_alloc(g->alloc, sizeof(uint4) * 4 * C, g->stream);
-      g->chst = (uint4 *)dev_alloc(g->alloc, sizeof(uint4) * C, g->stream);
+      g->inbuf = (uint4 *)dev_alloc16(g->alloc, sizeof(uint4) * 4 * C, g->stream, &g->inbuf_held);
+      g->chst = (uint4 *)dev_alloc16(g->alloc, sizeof(uint4) * C, g->stream, &g->chst_held);
       ok = ok && g->mail && g->ack && g->inbuf && g->chst;
     }
     if (!ok) {
@@ -582,8 +584,8 @@ int hsga_set_fossil_sampling(hsga_grid *g, uint64_t every, uint32_t k, uint32_t 
   // all of it held from now on, so that a run under stream capture allocates
   // nothing
   const size_t scratch = sample_scratch_bytes(k);
-  g->fossil_words = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * 4 * (size_t)capacity,
-                                          g->stream);
+  g->fossil_words = (uint32_t *)dev_alloc16(g->alloc, sizeof(uint32_t) * 4 * (size_t)capacity,
+                                            g->stream, &g->fossil_words_held);
   g->fossil_where = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * 2 * (size_t)capacity,
                                           g->stream);
   if (scratch) g->fossil_scratch = (uint32_t *)dev_alloc(g->alloc, scratch, g->stream);
@@ -718,8 +720,9 @@ int hsga_sample_surfaces(hsga_grid *g, uint32_t k, uint32_t *out_words,
   if (g->wide) {
     // pick (island, slot) as for one-word surfaces, then gather wide records
     const size_t rw = 2 + 2 * (size_t)g->p.words;
-    uint32_t *staging = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * (6 + rw) * (size_t)k,
-                                              g->stream);
+    void *held = nullptr;
+    uint32_t *staging = (uint32_t *)dev_alloc16(
+        g->alloc, sizeof(uint32_t) * (6 + rw) * (size_t)k, g->stream, &held);
     if (!staging) return HSGA_ERR_OOM;
     uint32_t *pick = staging + 4 * (size_t)k, *wide = staging + 6 * (size_t)k;
     cudaError_t e = launch_sample(g->p, (uint32_t)g->G, k, g->trait[g->cur], nullptr, staging,
@@ -734,7 +737,7 @@ int hsga_sample_surfaces(hsga_grid *g, uint32_t k, uint32_t *out_words,
     if (e == cudaSuccess && out_island_slot)
       e = cudaMemcpyAsync(out_island_slot, pick, sizeof(uint32_t) * 2 * k, cudaMemcpyDefault,
                           g->stream);
-    dev_free(g->alloc, staging, g->stream);
+    dev_free(g->alloc, held, g->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     return cuda_status(e);
   }
@@ -745,8 +748,9 @@ int hsga_sample_surfaces(hsga_grid *g, uint32_t k, uint32_t *out_words,
                       (is_device_ptr(out_island_slot) && ((uintptr_t)out_island_slot % 8) == 0);
   uint32_t *dw = out_words, *di = out_island_slot;
   uint32_t *staging = nullptr;
+  void *held = nullptr;
   if (!dev_words || !dev_is) {
-    staging = (uint32_t *)dev_alloc(g->alloc, sizeof(uint32_t) * 6 * (size_t)k, g->stream);
+    staging = (uint32_t *)dev_alloc16(g->alloc, sizeof(uint32_t) * 6 * (size_t)k, g->stream, &held);
     if (!staging) return HSGA_ERR_OOM;
     if (!dev_words) dw = staging;
     if (!dev_is) di = staging + 4 * (size_t)k;
@@ -761,7 +765,7 @@ int hsga_sample_surfaces(hsga_grid *g, uint32_t k, uint32_t *out_words,
     e = cudaMemcpyAsync(out_island_slot, di, sizeof(uint32_t) * 2 * (size_t)k, cudaMemcpyDefault,
                         g->stream);
   if (staging) {
-    dev_free(g->alloc, staging, g->stream);
+    dev_free(g->alloc, held, g->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   }
   return cuda_status(e);
@@ -1006,6 +1010,9 @@ AllocHooks current_allocator() {
 }
 void *device_alloc(const AllocHooks &h, size_t bytes, cudaStream_t s) {
   return dev_alloc(Allocator{h.alloc, h.free_fn, h.ctx}, bytes, s);
+}
+void *device_alloc16(const AllocHooks &h, size_t bytes, cudaStream_t s, void **held) {
+  return dev_alloc16(Allocator{h.alloc, h.free_fn, h.ctx}, bytes, s, held);
 }
 void device_free(const AllocHooks &h, void *ptr, cudaStream_t s) {
   dev_free(Allocator{h.alloc, h.free_fn, h.ctx}, ptr, s);

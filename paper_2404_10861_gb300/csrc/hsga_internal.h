@@ -152,6 +152,7 @@ struct AllocHooks {
 };
 AllocHooks current_allocator();
 void *device_alloc(const AllocHooks &h, size_t bytes, cudaStream_t s);
+void *device_alloc16(const AllocHooks &h, size_t bytes, cudaStream_t s, void **held);
 void device_free(const AllocHooks &h, void *ptr, cudaStream_t s);
 bool device_pointer(const void *ptr);
 

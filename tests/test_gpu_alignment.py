@@ -73,3 +73,32 @@ def test_resident_grids(hb, orc, kw):
     dict(rows=181, cols=199, p_del=0.2), dict(rows=9, cols=7, policy="hybrid", bits=2)])
 def test_streamed_grids_of_32_agents(hb, orc, kw):
     check(hb, orc, kernel=hb.KERNEL_STREAMED, **kw)
+
+
+@pytest.mark.parametrize("k", [30, 1200])
+def test_samples_and_fossils(hb, orc, k):
+    kw = dict(rows=40, cols=41, n=32, tournament=2, policy="tilted", bits=1, p_ben=0.1, seed=6)
+    c = oracle_config(orc, kw)
+    t, s = orc.run(c, generations=8)[:2]
+    want = orc.sample(c, t, s, 8, k)
+    with eight_byte_memory(hb), hb.Grid(**kw) as g, hb.Batch() as b, \
+            hb.Grid(**dict(kw, words=2)) as w:
+        hb.hsga_set_fossil_sampling(g.handle, 4, k, 2 * k)
+        g.run(8)
+        rid = b.add(8, **kw)
+        b.run(8)
+        w.run(8)
+        words, where = hb.hsga_get_fossils(g.handle, 2 * k)
+        got = [g.sample(k), b.sample(rid, k), (words[k:], where[k:])]
+        assert np.array_equal(w.sample(k)[1], want[1])
+    for x, y in got:
+        assert np.array_equal(x, want[0]) and np.array_equal(y, want[1])
+
+
+def test_buffered_channels(hb):
+    kw = dict(rows=9, cols=7, n=32, tournament=2, policy="tilted", bits=1, seed=7, mode="buffered")
+    with eight_byte_memory(hb), hb.Grid(**kw) as g:
+        g.run(40)
+        g.sync()
+        chan, _ = g.buffers()
+    assert chan[:, :, 0].min() > 0 and chan[:, :, 2].max() <= 4
