@@ -473,7 +473,10 @@ int hsga_batch_get_stats(const hsga_batch *b, hsga_batch_stats *out);
 int hsga_run_footprint(const hsga_config *cfg, uint64_t *bytes);
 
 /* Waits for the batch's stream (all ticks issued so far) and returns the first
- * error a kernel reported. */
+ * error a kernel reported (HSGA_ERR_WAIT_TIMEOUT, HSGA_ERR_DEVICE).
+ * hsga_batch_get_population and hsga_batch_sample return it too, and the
+ * batch's populations are not valid from then on: once a call has returned
+ * it, so does every later hsga_batch_run. */
 int hsga_batch_synchronize(hsga_batch *b);
 
 void hsga_batch_destroy(hsga_batch *b);

@@ -166,6 +166,7 @@ struct hsga_batch {
   bool graph_valid = false;
   int sms = 0;
   uint64_t launches = 0, replications = 0, phases = 0;
+  int broken = HSGA_OK;  // the first error of a tick that the host has read
 };
 
 namespace {
@@ -387,6 +388,19 @@ cudaError_t run_ticks(hsga_batch *b, uint64_t L) {
   return e;
 }
 
+// Waits for the batch's stream, into which the calls before may have put copies
+// to the caller, and reads the ticks' error word: a tick whose bounded wait for
+// a copy ran out has left islands behind, and no population is valid any more.
+int finish(hsga_batch *b) {
+  int err = 0;
+  cudaError_t e = cudaMemcpyAsync(&err, b->d_tick + 1, sizeof(int), cudaMemcpyDeviceToHost,
+                                  b->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  if (e != cudaSuccess) return HSGA_ERR_CUDA;
+  if (err != 0) b->broken = err == kDevErrWaitTimeout ? HSGA_ERR_WAIT_TIMEOUT : HSGA_ERR_DEVICE;
+  return b->broken;
+}
+
 int free_run(hsga_batch *b, HostRun &R) {
   for (int j = 0; j < 2; ++j) {
     device_free(b->alloc, R.trait[j], b->stream);
@@ -487,6 +501,7 @@ int hsga_batch_add(hsga_batch *b, const hsga_config *cfg, uint64_t generations,
 int hsga_batch_run(hsga_batch *b, uint64_t ticks) {
   if (!b) return HSGA_ERR_INVALID_ARG;
   if (stream_capturing(b->stream)) return HSGA_ERR_NOT_CAPTURABLE;
+  if (b->broken != HSGA_OK) return b->broken;
   cudaError_t e = upload_runs(b);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? HSGA_ERR_OOM : HSGA_ERR_CUDA;
   uint64_t left = ticks;
@@ -539,8 +554,7 @@ int hsga_batch_get_population(hsga_batch *b, uint32_t run, uint32_t *trait, uint
   if (e == cudaSuccess && surf)
     e = cudaMemcpyAsync(surf, R.surf[par], sizeof(uint64_t) * R.agents, cudaMemcpyDefault,
                         b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  return e == cudaSuccess ? HSGA_OK : HSGA_ERR_CUDA;
+  return e == cudaSuccess ? finish(b) : HSGA_ERR_CUDA;
 }
 
 int hsga_batch_sample(hsga_batch *b, uint32_t run, uint32_t k, uint32_t *out_words,
@@ -576,8 +590,7 @@ int hsga_batch_sample(hsga_batch *b, uint32_t run, uint32_t k, uint32_t *out_wor
                         cudaMemcpyDefault, b->stream);
   device_free(b->alloc, scratch, b->stream);
   device_free(b->alloc, held, b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  return e == cudaSuccess ? HSGA_OK : HSGA_ERR_CUDA;
+  return e == cudaSuccess ? finish(b) : HSGA_ERR_CUDA;
 }
 
 int hsga_batch_remove(hsga_batch *b, uint32_t run) {
@@ -619,13 +632,7 @@ int hsga_run_footprint(const hsga_config *cfg, uint64_t *bytes) {
 int hsga_batch_synchronize(hsga_batch *b) {
   if (!b) return HSGA_ERR_INVALID_ARG;
   if (stream_capturing(b->stream)) return HSGA_ERR_NOT_CAPTURABLE;
-  // the ticks' bounded waits report a copy that did not arrive
-  int err = 0;
-  cudaError_t e = cudaMemcpyAsync(&err, b->d_tick + 1, sizeof(int), cudaMemcpyDeviceToHost,
-                                  b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  if (e != cudaSuccess) return HSGA_ERR_CUDA;
-  return err == 0 ? HSGA_OK : err == kDevErrWaitTimeout ? HSGA_ERR_WAIT_TIMEOUT : HSGA_ERR_DEVICE;
+  return finish(b);
 }
 
 void hsga_batch_destroy(hsga_batch *b) {
