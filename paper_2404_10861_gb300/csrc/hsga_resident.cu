@@ -914,7 +914,8 @@ constexpr uint32_t kOneBlockAgents = 768;
 // Tiles of one island poll again just before their neighbours' records arrive
 // once they spread over most of the device: 10x12 islands in 120 tiles 1.31 us
 // per generation, in 60 tiles of two 0.76; 12x12 0.94 and 0.73; 8x12 in 96
-// tiles 0.69.
+// tiles 0.69.  A torus of one row is cut into pairs along it: 1x150 0.76, 2.6
+// streamed.
 constexpr uint32_t kMostSingles = 96;
 
 // Islands of a tile up to which tiles keep their records apart.
@@ -948,9 +949,12 @@ bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
       const uint32_t tiles_r = (p.rows + tr - 1) / tr;
       if (tiles_r > (uint32_t)sms) continue;
       const uint32_t most_c = (uint32_t)sms / tiles_r;
-      const uint32_t tc = (p.cols + most_c - 1) / most_c;
+      uint32_t tc = (p.cols + most_c - 1) / most_c;
+      if (tr * tc == 1u && p.islands > kMostSingles) {
+        if (p.rows > 1u) continue;  // tiles of two rows follow
+        tc = 2u;
+      }
       if (bytes((uint64_t)tr * tc) > (uint32_t)smem) continue;
-      if (tr * tc == 1u && p.islands > kMostSingles) continue;
       const double edge = (p.rows > tr ? 2.0 * tc : 0.0) + (p.cols > tc ? 2.0 * tr : 0.0);
       double cost = (double)tr * tc * p.n / 32.0 + 0.1 * edge;
       // small tiles (a warp or two per island) that all have the same size:
