@@ -101,7 +101,7 @@ cudaError_t launch_step_resident(const RunParams &p, const ResidentPlan &plan, u
                                  uint32_t ngen, bool premigrated, uint32_t *t, uint64_t *s,
                                  uint64_t *rec, int *err, cudaStream_t stream);
 
-bool resident_warp_plan(const RunParams &p, ResidentPlan *out);
+bool resident_warp_plan(const RunParams &p, ResidentPlan *out, bool grid_only);
 cudaError_t launch_step_resident_warp(const RunParams &p, const ResidentPlan &plan, uint32_t G0,
                                       uint32_t ngen, bool premigrated, uint32_t *t, uint64_t *s,
                                       uint64_t *rec, int *err, cudaStream_t stream);

@@ -922,7 +922,7 @@ constexpr uint32_t kMostSingles = 96;
 constexpr uint32_t kMostApart = 96;
 
 bool resident_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
-  if (resident_warp_plan(p, out)) return true;
+  if (resident_warp_plan(p, out, grid_only)) return true;
   int dev = 0, sms = 0, coop = 0, smem = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

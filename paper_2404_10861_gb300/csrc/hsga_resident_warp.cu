@@ -2,14 +2,15 @@
 // grids whose islands are not 32 agents: one island per warp with its genomes
 // in registers (lane = agent, AP agents per lane).
 //
-// A block holds a 2^ltr x 2^ltc tile of four islands or more; neighbours inside the tile
-// exchange emigrants through shared memory after one block barrier per
-// migration, and only tile edges publish records in global memory (four
-// 64-bit words, each stamped with the migration's number), which neighbouring
-// tiles poll.  Latency bounds such a grid, and this kernel has less of it than
-// groups of islands per warp on a tile per SM (hsga_resident.cu): us per
-// generation 15x15 islands of 22 1.30 against 1.82, 8x19 of 27 with a tournament
-// of 5 1.43 against 2.15, 64x64 of 17 1.74 against 1.92; 64x64 of 48 2.34 against 2.25.
+// A few islands run in one block, with a block barrier per migration.  More are
+// cut into tiles of four to a block: neighbours inside a tile exchange emigrants
+// through shared memory after one block barrier per migration, and only tile
+// edges publish records in global memory (four 64-bit words, each stamped with
+// the migration's number), which neighbouring tiles poll.  Latency bounds such a
+// grid, and this kernel has less of it than groups of islands per warp on a tile
+// per SM (hsga_resident.cu): us per generation 15x15 islands of 22 1.30 against
+// 1.82, 8x19 of 27 with a tournament of 5 1.43 against 2.15, 64x64 of 17 1.70
+// against 1.92; 64x64 of 48 2.34 against 2.25.
 //
 // Waits are bounded (kWaitNs, kMaxSpins); a warp whose wait gave up reaches the
 // block's next barrier, whose reduction makes the block leave together.
@@ -23,6 +24,12 @@ namespace {
 
 constexpr uint32_t kBatch = 16;  // generations whose per-island RNG blocks are batched
 constexpr uint32_t kMaxSpins = 1u << 22;
+
+// Islands that one block takes alone, of up to 32 agents and of more.  us per
+// generation in one block and in tiles, whose polls differ by 0.1 between
+// devices: 2x4 islands of 17 0.73 and 1.06, 4x4 0.89 and 1.03, 3x7 1.07 and
+// 1.05-1.17, 4x6 1.10 and 1.00-1.08; of 64 3x4 1.11 and 1.23, 2x7 1.25 and 1.19.
+constexpr uint32_t kOneBlockIslands = 22, kOneBlockLarge = 12;
 
 // Whether generation G migrates, and its migration number G / interval, in
 // 32-bit arithmetic with the every-generation case first: a 64-bit modulo
@@ -80,13 +87,15 @@ __device__ bool wait_records_warp(const uint64_t *r, bool polled, uint32_t seq, 
   return false;
 }
 
-template <int AP, bool TRACKED>
-__global__ void __launch_bounds__(1024)
+// ONE: the grid is one tile, and no record leaves the block.
+template <int AP, bool TRACKED, bool ONE>
+__global__ void __launch_bounds__(32 * kOneBlockIslands)
     step_resident_warp_kernel(RunParams p, uint32_t G0, uint32_t ngen, int premigrated,
-                         uint32_t tile, uint32_t *__restrict__ tplane,
-                         uint64_t *__restrict__ splane, uint64_t *__restrict__ rec,
-                         int *__restrict__ err) {
-  __shared__ uint4 srec[2 * 32];
+                              uint32_t tile_r, uint32_t tile_c, uint32_t *__restrict__ tplane,
+                              uint64_t *__restrict__ splane, uint64_t *__restrict__ rec,
+                              int *__restrict__ err) {
+  constexpr uint32_t kSlots = ONE ? kOneBlockIslands : 4;  // islands of a block
+  __shared__ uint4 srec[2 * kSlots];
   const uint32_t lane = threadIdx.x & 31u;
   uint32_t pt[AP];
   uint64_t ps[AP];
@@ -96,20 +105,19 @@ __global__ void __launch_bounds__(1024)
   bool nb_inside = true, publish_global, polls;
   const uint64_t *poll_word;  // lane 4d + j: word j of direction d's record
   {
-    const uint32_t ltr = tile & 0xFFu, ltc = tile >> 8;
-    const uint32_t tiles_c = (p.cols + (1u << ltc) - 1) >> ltc;
-    const uint32_t tr = blockIdx.x / tiles_c, tc = blockIdx.x - tr * tiles_c;
+    const uint32_t tiles_c = (p.cols + tile_c - 1) / tile_c;
+    const uint32_t r0 = blockIdx.x / tiles_c * tile_r, c0 = blockIdx.x % tiles_c * tile_c;
     const uint32_t w = threadIdx.x >> 5;
-    const uint32_t r = (tr << ltr) + (w >> ltc), c = (tc << ltc) + (w & ((1u << ltc) - 1));
+    const uint32_t r = r0 + w / tile_c, c = c0 + w % tile_c;
     const bool active = r < p.rows && c < p.cols;
     isl = active ? r * p.cols + c : p.islands;
     if (active && lane < 4) {
       nb_island = neighbour(p, isl, lane);
-      const uint32_t nr = nb_island / p.cols, nc = nb_island - nr * p.cols;
-      nb_inside = (nr >> ltr) == tr && (nc >> ltc) == tc;
-      nb_slot = ((nr & ((1u << ltr) - 1)) << ltc) | (nc & ((1u << ltc) - 1));
+      const uint32_t nr = nb_island / p.cols - r0, nc = nb_island % p.cols - c0;  // wrap if outside
+      nb_inside = nr < tile_r && nc < tile_c;
+      nb_slot = nb_inside ? nr * tile_c + nc : 0u;
     }
-    publish_global = __any_sync(kFull, !nb_inside);
+    publish_global = !ONE && __any_sync(kFull, !nb_inside);
     // lane 4d + j polls word j of direction d's record (both buffers: +buf offset)
     const uint32_t d = (lane >> 2) & 3u;
     const uint32_t nb_d = __shfl_sync(kFull, nb_island, d);
@@ -165,7 +173,7 @@ __global__ void __launch_bounds__(1024)
                 sv = ps[1];
               }
             }
-            srec[buf * 32 + (threadIdx.x >> 5)] =
+            srec[buf * kSlots + (threadIdx.x >> 5)] =
                 make_uint4(tv, (uint32_t)sv, (uint32_t)(sv >> 32), dir);
             if (publish_global) {
               uint64_t *r = rec + ((size_t)buf * p.islands + isl) * 4;
@@ -180,7 +188,9 @@ __global__ void __launch_bounds__(1024)
         {
           // every warp of the tile arrives here once per migration, also
           // after a failed wait, so the block leaves together
-          if (__syncthreads_or(wfail ? 1 : 0)) {
+          if constexpr (ONE) {
+            __syncthreads();
+          } else if (__syncthreads_or(wfail ? 1 : 0)) {
             failed = true;
             break;
           }
@@ -192,23 +202,25 @@ __global__ void __launch_bounds__(1024)
       if (do_mig) {
         // a2: records from other tiles: one warp-wide wait, then lane d < 4
         // gathers the four words of direction d
-        uint32_t word = 0;
-        const bool ok =
-            wait_records_warp(poll_word + (size_t)buf * p.islands * 4, polls, seq, err, &word);
-        const uint32_t src = (lane & 3u) << 2;
-        const uint32_t w0 = __shfl_sync(kFull, word, src);
-        const uint32_t w1 = __shfl_sync(kFull, word, src + 1);
-        const uint32_t w2 = __shfl_sync(kFull, word, src + 2);
-        const uint32_t w3 = __shfl_sync(kFull, word, src + 3);
-        // after a failed wait the warp stops work and goes on to the next
-        // barrier, where the block leaves together
-        if (!ok) {
-          if (lane == 0) atomicCAS(err, 0, kDevErrWaitTimeout);
-          wfail = true;
+        uint4 r = make_uint4(0, 0, 0, 0);
+        if (publish_global) {  // some neighbour lies in another tile
+          uint32_t word = 0;
+          const bool ok =
+              wait_records_warp(poll_word + (size_t)buf * p.islands * 4, polls, seq, err, &word);
+          const uint32_t src = (lane & 3u) << 2;
+          r.x = __shfl_sync(kFull, word, src);
+          r.y = __shfl_sync(kFull, word, src + 1);
+          r.z = __shfl_sync(kFull, word, src + 2);
+          r.w = __shfl_sync(kFull, word, src + 3);
+          // after a failed wait the warp stops work and goes on to the next
+          // barrier, where the block leaves together
+          if (!ok) {
+            if (lane == 0) atomicCAS(err, 0, kDevErrWaitTimeout);
+            wfail = true;
+          }
+          if (wfail) continue;
         }
-        if (wfail) continue;
-        uint4 r = make_uint4(w0, w1, w2, w3);
-        if (lane < 4 && nb_inside) r = srec[buf * 32 + nb_slot];
+        if (lane < 4 && nb_inside) r = srec[buf * kSlots + nb_slot];
         const bool arrive = lane < 4 && r.w == ((lane + 2u) & 3u);
         const uint32_t arrivals = __ballot_sync(kFull, arrive);
         const uint32_t place[4] = {mig.x, mig.y, mig.z, mig.w};
@@ -244,33 +256,39 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-using WarpFn = void (*)(RunParams, uint32_t, uint32_t, int, uint32_t, uint32_t *, uint64_t *,
-                        uint64_t *, int *);
+using WarpFn = void (*)(RunParams, uint32_t, uint32_t, int, uint32_t, uint32_t, uint32_t *,
+                        uint64_t *, uint64_t *, int *);
 
+template <bool ONE>
 WarpFn pick(const RunParams &p) {
-  const bool tracked = p.policy != HSGA_NONE;
-  if (p.n <= 32)
-    return tracked ? step_resident_warp_kernel<1, true> : step_resident_warp_kernel<1, false>;
-  return tracked ? step_resident_warp_kernel<2, true> : step_resident_warp_kernel<2, false>;
-}
-
-uint32_t log2_of(uint32_t x) {
-  uint32_t l = 0;
-  while ((1u << l) < x) ++l;
-  return l;
+  if (p.policy != HSGA_NONE)
+    return p.n <= 32 ? step_resident_warp_kernel<1, true, ONE>
+                     : step_resident_warp_kernel<2, true, ONE>;
+  return p.n <= 32 ? step_resident_warp_kernel<1, false, ONE>
+                   : step_resident_warp_kernel<2, false, ONE>;
 }
 
 }  // namespace
 
-// Tiles of four islands whose blocks are all resident at once; of 2x2, 1x4 and
-// 4x1 the one with the fewest polled edges.
-bool resident_warp_plan(const RunParams &p, ResidentPlan *out) {
-  if (p.n == 32 || p.islands < 8u || p.islands > (p.n <= 32 ? 4096u : 2048u)) return false;
+// One block for a few islands; else tiles of four islands whose blocks are all
+// resident at once: of 2x2, 1x4 and 4x1 the one with the fewest polled edges.
+bool resident_warp_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
+  if (p.n == 32 || p.islands > (p.n <= 32 ? 4096u : 2048u)) return false;
+  if (!grid_only && p.islands <= (p.n <= 32 ? kOneBlockIslands : kOneBlockLarge)) {
+    out->tile = ResidentTile{p.rows, p.cols, 1, 0, 0, 0};
+    out->blocks = 1;
+    out->threads = (int)p.islands * 32;
+    out->smem = 0;
+    out->one_block = true;
+    out->warp = true;
+    return true;
+  }
+  if (p.islands < 8u) return false;
   int dev = 0, sms = 0, coop = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  if (!coop || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pick(p), 128, 0) !=
+  if (!coop || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pick<false>(p), 128, 0) !=
                    cudaSuccess)
     return false;
   double best = 1e30;
@@ -299,9 +317,13 @@ cudaError_t launch_step_resident_warp(const RunParams &p, const ResidentPlan &pl
                                       uint64_t *rec, int *err, cudaStream_t stream) {
   RunParams pp = p;
   int prem = premigrated ? 1 : 0;
-  uint32_t tile = log2_of(plan.tile.rows) | log2_of(plan.tile.cols) << 8;
-  void *args[] = {&pp, &G0, &ngen, &prem, &tile, &t, &s, &rec, &err};
-  return cudaLaunchCooperativeKernel((const void *)pick(p), dim3(plan.blocks), dim3(plan.threads),
+  uint32_t tile_r = plan.tile.rows, tile_c = plan.tile.cols;
+  if (plan.one_block) {
+    pick<true>(p)<<<1, plan.threads, 0, stream>>>(pp, G0, ngen, prem, tile_r, tile_c, t, s, rec, err);
+    return cudaGetLastError();
+  }
+  void *args[] = {&pp, &G0, &ngen, &prem, &tile_r, &tile_c, &t, &s, &rec, &err};
+  return cudaLaunchCooperativeKernel((const void *)pick<false>(p), dim3(plan.blocks), dim3(plan.threads),
                                      args, 0, stream);
 }
 
