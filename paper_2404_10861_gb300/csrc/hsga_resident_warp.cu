@@ -16,6 +16,8 @@
 // block's next barrier, whose reduction makes the block leave together.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "hsga_internal.h"
 #include "hsga_island.cuh"
 
@@ -29,7 +31,25 @@ constexpr uint32_t kMaxSpins = 1u << 22;
 // generation in one block and in tiles, whose polls differ by 0.1 between
 // devices: 2x4 islands of 17 0.73 and 1.06, 4x4 0.89 and 1.03, 3x7 1.07 and
 // 1.05-1.17, 4x6 1.10 and 1.00-1.08; of 64 3x4 1.11 and 1.23, 2x7 1.25 and 1.19.
+// Where fewer than every other generation migrates, tiles do not poll often
+// enough to lose: 4x4 of 17 0.65 and 0.61 with an interval of 4.
 constexpr uint32_t kOneBlockIslands = 22, kOneBlockLarge = 12;
+
+// Blocks of a tile per SM: 64 registers a thread, to which the launch bound of
+// 1,024 holds the compiler.  68x71 islands of 24 in nine to an SM 2.03 us per
+// generation, in eight 1.84.
+constexpr int kTilesPerSM = 8;
+
+// Most islands of n agents for which tiles of four are the faster kernel.  A
+// lane per agent takes as long for 17 agents as for 31, and for 33 as for 64; a
+// large tile's children are numbered flat.  us here and in large tiles: 64x64
+// islands of 9 1.72, 65x66 1.85 and 1.63, 64x76 1.88 and 1.68; of 17 to 31 64x76
+// 1.89 and 2.00 (tournament 5 2.50 and 2.72); of 48 54x54 1.88 and 2.03, 60x60
+// 2.12 and 2.04; of 64 54x54 1.89 and 2.27, 65x66 2.61 and 2.59, 66x66 2.62 and
+// 2.88.  (Beyond 4,864 islands on 152 SMs the tiles do not fit.)
+constexpr uint32_t most_islands(uint32_t n) {
+  return n <= 16 ? 4096u : n <= 32 || n > 48 ? 0xFFFFFFFFu : 3072u;
+}
 
 // Whether generation G migrates, and its migration number G / interval, in
 // 32-bit arithmetic with the every-generation case first: a 64-bit modulo
@@ -89,7 +109,7 @@ __device__ bool wait_records_warp(const uint64_t *r, bool polled, uint32_t seq, 
 
 // ONE: the grid is one tile, and no record leaves the block.
 template <int AP, bool TRACKED, bool ONE>
-__global__ void __launch_bounds__(32 * kOneBlockIslands)
+__global__ void __launch_bounds__(ONE ? 32 * kOneBlockIslands : 1024)
     step_resident_warp_kernel(RunParams p, uint32_t G0, uint32_t ngen, int premigrated,
                               uint32_t tile_r, uint32_t tile_c, uint32_t *__restrict__ tplane,
                               uint64_t *__restrict__ splane, uint64_t *__restrict__ rec,
@@ -203,7 +223,7 @@ __global__ void __launch_bounds__(32 * kOneBlockIslands)
         // a2: records from other tiles: one warp-wide wait, then lane d < 4
         // gathers the four words of direction d
         uint4 r = make_uint4(0, 0, 0, 0);
-        if (publish_global) {  // some neighbour lies in another tile
+        if constexpr (!ONE) {
           uint32_t word = 0;
           const bool ok =
               wait_records_warp(poll_word + (size_t)buf * p.islands * 4, polls, seq, err, &word);
@@ -273,8 +293,9 @@ WarpFn pick(const RunParams &p) {
 // One block for a few islands; else tiles of four islands whose blocks are all
 // resident at once: of 2x2, 1x4 and 4x1 the one with the fewest polled edges.
 bool resident_warp_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
-  if (p.n == 32 || p.islands > (p.n <= 32 ? 4096u : 2048u)) return false;
-  if (!grid_only && p.islands <= (p.n <= 32 ? kOneBlockIslands : kOneBlockLarge)) {
+  if (p.n == 32 || p.islands > most_islands(p.n)) return false;
+  if (!grid_only && p.islands <= (p.n <= 32 ? kOneBlockIslands : kOneBlockLarge) &&
+      (p.islands < 8u || p.interval == 1u || p.interval == 2u)) {
     out->tile = ResidentTile{p.rows, p.cols, 1, 0, 0, 0};
     out->blocks = 1;
     out->threads = (int)p.islands * 32;
@@ -296,7 +317,7 @@ bool resident_warp_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
     const uint32_t tc = 4 / tr;
     const uint32_t tiles_c = (p.cols + tc - 1) / tc;
     const uint64_t tiles = (uint64_t)((p.rows + tr - 1) / tr) * tiles_c;
-    if (tiles > (uint64_t)per_sm * sms) continue;
+    if (tiles > (uint64_t)std::min(per_sm, kTilesPerSM) * sms) continue;
     const double edges = (p.rows > tr ? 2.0 * tc : 0.0) + (p.cols > tc ? 2.0 * tr : 0.0);
     if (edges < best) {
       best = edges;

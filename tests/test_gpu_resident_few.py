@@ -23,11 +23,11 @@ def hb():
 
 @pytest.mark.parametrize("rows,cols,n,kernel,kw", [
     (1, 1, 1, ONE, {}), (1, 1, 64, ONE, dict(tournament=5)), (1, 2, 33, ONE, {}),
-    (2, 2, 31, ONE, dict(policy="none")), (2, 4, 17, ONE, dict(interval=3)),
+    (2, 2, 31, ONE, dict(policy="none")), (2, 4, 17, ONE, dict(interval=2)), (2, 4, 17, TILES, dict(interval=3)),
     (2, 11, 31, ONE, dict(tournament=3)), (11, 2, 9, ONE, dict(policy="hybrid", bits=2)),
     (1, 22, 20, ONE, dict(policy="none", p_del=0.2)), (1, 23, 20, TILES, {}),
     (3, 4, 64, ONE, {}), (1, 12, 33, ONE, dict(tournament=7, p_del=0.2)),
-    (1, 13, 33, TILES, {}), (3, 4, 40, ONE, dict(interval=0))])
+    (1, 13, 33, TILES, {}), (3, 4, 40, TILES, dict(interval=0)), (1, 7, 40, ONE, dict(interval=0))])
 def test_few_islands(hb, orc, rows, cols, n, kernel, kw):
     kw = dict(dict(rows=rows, cols=cols, n=n, tournament=2, policy="tilted", bits=1, p_ben=0.1,
                    seed=rows + cols), **kw)
