@@ -879,11 +879,16 @@ uint32_t small_kc(uint32_t I, uint32_t n) {
 }
 
 // Islands per group for any other tile of I islands: small groups where
-// larger ones would leave most warps without one.
-uint32_t group_for(uint32_t I) { return I <= 32u ? 2u : I <= 64u ? 4u : kMaxGroup; }
+// larger ones would leave most warps without one.  Islands of n > 24 agents fill
+// a warp's lanes two at a time: 66x66 islands (33 to a tile) of 28 2.12 us per
+// generation in groups of two, 2.29 of four; of 48 2.48 and 2.82; of 17 2.10 and
+// 2.02; 76x80 (40) of 48 2.52 and 2.88; 80x80 (45) of 33 2.82 and 2.63.
+uint32_t group_for(uint32_t I, uint32_t n) {
+  return I <= (n > 24u ? 40u : 32u) ? 2u : I <= 64u ? 4u : kMaxGroup;
+}
 
 ResidentFn pick(const RunParams &p, const ResidentTile &t, bool one) {
-  const uint32_t I = t.rows * t.cols, kg = group_for(I);
+  const uint32_t I = t.rows * t.cols, kg = group_for(I, p.n);
   if (one && small_kc(I, p.n) == 1u) return pick_small<1, true>(p);
   switch (small_kc(I, p.n)) {
     case 1: return pick_small<1>(p);
@@ -899,7 +904,7 @@ ResidentFn pick(const RunParams &p, const ResidentTile &t, bool one) {
 // as few rounds of at most 32 warps as the groups need.
 uint32_t threads_for(uint32_t I, uint32_t n) {
   if (const uint32_t kc = small_kc(I, n)) return 32u * small_warps(I, kc);
-  const uint32_t kg = group_for(I), groups = (I + kg - 1u) / kg;
+  const uint32_t kg = group_for(I, n), groups = (I + kg - 1u) / kg;
   const uint32_t most = group_warps(kg), rounds = (groups + most - 1u) / most;
   return 32u * ((groups + rounds - 1u) / rounds);
 }
