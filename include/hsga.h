@@ -91,11 +91,13 @@ typedef enum hsga_policy {
 
 /* Which kernel advances generations. */
 typedef enum hsga_kernel {
-  HSGA_KERNEL_AUTO = 0,      /* resident when the grid fits on chip, else streamed */
+  HSGA_KERNEL_AUTO = 0,      /* resident when the grid fits on chip, else streamed; calls of
+                                up to four generations are streamed either way */
   HSGA_KERNEL_STREAMED = 1,  /* one launch per generation, population in HBM */
-  HSGA_KERNEL_RESIDENT = 2,  /* persistent launch, genomes in shared memory; grids of a
-                                few islands run in one block (block barriers), larger
-                                ones as a cooperative grid (stamped neighbour records) */
+  HSGA_KERNEL_RESIDENT = 2,  /* persistent launch, genomes in shared memory or registers;
+                                grids of a few islands run in one block (block barriers),
+                                larger ones as a cooperative grid (stamped neighbour
+                                records) */
   HSGA_KERNEL_RESIDENT_GRID = 3  /* resident, always the cooperative multi-block form */
 } hsga_kernel;
 

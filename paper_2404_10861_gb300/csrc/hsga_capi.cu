@@ -398,7 +398,8 @@ int hsga_init_grid(const hsga_config *cfg, void *cuda_stream, hsga_grid **out) {
   }
   const bool aligned = (((uintptr_t)g->trait[0] | (uintptr_t)g->trait[1] |
                          (uintptr_t)g->surf[0] | (uintptr_t)g->surf[1]) & 15u) == 0;
-  if (!g->resident && !g->async && !stream_plan(g->p, aligned, &g->splan)) {
+  const bool streams = !g->resident || cfg->kernel == HSGA_KERNEL_AUTO;  // or short calls
+  if (streams && !g->async && !stream_plan(g->p, aligned, &g->splan)) {
     free_grid(g);
     return HSGA_ERR_CUDA;
   }
@@ -505,6 +506,22 @@ int hsga_run_generations(hsga_grid *g, uint64_t n) {
 }
 
 namespace {
+
+// A resident launch loads the population into the SMs' shared memory, sets its
+// tables up and stores the population again.  Where the caller leaves the kernel
+// open, calls of so few generations that this is most of their time are
+// streamed: us per call of 1, 2, 3 and 4 generations, back to back, streamed 64x64
+// islands 2.6, 4.9, 7.1, 9.5, resident 8.3, 10.3, 12.4, 12.4; 180x190 6.5, 12.8,
+// 19.2, 25.5 and 14.4, 18.5, 22.6, 26.7; tournament 5 10.9, 21.6, 32.4, 43.1 and
+// 18.5, 26.7, 34.9, 41.1; 4x4 2.5, 4.2, 6.0, 7.6 and 6.2, 6.3, 6.3, 8.3; 1x1 2.7,
+// 5.3, 7.8, 10.4 and 6.2, 6.2, 6.2, 6.3.  (Not under capture, where a graph is
+// launched any number of times: resident launches work in place, streamed ones
+// go from plane to plane.)
+bool short_call(const hsga_grid *g, uint64_t n) {
+  const uint64_t most = g->p.islands < 64u ? 2u : g->p.tournament > 2u ? 3u : 4u;
+  return g->cfg.kernel == HSGA_KERNEL_AUTO && n <= most && !stream_capturing(g->stream);
+}
+
 int advance(hsga_grid *g, uint64_t n) {
   cudaError_t e = cudaSuccess;
   if (g->buffered) {
@@ -528,7 +545,7 @@ int advance(hsga_grid *g, uint64_t n) {
       g->launches++;
       done += m;
     }
-  } else if (g->resident) {
+  } else if (g->resident && !short_call(g, n)) {
     // Launch in slices so a single launch stays short.
     const uint64_t slice = 1u << 16;
     uint64_t done = 0;
@@ -549,7 +566,7 @@ int advance(hsga_grid *g, uint64_t n) {
       const uint64_t G = g->G + k;
       const bool do_mig = migrates(g->p, G) && !(g->premigrated && k == 0);
       Moves mv;
-      if (g->splan.moves_ahead) {
+      if (g->splan.moves_ahead && !g->resident) {  // a resident grid's records stay clear
         const size_t even = (k & 1) ? g->p.islands : 0, odd = g->p.islands - even;
         if (do_mig && k >= 2) mv.now = moves + 4 * even;
         if (k >= 1 && k + 1 < n && migrates(g->p, G + 1)) {
