@@ -285,7 +285,15 @@ bool staged_stream_plan(const RunParams &p, StreamPlan *out) {
   // eight, both with their draws after the wait)
   const uint32_t one_round =
       kSmallStageGroup * kStagedWarps * kSmallStagedBlocksPerSM * (uint32_t)sms;
-  out->group = (int)(p.islands <= one_round ? kSmallStageGroup : kStageGroup);
+  // two rounds of them, too, are faster than one full round of eights and a
+  // partial one (with larger tournaments only where that one gives a scheduler
+  // more than one more warp): 24,000 islands 5.50 us against 6.22, 28,000 5.71
+  // and 6.39, tournament 5 9.32 and 8.21, 9.27 and 11.26; 20,500 5.35 and 5.62,
+  // 9.22 and 8.02; three rounds, 31,000, 6.12 and 6.46, but 33,000 6.66 and 6.48
+  const uint32_t eights = kStageGroup * kStagedWarps * kStagedBlocksPerSM * (uint32_t)sms;
+  const uint32_t least = p.tournament == 2u ? eights : eights + eights / 4u;
+  const bool small = p.islands <= one_round || (p.islands > least && p.islands <= 2u * one_round);
+  out->group = (int)(small ? kSmallStageGroup : kStageGroup);
   return true;
 }
 
