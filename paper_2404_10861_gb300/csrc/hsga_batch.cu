@@ -36,7 +36,8 @@ struct BatchRun {  // device descriptor of one run
 };
 
 struct WorkItem {
-  uint32_t run, isl0;
+  uint32_t run : 28, group : 4;  // group: islands, up to kFlatGroup
+  uint32_t isl0;
 };
 
 // 16 warps (<= 128 registers, the runs' round keys among them): 104 ms for a
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(kFlatThreads, kBatchBlocksPerSM)
   // children written are the first parents read
   const bool back = may_back != 0u && par != 0u;
   const auto item = [&](uint32_t k) { return items[back ? n_items - 1u - k : k]; };
-  WorkItem w = i < n_items ? item(i) : WorkItem{0u, 0u};
+  WorkItem w = i < n_items ? item(i) : WorkItem{0u, 0u, 0u};
   while (i < n_items) {
     const uint32_t run = w.run;
     const BatchRun &R = runs[run];
@@ -96,13 +97,13 @@ __global__ void __launch_bounds__(kFlatThreads, kBatchBlocksPerSM)
     flat_heads(keys, p.n, G, st);
     __syncwarp();
     do {
-      const uint32_t isl0 = w.isl0;
+      const uint32_t isl0 = w.isl0, group = w.group;
       i += nwarps;
       if (i < n_items) w = item(i);
       const bool ok = t2 ? flat_group<1, true, 0, false>(p, keys, dep, do_mig, bulk, isl0,
-                                                         kFlatGroup, G, false, 0u, false, tin, sin, tout, sout, st)
+                                                         group, G, false, 0u, false, tin, sin, tout, sout, st)
                          : flat_group<1, false, 0, false>(p, keys, dep, do_mig, bulk, isl0,
-                                                          kFlatGroup, G, false, 0u, false, tin, sin, tout, sout, st);
+                                                          group, G, false, 0u, false, tin, sin, tout, sout, st);
       if (!ok) {
         // give up: record the timeout, wait (bounded) for the copy, leave
         if (lane == 0) {
@@ -156,6 +157,7 @@ struct hsga_batch {
   // (finishing tick, items up to and including that run)
   std::vector<std::pair<uint64_t, uint32_t>> prefix;
   uint32_t stage_bytes = 0;  // shared memory per warp for the largest island in the list
+  uint32_t least = kFlatGroup;  // islands per item (group_of)
   uint32_t back = 0;         // odd ticks walk the list backwards
   int most_per_sm = 1;       // blocks that an SM keeps resident with it
   int per_sm = 0;            // blocks per SM that ticks are launched with
@@ -214,6 +216,29 @@ cudaError_t upload_runs(hsga_batch *b) {
   return e;
 }
 
+// Islands per item of a run: a multiple of what starts on 16-byte boundaries.
+uint32_t group_of(const HostRun &R, uint32_t least) {
+  const uint32_t step = (R.p.n & 3u) == 0u ? 1u : (R.p.n & 1u) == 0u ? 2u : 4u;
+  return (least + step - 1u) / step * step;
+}
+
+// The fewest islands per item, two at least, that leave every item of the active
+// runs a warp of its own, so that a tick is one item's latency; eight if none do.
+// One run of 64x64 islands of 32 3.95 us per tick, in items of four 4.60, of eight
+// 5.39, with a tournament of 5 4.63, 5.79 and 7.79; 100x100 in items of five 4.98
+// and 6.58, of eight 5.91 and 8.51.
+uint32_t fewest_islands(const hsga_batch *b) {
+  const uint64_t warps = (uint64_t)b->sms * (uint64_t)b->most_per_sm * kFlatWarps;
+  for (uint32_t least = 2; least < kFlatGroup; ++least) {
+    uint64_t items = 0;
+    for (const HostRun &R : b->runs)
+      if (active_at(R, b->tick))
+        items += (R.p.islands + group_of(R, least) - 1u) / group_of(R, least);
+    if (items <= warps) return least;
+  }
+  return kFlatGroup;
+}
+
 // Work list of the runs active at the current tick, ordered by finishing tick,
 // latest first.
 cudaError_t rebuild_items(hsga_batch *b) {
@@ -228,12 +253,8 @@ cudaError_t rebuild_items(hsga_batch *b) {
   uint32_t n_max = 1;
   uint64_t agents = 0;
   for (uint32_t r : order) {
-    const HostRun &R = b->runs[r];
-    agents += R.agents;
-    n_max = std::max(n_max, R.p.n);
-    for (uint32_t i0 = 0; i0 < R.p.islands; i0 += kFlatGroup)
-      b->h_items.push_back(WorkItem{r, i0});
-    b->prefix.push_back({R.start_tick + R.budget, (uint32_t)b->h_items.size()});
+    agents += b->runs[r].agents;
+    n_max = std::max(n_max, b->runs[r].p.n);
   }
   b->stage_bytes = flat_stage_bytes(n_max, 1);
   b->back = exceeds_l2(24u * agents) ? 1u : 0u;  // both planes of 12-byte genomes
@@ -245,6 +266,14 @@ cudaError_t rebuild_items(hsga_batch *b) {
                                                       kFlatWarps * b->stage_bytes);
   if (e != cudaSuccess) return e;
   b->most_per_sm = std::max(per_sm, 1);
+  b->least = fewest_islands(b);
+  for (uint32_t r : order) {
+    const HostRun &R = b->runs[r];
+    const uint32_t group = group_of(R, b->least);
+    for (uint32_t i0 = 0; i0 < R.p.islands; i0 += group)
+      b->h_items.push_back(WorkItem{r, group, i0});
+    b->prefix.push_back({R.start_tick + R.budget, (uint32_t)b->h_items.size()});
+  }
   const size_t n = b->h_items.size();
   if (n > b->items_cap) {
     device_free(b->alloc, b->d_items, b->stream);
@@ -514,7 +543,8 @@ int hsga_batch_run(hsga_batch *b, uint64_t ticks) {
         phase_end = std::min(phase_end, R.start_tick + R.budget);
       }
     if (!any) break;
-    if (b->items_dirty) {
+    // (the runs that others have left behind may do with smaller items)
+    if (b->items_dirty || fewest_islands(b) < b->least) {
       e = rebuild_items(b);
       if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? HSGA_ERR_OOM : HSGA_ERR_CUDA;
     }
