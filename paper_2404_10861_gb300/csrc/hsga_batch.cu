@@ -611,7 +611,7 @@ int hsga_batch_sample(hsga_batch *b, uint32_t run, uint32_t k, uint32_t *out_wor
   }
   cudaError_t e = launch_sample(R.p, (uint32_t)G, k, R.trait[par], R.surf[par], staging,
                                 staging + 4 * (size_t)k, scratch, b->stream);
-  b->launches++;
+  b->launches += sample_launches(k);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(out_words, staging, sizeof(uint32_t) * 4 * k, cudaMemcpyDefault,
                         b->stream);

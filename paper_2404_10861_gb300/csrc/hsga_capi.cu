@@ -476,7 +476,7 @@ int take_fossils(hsga_grid *g) {
                                 g->surf[g->cur], g->fossil_words + 4 * (size_t)g->fossil_count,
                                 g->fossil_where + 2 * (size_t)g->fossil_count, g->fossil_scratch,
                                 g->stream, g->tcount);
-  g->launches++;
+  g->launches += sample_launches(g->fossil_k);
   g->fossil_count += g->fossil_k;
   return cuda_status(e);
 }
@@ -747,7 +747,7 @@ int hsga_sample_surfaces(hsga_grid *g, uint32_t k, uint32_t *out_words,
     if (e == cudaSuccess)
       e = launch_gather_wide(g->p, (uint32_t)g->G, k, g->trait[g->cur], g->surf[g->cur], pick,
                              wide, g->stream);
-    g->launches += 2;
+    g->launches += sample_launches(k) + 1u;
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(out_words, wide, sizeof(uint32_t) * rw * k, cudaMemcpyDefault,
                           g->stream);
@@ -774,7 +774,7 @@ int hsga_sample_surfaces(hsga_grid *g, uint32_t k, uint32_t *out_words,
   }
   cudaError_t e = launch_sample(g->p, (uint32_t)g->G, k, g->trait[g->cur], g->surf[g->cur], dw,
                                 di, g->sample_scratch, g->stream, g->tcount);
-  g->launches++;
+  g->launches += sample_launches(k);
   if (e == cudaSuccess && !dev_words)
     e = cudaMemcpyAsync(out_words, dw, sizeof(uint32_t) * 4 * (size_t)k, cudaMemcpyDefault,
                         g->stream);

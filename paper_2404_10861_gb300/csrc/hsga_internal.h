@@ -111,6 +111,7 @@ cudaError_t launch_migrate(const RunParams &p, uint32_t G, uint32_t *t, uint64_t
 
 // Scratch that launch_sample needs for k genomes (8-byte aligned; may be 0).
 size_t sample_scratch_bytes(uint32_t k);
+uint32_t sample_launches(uint32_t k);  // kernels that it launches
 
 // T: per-genome deposition counters (free-running grids) written as word 3,
 // or NULL to write G.

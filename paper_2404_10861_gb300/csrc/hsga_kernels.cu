@@ -192,6 +192,8 @@ size_t sample_scratch_bytes(uint32_t k) {
   return k <= kSampleOneBlock ? 0 : (size_t)k * sizeof(uint2) + (size_t)sample_buckets(k) * 4;
 }
 
+uint32_t sample_launches(uint32_t k) { return k <= kSampleOneBlock ? 1u : 2u; }
+
 cudaError_t launch_sample(const RunParams &p, uint32_t G, uint32_t k, const uint32_t *t,
                           const uint64_t *s, uint32_t *out_words, uint32_t *out_is,
                           uint32_t *scratch, cudaStream_t stream, const uint32_t *T) {
