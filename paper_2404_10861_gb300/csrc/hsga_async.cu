@@ -53,7 +53,7 @@ __device__ __forceinline__ void counter_step(const RunParams &p, const PhiloxHea
   const uint32_t n = NN ? (uint32_t)NN : p.n;
   uint32_t pt[1] = {t}, pT[1] = {T};
   uint64_t ps[1] = {s};
-  const Words4 w = philox_tail<true>(p, h, isl);
+  const Words4 w = philox_tail(p, h, isl);
   uint32_t best = uindex_nn<NN>(w.x, n);
   uint32_t fbest = fetch32<1>(pt, best);
   if (T2 || p.tournament >= 2) {
@@ -303,7 +303,7 @@ constexpr int kBufferedBlocksPerSM = 8;
 // generation at 16.8M agents when the one-generation case runs the general
 // loop).
 template <bool TRACKED, bool T2, bool TWO, int IPW, bool FLT, int NN = 0, bool SLICED = false>
-__global__ void __launch_bounds__(kResidentThreads, kAsyncBlocksPerSM)
+__global__ void __launch_bounds__(kFreeThreads, kAsyncBlocksPerSM)
     step_async_kernel(RunParams p, uint32_t G0, uint32_t ngen, uint32_t slice,
                       uint32_t *__restrict__ tplane,
                       uint64_t *__restrict__ splane, uint32_t *__restrict__ Tplane,
@@ -543,7 +543,7 @@ __device__ __forceinline__ void buffered_generation(const RunParams &p, Octet<IP
 }
 
 template <bool TRACKED, bool T2, bool TWO, int IPW, bool FLT, int NN = 0, bool SLICED = false>
-__global__ void __launch_bounds__(kResidentThreads, kBufferedBlocksPerSM)
+__global__ void __launch_bounds__(kFreeThreads, kBufferedBlocksPerSM)
     step_buffered_kernel(RunParams p, uint32_t G0, uint32_t ngen, uint32_t slice,
                          uint32_t *__restrict__ tplane,
                          uint64_t *__restrict__ splane, uint32_t *__restrict__ Tplane,
@@ -684,13 +684,13 @@ BufferedFn pick_buffered(bool tracked, bool t2, bool two, bool flt, bool n32, bo
 // blocks than the device keeps resident at once, so that every island
 // advances in the same pass over the grid (warps then own several octets).
 uint32_t resident_blocks(const void *fn, uint32_t islands, uint32_t ipw, int max_per_sm) {
-  const uint32_t wpb = kResidentThreads / 32;
+  const uint32_t wpb = kFreeThreads / 32;
   const uint32_t octets = (islands + ipw - 1) / ipw;
   const uint32_t need = (octets + wpb - 1) / wpb;
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kResidentThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kFreeThreads, 0);
   if (per_sm > max_per_sm) per_sm = max_per_sm;
   const uint32_t cap = (uint32_t)(sms > 0 ? sms : 1) * (uint32_t)(per_sm > 0 ? per_sm : 1);
   return need < cap ? need : cap;
@@ -706,7 +706,7 @@ cudaError_t launch_step_buffered(const RunParams &p, uint32_t G0, uint32_t ngen,
                                 p.policy == HSGA_HYBRID, p.flt, p.n == 32, slice > 1);
   const uint32_t blocks = resident_blocks((const void *)fn, p.islands, kBufferedIslandsPerWarp,
                                           kBufferedBlocksPerSM);
-  fn<<<blocks, kResidentThreads, 0, stream>>>(p, G0, ngen, slice > 0 ? slice : 1, t, s, T,
+  fn<<<blocks, kFreeThreads, 0, stream>>>(p, G0, ngen, slice > 0 ? slice : 1, t, s, T,
                                                mail, ack, inbuf, chst, log, log_G0, log_gens);
   return cudaGetLastError();
 }
@@ -719,7 +719,7 @@ cudaError_t launch_step_async(const RunParams &p, uint32_t G0, uint32_t ngen, ui
                           p.flt, p.n == 32, slice > 1);
   const uint32_t blocks = resident_blocks((const void *)fn, p.islands, kAsyncIslandsPerWarp,
                                           kAsyncBlocksPerSM);
-  fn<<<blocks, kResidentThreads, 0, stream>>>(p, G0, ngen, slice > 0 ? slice : 1, t, s, T, rec,
+  fn<<<blocks, kFreeThreads, 0, stream>>>(p, G0, ngen, slice > 0 ? slice : 1, t, s, T, rec,
                                                seen, log, log_G0, log_gens);
   return cudaGetLastError();
 }

@@ -309,19 +309,16 @@ __device__ __forceinline__ PhiloxHead philox_head(uint32_t k0, uint32_t k1, uint
                     (uint32_t)p0};
 }
 
-// Rounds 2-10 after a precomputed head; RK as below.
-template <bool RK>
+// Rounds 2-10 after a precomputed head.
 __device__ __forceinline__ Words4 philox_tail(const RunParams &p, const PhiloxHead &h,
                                               uint32_t c1_in) {
   uint32_t c0 = h.x0 ^ c1_in, c1 = h.c1, c2 = h.c2, c3 = h.c3;
 #pragma unroll
   for (int r = 1; r < 10; ++r) {
-    const uint32_t k0 = RK ? p.rk0[r] : p.k0 + (uint32_t)r * kPhiloxW0;
-    const uint32_t k1 = RK ? p.rk1[r] : p.k1 + (uint32_t)r * kPhiloxW1;
     const uint64_t p0 = (uint64_t)c0 * kPhiloxM0;
     const uint64_t p1 = (uint64_t)c2 * kPhiloxM1;
-    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k0;
-    const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k1;
+    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ p.rk0[r];
+    const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ p.rk1[r];
     c0 = n0;
     c1 = (uint32_t)p1;
     c2 = n2;
@@ -372,15 +369,6 @@ __device__ __forceinline__ Words4 lane_tail(const RunParams &p, const LaneHead &
     c3 = (uint32_t)p0;
   }
   return Words4{c0, c1, c2, c3};
-}
-
-// RK: the run's round keys are precomputed in the parameter block (single-run
-// kernels); otherwise they are derived from the key in registers.
-template <bool RK>
-__device__ __forceinline__ Words4 philox_p(const RunParams &p, uint32_t c0, uint32_t c1,
-                                           uint32_t c2, uint32_t c3) {
-  if constexpr (RK) return philox_rk(p, c0, c1, c2, c3);
-  else return philox(p.k0, p.k1, c0, c1, c2, c3);
 }
 
 // Neighbour of island `isl` in direction d (0 N, 1 E, 2 S, 3 W).

@@ -21,7 +21,7 @@ constexpr int kStagedThreads = 256;     // staged streamed kernel (n = 32) block
 constexpr int kStagedBlocksPerSM = 2;
 constexpr int kSmallStagedBlocksPerSM = 3;  // groups of four islands: 24 warps
 constexpr uint32_t kStagedStages = 2;   // most groups in flight per warp
-constexpr int kResidentThreads = 128;   // free-running, float and wide kernels: 4 warps
+constexpr int kFreeThreads = 128;       // free-running kernels: 4 warps
 constexpr uint64_t kWaitNs = 1000000000ull; // bounded device wait: 1 s
 
 // The resident kernel cuts the torus into tiles of rows x cols islands (the

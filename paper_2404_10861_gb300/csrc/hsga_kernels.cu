@@ -1,13 +1,14 @@
-// hsga_kernels.cu -- streamed generation kernel, explicit migration,
-// end-state sampling and the site-function kernel.
+// hsga_kernels.cu -- dispatch of the streamed generation kernels, explicit
+// migration, end-state sampling, and the kernels that show the generator and the
+// site functions by themselves.
 //
-// Streamed kernel: one launch advances one synchronous generation of the
-// whole grid; the population ping-pongs between two structure-of-arrays
-// planes in HBM (uint32 traits, uint64 surfaces: 12 bytes per agent,
-// coalesced 128 B / 256 B per island).  The kernel boundary is the
-// generation barrier.  Migration needs no exchange buffer: the receiver
-// recomputes each neighbour's emigrant choice from the counter-based RNG and
-// gathers that genome straight from the neighbour's parent plane.
+// Streamed: one launch advances one synchronous generation of the whole
+// grid (hsga_staged.cu, hsga_flat.cu); the population ping-pongs between two
+// structure-of-arrays planes in HBM (uint32 traits, uint64 surfaces: 12 bytes per
+// agent).  The kernel boundary is the generation barrier.  Migration needs no
+// exchange buffer: the receiver works each neighbour's emigrant out from the
+// counter-based generator and gathers that genome straight from the neighbour's
+// parent plane.
 #include <cuda_runtime.h>
 
 #include "hsga_internal.h"

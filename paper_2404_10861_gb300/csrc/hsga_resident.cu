@@ -25,7 +25,7 @@
 // tournament 2), against the kernel before them, which held an island per
 // warp in registers and spent 294 warp instructions per island-generation:
 //   4x4 islands    0.51 us (0.90)   87 warp instructions, 116 with migration
-//   64x64          1.27-1.56 (1.75) 120; a read of a remote record alone is
+//   64x64          1.27 us (1.75)   120; a read of a remote record alone is
 //                                   0.35 us, without migration 0.61 us
 //   128x128        2.31 (6.4 on the streamed kernel: it did not fit before)
 //                                   80; without migration 1.77 us, 64

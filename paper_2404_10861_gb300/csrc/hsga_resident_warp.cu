@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(ONE ? 32 * kOneBlockIslands : 1024)
       uint32_t ct[AP];
       uint64_t cs[AP];
       if (dep.two)
-        replicate<AP, TRACKED, false, true, true>(p, dep, isl, G, w, pt, ps, ct, cs);
+        replicate<AP, TRACKED, false, true>(p, dep, isl, G, w, pt, ps, ct, cs);
       else
         replicate<AP, TRACKED>(p, dep, isl, G, w, pt, ps, ct, cs);
 #pragma unroll

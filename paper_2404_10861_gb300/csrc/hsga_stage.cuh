@@ -1,13 +1,12 @@
 // hsga_stage.cuh -- staging of island groups in shared memory by bulk
-// asynchronous copies, shared by the single-run staged generation kernel
+// asynchronous copies: the barrier and copy primitives, also the flat kernel's
+// (hsga_flat.cuh), and the parts of the staged generation kernel
 // (hsga_staged.cu).
 //
-// A warp owns a ring of up to kStagedStages stages; a stage holds one group of
-// eight 32-agent islands: 1,024 bytes of traits, then 2,048 bytes of surfaces,
-// each contiguous in the island-major planes, copied by one lane with
-// cp.async.bulk and completing on the stage's mbarrier.  The helpers below are
-// the barrier and copy primitives, a group's immigrants, and its replication
-// from a stage.
+// A warp of it owns a ring of up to kStagedStages stages; a stage holds one group of
+// eight (or four) 32-agent islands: 1,024 bytes of traits, then 2,048 bytes of
+// surfaces, each contiguous in the island-major planes, copied by one lane with
+// cp.async.bulk and completing on the stage's mbarrier.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -191,6 +190,33 @@ __device__ __forceinline__ void replicate_group(const RunParams &p, const Deposi
     __stcs(to + 32u * i, mutate<DEL>(p, fbest[i], w[i].z));
     if constexpr (TRACKED) __stcs(so + 32u * i, deposit_into<TWO>(dep, cs[i], w[i].w));
   }
+}
+
+// a2-a6 of one 32-agent island in registers (lane = agent).
+template <bool TRACKED, bool T2, bool MIG>
+__device__ __noinline__ void single_island(const RunParams &p, const Deposit &dep, uint32_t G,
+                                           uint32_t isl, const uint32_t *__restrict__ tin,
+                                           const uint64_t *__restrict__ sin,
+                                           uint32_t *__restrict__ tout,
+                                           uint64_t *__restrict__ sout) {
+  const size_t a = (size_t)isl * 32u + (threadIdx.x & 31u);
+  uint32_t pt[1] = {__ldcs(tin + a)}, ct[1];
+  uint64_t ps[1] = {0}, cs[1];
+  if constexpr (TRACKED) ps[0] = __ldcs(sin + a);
+  Words4 w[1];
+  replication_words<1>(p, isl, G, w);
+  if constexpr (MIG) {
+    const Arrival in = arrival_of<TRACKED>(p, derive_move<1>(p, isl, G), isl, tin, sin);
+    const uint32_t landing = __ballot_sync(kFull, in.at != kNoArrival);
+#pragma unroll
+    for (uint32_t d = 0; d < 4; ++d)
+      if (landing >> d & 1u)
+        land<1, TRACKED>(__shfl_sync(kFull, in.at, d), d, in.it, in.is, pt, ps);
+  }
+  if (dep.two) replicate<1, TRACKED, T2, true>(p, dep, isl, G, w, pt, ps, ct, cs);
+  else replicate<1, TRACKED, T2, false>(p, dep, isl, G, w, pt, ps, ct, cs);
+  __stcs(tout + a, ct[0]);
+  if constexpr (TRACKED) __stcs(sout + a, cs[0]);
 }
 
 template <uint32_t GR>

@@ -190,8 +190,7 @@ __global__ void __launch_bounds__(kStagedThreads, (kStagedBlocks<GR>))
   // the last islands, too few for a group, on the register path, one to a warp
   // (333x337 islands 16.2 us; all of them on one warp 18.5)
   const uint32_t rest = nfull * GR + (nwarps - 1u - warp);
-  if (rest < p.islands)
-    partial_group<1, TRACKED, T2>(p, dep, G, MIG, rest, 1u, tin, sin, tout, sout);
+  if (rest < p.islands) single_island<TRACKED, T2, MIG>(p, dep, G, rest, tin, sin, tout, sout);
 }
 
 template <bool TRACKED, bool T2, bool TWO, bool DEL, bool MIG, uint32_t GR>
