@@ -69,6 +69,7 @@ KERNEL_SOURCES = ["paper_2404_10861_gb300/csrc/hsga_device.cuh",
                   "paper_2404_10861_gb300/csrc/hsga_kernels.cu",
                   "paper_2404_10861_gb300/csrc/hsga_moves.cuh",
                   "paper_2404_10861_gb300/csrc/hsga_stage.cuh",
+                  "paper_2404_10861_gb300/csrc/hsga_sync.cuh",
                   "paper_2404_10861_gb300/csrc/hsga_staged.cu"]
 PROFILE = os.path.join(ROOT, "profiles", "step_streamed_wafer.md")
 FREE_RUNNING_SOURCES = ["paper_2404_10861_gb300/csrc/hsga_device.cuh",

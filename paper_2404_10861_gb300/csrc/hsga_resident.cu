@@ -43,6 +43,7 @@
 
 #include "hsga_internal.h"
 #include "hsga_island.cuh"
+#include "hsga_sync.cuh"
 
 namespace hsga {
 
@@ -71,12 +72,6 @@ __device__ __forceinline__ uint32_t record_slot(const RunParams &p, const Reside
   return (tr * t.tiles_c + tc) * t.stride + (r - tr * t.rows) * t.cols + c - tc * t.cols;
 }
 constexpr uint32_t kBuf1 = 1u << 31;    // migration word: record buffer 1
-
-__device__ __forceinline__ uint64_t ld_relaxed64(const uint64_t *p) {
-  uint64_t v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
 
 // A record as one single-copy atomic access: 16 bytes, or 8 (trait, stamp)
 // when there is no surface.  (An untracked record is not simply a 16-byte one
@@ -109,31 +104,23 @@ __device__ __forceinline__ void st_record(uint4 *p, const uint4 &r) {
         "l"(a), "l"(b)
         : "memory");
   } else {
-    const uint64_t v = ((uint64_t)r.w << 32) | r.x;
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+    st_relaxed64((uint64_t *)p, ((uint64_t)r.w << 32) | r.x);
   }
-}
-
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
 }
 
 // Bounded wait of a whole warp until ready() holds on every lane: gives up
 // (on every lane, returning false) after limit_ns of the global timer or
 // kMaxSpins polls, whichever comes first, or as soon as an error has been
 // reported in *err.
-constexpr uint32_t kMaxSpins = 1u << 22;
 
 template <class F>
 __device__ __forceinline__ bool wait_warp(const F &ready, const int *err, uint64_t limit_ns) {
   if (__all_sync(kFull, ready())) return true;
-  const uint64_t t0 = global_ns();
+  const uint64_t t0 = now_ns();
   for (uint32_t spin = 1; spin < kMaxSpins; ++spin) {
     if (__all_sync(kFull, ready())) return true;
     if ((spin & 255u) == 0) {
-      const bool stop = *(volatile const int *)err != 0 || global_ns() - t0 > limit_ns;
+      const bool stop = *(volatile const int *)err != 0 || now_ns() - t0 > limit_ns;
       if (__any_sync(kFull, stop)) return false;
     }
   }
@@ -147,7 +134,7 @@ __device__ __forceinline__ bool wait_warp(const F &ready, const int *err, uint64
 __global__ void wait_probe_kernel(const uint64_t *record, uint32_t seq, uint64_t limit_ns,
                                   int *err, uint64_t *out) {
   const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t t0 = global_ns();
+  const uint64_t t0 = now_ns();
   const auto carries = [&](uint32_t j) { return (uint32_t)(ld_relaxed64(record + j) >> 32) == seq; };
   const bool ok = wait_warp(
       [&] { return lane > 0 || (carries(0) && carries(1) && carries(2) && carries(3)); }, err,
@@ -155,7 +142,7 @@ __global__ void wait_probe_kernel(const uint64_t *record, uint32_t seq, uint64_t
   const bool ok_words = wait_warp([&] { return lane > 3 || carries(lane); }, err, limit_ns);
   if (lane == 0) {
     out[0] = (ok && ok_words) ? 1u : 0u;
-    out[1] = global_ns() - t0;
+    out[1] = now_ns() - t0;
   }
 }
 

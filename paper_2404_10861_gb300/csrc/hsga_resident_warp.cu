@@ -20,12 +20,12 @@
 
 #include "hsga_internal.h"
 #include "hsga_island.cuh"
+#include "hsga_sync.cuh"
 
 namespace hsga {
 namespace {
 
 constexpr uint32_t kBatch = 16;  // generations whose per-island RNG blocks are batched
-constexpr uint32_t kMaxSpins = 1u << 22;
 
 // Islands that one block takes alone, of up to 32 agents and of more.  us per
 // generation in one block and in tiles, whose polls differ by 0.1 between
@@ -66,22 +66,6 @@ __device__ __forceinline__ bool migration_of(const RunParams &p, uint32_t G, uin
   return q * p.interval == G;
 }
 
-__device__ __forceinline__ uint64_t ld_relaxed64(const uint64_t *p) {
-  uint64_t v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void st_relaxed64(uint64_t *p, uint64_t v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
 // The whole warp waits for the records of its island's neighbours
 // in other tiles at once.  Lane 4d + j (< 16) polls word j of the record of
 // direction d (if `polled`: that neighbour lies in another tile), so every
@@ -90,7 +74,7 @@ __device__ __forceinline__ uint64_t global_ns() {
 // Returns false (on every lane) when it gave up.
 __device__ bool wait_records_warp(const uint64_t *r, bool polled, uint32_t seq, const int *err,
                                   uint32_t *word) {
-  const uint64_t t0 = global_ns();
+  const uint64_t t0 = now_ns();
   for (uint32_t spin = 1; spin < kMaxSpins; ++spin) {
     bool ready = true;
     if (polled) {
@@ -100,7 +84,7 @@ __device__ bool wait_records_warp(const uint64_t *r, bool polled, uint32_t seq, 
     }
     if (__all_sync(kFull, ready)) return true;
     if ((spin & 255u) == 0) {
-      const bool stop = *(volatile const int *)err != 0 || global_ns() - t0 > kWaitNs;
+      const bool stop = *(volatile const int *)err != 0 || now_ns() - t0 > kWaitNs;
       if (__any_sync(kFull, stop)) return false;
     }
   }

@@ -14,6 +14,7 @@
 #include "hsga_internal.h"
 #include "hsga_island.cuh"
 #include "hsga_moves.cuh"
+#include "hsga_sync.cuh"
 
 namespace hsga {
 
@@ -28,12 +29,6 @@ constexpr uint32_t kMaxPolls = 1u << 24;
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint64_t now_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
