@@ -288,7 +288,6 @@ bool resident_warp_plan(const RunParams &p, ResidentPlan *out, bool grid_only) {
     out->warp = true;
     return true;
   }
-  if (p.islands < 8u) return false;
   int dev = 0, sms = 0, coop = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
