@@ -518,7 +518,16 @@ namespace {
 // launched any number of times: resident launches work in place, streamed ones
 // go from plane to plane.)
 bool short_call(const hsga_grid *g, uint64_t n) {
-  const uint64_t most = g->p.islands < 64u ? 2u : g->p.tournament > 2u ? 3u : 4u;
+  // a streamed generation takes the longer the more draws a lane evaluates (43x43
+  // islands of 64 with a tournament of 7 6.9 us), a resident one the less where not
+  // every generation migrates
+  const RunParams &p = g->p;
+  const uint32_t t = p.tournament;
+  const uint32_t blocks = (t > 2u ? 1u + (t + 1u) / 4u : 1u) * (p.n > 32u ? 2u : 1u);
+  const uint64_t most = blocks > 2u                                         ? 1u
+                        : p.islands < 64u || p.n > 32u || p.interval != 1u ? 2u
+                        : blocks == 2u                                      ? 3u
+                                                                            : 4u;
   return g->cfg.kernel == HSGA_KERNEL_AUTO && n <= most && !stream_capturing(g->stream);
 }
 

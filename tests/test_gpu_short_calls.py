@@ -24,7 +24,8 @@ def hb():
 @pytest.mark.parametrize("kw", [
     dict(rows=1, cols=1), dict(rows=4, cols=4, tournament=5), dict(rows=4, cols=4, n=17),
     dict(rows=9, cols=8, policy="none"), dict(rows=64, cols=64, policy="hybrid", bits=2),
-    dict(rows=65, cols=66, n=48), dict(rows=100, cols=100, interval=2, coarsen=2),
+    dict(rows=65, cols=66, n=48), dict(rows=30, cols=31, n=40, tournament=7),
+    dict(rows=9, cols=9, tournament=9), dict(rows=100, cols=100, interval=2, coarsen=2),
     dict(rows=150, cols=160, p_del=0.2), dict(rows=170, cols=150, tournament=5),
     dict(rows=300, cols=290, n=1)])
 def test_cut_runs(hb, orc, kw):
@@ -48,7 +49,9 @@ def test_cut_runs(hb, orc, kw):
         got = g.population()
     want = orc.run(c, trait, surf, G0=30, generations=sum(calls))[:2]
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
-    most = 2 if c.rows * c.cols < 64 else 3 if c.tournament > 2 else 4
+    blocks = (1 if c.tournament <= 2 else 1 + -(-(c.tournament - 2) // 4)) * (2 if c.n > 32 else 1)
+    few = c.rows * c.cols < 64 or c.n > 32 or c.interval != 1
+    most = 1 if blocks > 2 else 2 if few else 3 if blocks == 2 else 4
     assert launches == [n if n <= most else 1 for n in calls]
 
 
