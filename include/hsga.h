@@ -158,8 +158,8 @@ typedef enum hsga_fitness {
  * surf[a K + w]); sample records are 2 + 2K words (trait, the surface words
  * as (low, high) 32-bit pairs, T), i.e. four words when K = 1.  K > 1 needs
  * synchronous migration, a surface policy, agents_per_island <= 32 and the
- * AUTO or STREAMED kernel (a warp-per-island path); fossil sampling,
- * batches and the allocation-free entry point need K = 1. */
+ * AUTO or STREAMED kernel; fossil sampling, batches and the allocation-free
+ * entry point need K = 1. */
 /* Run configuration (plain data, caller-owned; copied by hsga_init_grid). */
 typedef struct hsga_config {
   uint32_t rows, cols;          /* toroidal island grid, each >= 1 */

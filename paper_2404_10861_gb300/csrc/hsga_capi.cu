@@ -147,7 +147,7 @@ int validate(const hsga_config *c) {
   if (c->p_beneficial + c->p_deleterious > 1.0) return HSGA_ERR_INVALID_ARG;
   if (c->kernel > HSGA_KERNEL_RESIDENT_GRID || c->reserved != 0) return HSGA_ERR_INVALID_ARG;
   if (c->fitness > HSGA_FITNESS_FLOAT) return HSGA_ERR_INVALID_ARG;
-  if (K > 1) {  // wide surfaces: the synchronous warp-per-island path
+  if (K > 1) {  // wide surfaces: streamed synchronous generations
     if (c->surface_policy == HSGA_NONE || c->agents_per_island > 32) return HSGA_ERR_INVALID_ARG;
     if (c->migration_mode != HSGA_MIGRATION_SYNC) return HSGA_ERR_UNSUPPORTED;
     if (c->kernel != HSGA_KERNEL_AUTO && c->kernel != HSGA_KERNEL_STREAMED)

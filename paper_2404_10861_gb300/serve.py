@@ -15,10 +15,13 @@ the whole GPU busy on its own; at most ``max_large`` of those run at a time,
 first come first served among them, while smaller requests are admitted in
 arrival order as soon as they fit, never queueing behind a large one.  A
 large run advances on a grid of its own (the single-run kernels, which
-stream a large grid faster than the batch's tick kernel) on a second stream
+advance a large grid faster than the batch's tick kernel) on a second stream
 beside the batch, in slices of the same length as the batch's, so it runs
 at nearly its speed alone; the small runs, which alone would leave the GPU
-idle between their short generations, overlap with it in the batch.
+idle between their short generations, overlap with it in the batch.  (Large
+runs that fit on chip, up to 35,264 islands of 32 agents, take the SMs for
+their slice and alternate with the batch; that is faster than streaming them
+beside it: four runs of 2^20 agents and 60 small ones 0.235 s against 0.254.)
 ``serve_alone`` is the reference policy: the same stream served one request
 at a time, each on its own grid.
 
